@@ -90,18 +90,12 @@ __global__ void __launch_bounds__(kLightWarps * 32) count_light_batch_kernel(
     int slots_log, unsigned long long* out, unsigned* status) {
   extern __shared__ __align__(16) unsigned char light_smem[];
   const int slots = 1 << slots_log;
-  unsigned long long* vals_all = reinterpret_cast<unsigned long long*>(light_smem);
-  uint32_t* keys_all = reinterpret_cast<uint32_t*>(vals_all + kLightWarps * slots);
   const int w = threadIdx.x >> 5;
   const unsigned lane = lane_id();
-  uint32_t* keys = keys_all + w * slots;
-  unsigned long long* vals = vals_all + w * slots;
-  for (int i = lane; i < slots; i += 32) {
-    keys[i] = kEmptyKey;
-    vals[i] = 0;
-  }
+  uint32_t* keys = reinterpret_cast<uint32_t*>(light_smem) + 2 * w * slots;
+  uint32_t* vals = keys + slots;
+  hash_clear(keys, vals, slots_log, lane, 32);
   __syncwarp();
-  const int max_log = slots_log;
   uint64_t bal = 0, unb = 0;
   bool full = false;
   int cur_graph = -1;
@@ -125,15 +119,11 @@ __global__ void __launch_bounds__(kLightWarps * 32) count_light_batch_kernel(
         work = d.work;
         mult_log = d.hash_mult_log;
       }
-      const int log_h = table_log(work[bp.row], max_log, mult_log);
+      const uint64_t wp = work[bp.row];
+      const int log_h = table_log(wp, slots_log, mult_log);
       const PivotGeom q = pivot_geom(g, bp.row);
-      full |= !hash_walk_dispatch(hash_group_log(work[bp.row], q.L, 5), lane, 32u, g, q, keys, vals, log_h, bal,
-                                  unb);
-      __syncwarp();
-      for (int i = lane; i < (1 << log_h); i += 32) {
-        keys[i] = kEmptyKey;
-        vals[i] = 0;
-      }
+      full |= !hash_count(hash_group_log(wp, q.L, 5), lane, 32u, g, q, keys, vals, log_h, bal, unb);
+      hash_clear(keys, vals, log_h, lane, 32);
       __syncwarp();
     }
   }
@@ -150,29 +140,23 @@ __global__ void __launch_bounds__(kMediumThreads) count_medium_batch_kernel(cons
                                                                             unsigned* status) {
   extern __shared__ __align__(16) unsigned char med_smem[];
   const int slots = 1 << slots_log;
-  unsigned long long* vals = reinterpret_cast<unsigned long long*>(med_smem);
-  uint32_t* keys = reinterpret_cast<uint32_t*>(vals + slots);
-  for (int i = threadIdx.x; i < slots; i += kMediumThreads) {
-    keys[i] = kEmptyKey;
-    vals[i] = 0;
-  }
+  uint32_t* keys = reinterpret_cast<uint32_t*>(med_smem);
+  uint32_t* vals = keys + slots;
+  hash_clear(keys, vals, slots_log, threadIdx.x, kMediumThreads);
   __syncthreads();
-  const int max_log = slots_log;
   bool full = false;
   for (int64_t t = blockIdx.x; t < n_piv; t += gridDim.x) {
     const BatchPivot bp = piv[t];
     const GraphDesc d = desc[bp.graph];
     const CsrView g = view_of(d);
-    const int log_h = table_log(d.work[bp.row], max_log, d.hash_mult_log);
+    const uint64_t wp = d.work[bp.row];
+    const int log_h = table_log(wp, slots_log, d.hash_mult_log);
     const PivotGeom q = pivot_geom(g, bp.row);
     uint64_t bal = 0, unb = 0;
-    full |= !hash_walk_dispatch(hash_group_log(d.work[bp.row], q.L, 5), threadIdx.x, (uint32_t)kMediumThreads, g, q,
-                                keys, vals, log_h, bal, unb);
+    full |= !hash_count(hash_group_log(wp, q.L, 5), threadIdx.x, (uint32_t)kMediumThreads, g, q, keys, vals, log_h,
+                        bal, unb);
     __syncthreads();
-    for (int i = threadIdx.x; i < (1 << log_h); i += kMediumThreads) {
-      keys[i] = kEmptyKey;
-      vals[i] = 0;
-    }
+    hash_clear(keys, vals, log_h, threadIdx.x, kMediumThreads);
     block_add_pair<kMediumThreads>(bal, unb, out + 2 * bp.graph);  // contains __syncthreads
   }
   if (full) atomicOr(status, DBBC_DEV_HASH_FULL);
@@ -332,9 +316,9 @@ static void plan_table_logs(dbbc_batch* b, const dbbc_graph* const* gs, int32_t 
   }
 }
 static size_t light_smem_bytes(const dbbc_batch* b) {
-  return (size_t)kLightWarps * ((size_t)1 << b->light_log) * 12;
+  return (size_t)kLightWarps * ((size_t)1 << b->light_log) * kHashSlotBytes;
 }
-static size_t medium_smem_bytes(const dbbc_batch* b) { return ((size_t)1 << b->medium_log) * 12; }
+static size_t medium_smem_bytes(const dbbc_batch* b) { return ((size_t)1 << b->medium_log) * kHashSlotBytes; }
 
 // Plan for the components of one union handle: every component shares the
 // union's CSR; pivots and hub items are tagged with their component.
@@ -513,9 +497,9 @@ static void enqueue_batch(dbbc_batch* b, cudaStream_t s) {
 
 static void set_batch_attributes() {
   DBBC_CUDA(cudaFuncSetAttribute(count_light_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)((size_t)kLightWarps * kLightSlots * 12)));
+                                 (int)((size_t)kLightWarps * kLightSlots * kHashSlotBytes)));
   DBBC_CUDA(cudaFuncSetAttribute(count_medium_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)((size_t)kMediumSlots * 12)));
+                                 (int)((size_t)kMediumSlots * kHashSlotBytes)));
   DBBC_CUDA(cudaFuncSetAttribute(DBBC_WIDE_SWEEP, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepSmem));
   DBBC_CUDA(cudaFuncSetAttribute(DBBC_NARROW_SWEEP, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNarrowSmem));
 }

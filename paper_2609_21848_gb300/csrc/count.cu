@@ -2,8 +2,8 @@
 // finalisation of Lemma 1, in three tiers chosen by a pivot's accepted wedges:
 //
 //   light  : one warp per pivot, open-addressing hash in the warp's slice of
-//            shared memory (packed u64 counter per endpoint: low 32 bits
-//            symmetric wedges B1, high 32 bits asymmetric wedges B2);
+//            shared memory (packed 32-bit counter per endpoint: low half
+//            symmetric wedges B1, high half asymmetric wedges B2);
 //   medium : one CTA per pivot, a larger shared hash shared by its warps;
 //   hub    : window sweep: a work item is a hub and a range of its endpoint
 //            ranks, owned by one CTA, whose counters for one window of ranks
@@ -24,32 +24,31 @@ __global__ void __launch_bounds__(kLightWarps * 32) count_light_kernel(CsrView g
                                                                        unsigned long long* out, unsigned* status) {
   extern __shared__ __align__(16) unsigned char light_smem[];
   const int slots = 1 << slots_log;
-  unsigned long long* vals_all = reinterpret_cast<unsigned long long*>(light_smem);
-  uint32_t* keys_all = reinterpret_cast<uint32_t*>(vals_all + kLightWarps * slots);
+  uint32_t* tables = reinterpret_cast<uint32_t*>(light_smem);
   const int w = threadIdx.x >> 5;
   const unsigned lane = lane_id();
-  uint32_t* keys = keys_all + w * slots;
-  unsigned long long* vals = vals_all + w * slots;
-  for (int i = lane; i < slots; i += 32) {
-    keys[i] = kEmptyKey;
-    vals[i] = 0;
-  }
+  uint32_t* keys = tables + 2 * w * slots;
+  uint32_t* vals = keys + slots;
+  hash_clear(keys, vals, slots_log, lane, 32);
   __syncwarp();
-  const int max_log = slots_log;
   uint64_t bal = 0, unb = 0;
   bool full = false;
   const int64_t nw = (int64_t)gridDim.x * kLightWarps;
-  for (int64_t t = (int64_t)blockIdx.x * kLightWarps + w; t < n_piv; t += nw) {
-    const int32_t p = piv[t];
-    const int log_h = table_log(work[p], max_log, hash_mult_log);
-    const PivotGeom q = pivot_geom(g, p);
-    full |= !hash_walk_dispatch(hash_group_log(work[p], q.L, 5), lane, 32u, g, q, keys, vals, log_h, bal, unb);
+  int64_t t = (int64_t)blockIdx.x * kLightWarps + w;
+  int32_t p = t < n_piv ? piv[t] : 0, p1 = t + nw < n_piv ? piv[t + nw] : 0;
+  PivotGeom q = pivot_geom(g, p);
+  uint64_t wp = work[p];
+  for (; t < n_piv; t += nw) {
+    // the next pivot's geometry and the row after it, while this one is walked
+    const PivotGeom q1 = pivot_geom(g, p1);
+    const uint64_t wp1 = work[p1];
+    p1 = t + 2 * nw < n_piv ? piv[t + 2 * nw] : 0;
+    const int log_h = table_log(wp, slots_log, hash_mult_log);
+    full |= !hash_count(hash_group_log(wp, q.L, 5), lane, 32u, g, q, keys, vals, log_h, bal, unb);
+    hash_clear(keys, vals, log_h, lane, 32);
     __syncwarp();
-    for (int i = lane; i < (1 << log_h); i += 32) {
-      keys[i] = kEmptyKey;
-      vals[i] = 0;
-    }
-    __syncwarp();
+    q = q1;
+    wp = wp1;
   }
   if (full) atomicOr(status, DBBC_DEV_HASH_FULL);
   block_add_pair<kLightWarps * 32>(bal, unb, out);
@@ -63,28 +62,28 @@ __global__ void __launch_bounds__(kMediumThreads) count_medium_kernel(CsrView g,
                                                                       unsigned long long* out, unsigned* status) {
   extern __shared__ __align__(16) unsigned char med_smem[];
   const int slots = 1 << slots_log;
-  unsigned long long* vals = reinterpret_cast<unsigned long long*>(med_smem);
-  uint32_t* keys = reinterpret_cast<uint32_t*>(vals + slots);
-  for (int i = threadIdx.x; i < slots; i += kMediumThreads) {
-    keys[i] = kEmptyKey;
-    vals[i] = 0;
-  }
+  uint32_t* keys = reinterpret_cast<uint32_t*>(med_smem);
+  uint32_t* vals = keys + slots;
+  hash_clear(keys, vals, slots_log, threadIdx.x, kMediumThreads);
   __syncthreads();
-  const int max_log = slots_log;
   uint64_t bal = 0, unb = 0;
   bool full = false;
-  for (int64_t t = blockIdx.x; t < n_piv; t += gridDim.x) {
-    const int32_t p = piv[t];
-    const int log_h = table_log(work[p], max_log, hash_mult_log);
-    const PivotGeom q = pivot_geom(g, p);
-    full |= !hash_walk_dispatch(hash_group_log(work[p], q.L, 5), threadIdx.x, (uint32_t)kMediumThreads, g, q, keys,
-                                vals, log_h, bal, unb);
+  int64_t t = blockIdx.x;
+  int32_t p = t < n_piv ? piv[t] : 0, p1 = t + gridDim.x < n_piv ? piv[t + gridDim.x] : 0;
+  PivotGeom q = pivot_geom(g, p);
+  uint64_t wp = work[p];
+  for (; t < n_piv; t += gridDim.x) {
+    const PivotGeom q1 = pivot_geom(g, p1);  // the next pivot's, while this one is walked
+    const uint64_t wp1 = work[p1];
+    p1 = t + 2 * (int64_t)gridDim.x < n_piv ? piv[t + 2 * (int64_t)gridDim.x] : 0;
+    const int log_h = table_log(wp, slots_log, hash_mult_log);
+    full |= !hash_count(hash_group_log(wp, q.L, 5), threadIdx.x, (uint32_t)kMediumThreads, g, q, keys, vals, log_h,
+                        bal, unb);
     __syncthreads();
-    for (int i = threadIdx.x; i < (1 << log_h); i += kMediumThreads) {
-      keys[i] = kEmptyKey;
-      vals[i] = 0;
-    }
+    hash_clear(keys, vals, log_h, threadIdx.x, kMediumThreads);
     __syncthreads();
+    q = q1;
+    wp = wp1;
   }
   if (full) atomicOr(status, DBBC_DEV_HASH_FULL);
   block_add_pair<kMediumThreads>(bal, unb, out);
@@ -188,9 +187,9 @@ CountProfiler::~CountProfiler() {
 static void launch_light(const dbbc_graph* g, const CsrView& view, cudaStream_t s, unsigned long long* d_out,
                          unsigned* d_status) {
   const int slots_log = tier_slots_log(g->tune.light_max_work, g->tune.hash_mult_log, 10);
-  const size_t smem = (size_t)kLightWarps * ((size_t)1 << slots_log) * 12;
+  const size_t smem = (size_t)kLightWarps * ((size_t)1 << slots_log) * kHashSlotBytes;
   DBBC_CUDA(cudaFuncSetAttribute(count_light_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)((size_t)kLightWarps * kLightSlots * 12)));
+                                 (int)((size_t)kLightWarps * kLightSlots * kHashSlotBytes)));
   const int64_t want = ceil_div<int64_t>(g->n_light, kLightWarps);
   const int64_t cap = (int64_t)num_sms() * blocks_per_sm((const void*)count_light_kernel, kLightWarps * 32, smem);
   count_light_kernel<<<(unsigned)std::min(want, cap), kLightWarps * 32, smem, s>>>(
@@ -202,9 +201,9 @@ static void launch_light(const dbbc_graph* g, const CsrView& view, cudaStream_t 
 static void launch_medium(const dbbc_graph* g, const CsrView& view, cudaStream_t s, unsigned long long* d_out,
                           unsigned* d_status) {
   const int slots_log = tier_slots_log(g->tune.medium_max_work, g->tune.hash_mult_log, 13);
-  const size_t smem = ((size_t)1 << slots_log) * 12;
+  const size_t smem = ((size_t)1 << slots_log) * kHashSlotBytes;
   DBBC_CUDA(cudaFuncSetAttribute(count_medium_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)((size_t)kMediumSlots * 12)));
+                                 (int)((size_t)kMediumSlots * kHashSlotBytes)));
   const int64_t cap = (int64_t)num_sms() * blocks_per_sm((const void*)count_medium_kernel, kMediumThreads, smem);
   count_medium_kernel<<<(unsigned)std::min<int64_t>(g->n_medium, cap), kMediumThreads, smem, s>>>(
       view, g->order + g->n_hub, g->work, g->n_medium, g->tune.hash_mult_log, slots_log, d_out, d_status);

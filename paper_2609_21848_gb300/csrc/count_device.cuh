@@ -4,15 +4,12 @@
 // lower neighbours, and one window of the hub sweep.
 #pragma once
 
+#include <type_traits>
+
 #include "internal.h"
 #include "common.cuh"
 
 namespace dbbc {
-
-// One packed increment: symmetric wedge -> +1, asymmetric -> +2^32.
-__device__ __forceinline__ unsigned long long wedge_inc(uint32_t x, uint32_t s1) {
-  return ((x ^ s1) & 1u) ? (1ull << 32) : 1ull;
-}
 
 // Lemma 1 contribution of one wedge, from its endpoint counter just before the
 // increment (sym = p, asym = q): adding a symmetric wedge to (p, q) closes p
@@ -27,6 +24,12 @@ __device__ __forceinline__ void wedge_contrib(unsigned long long old, unsigned l
   unb += sym ? q : p;
 }
 
+// Hash counters of the light and medium tiers: one 32-bit word per endpoint,
+// (asym << 16) | sym. A count never exceeds the pivot's accepted wedges, and
+// those are at most kMediumMaxWork in these tiers. One 32-bit shared atomic
+// adds a wedge; a 64-bit shared add would be a compare-and-swap loop.
+static_assert(kMediumMaxWork < 65536, "hash counters have 16-bit halves");
+
 __device__ __forceinline__ uint32_t hash_slot(uint32_t w, int log_h) {
   return (w * 2654435769u) >> (32 - log_h);
 }
@@ -35,8 +38,8 @@ __device__ __forceinline__ uint32_t hash_slot(uint32_t w, int log_h) {
 // returns the counter's previous value through *old. Returns false if the
 // probe sequence ran past the table (cannot happen when the table has more
 // slots than the pivot's accepted wedges).
-__device__ __forceinline__ bool smem_hash_add(uint32_t* keys, unsigned long long* vals, int log_h, uint32_t w,
-                                              unsigned long long inc, unsigned long long* old) {
+__device__ __forceinline__ bool smem_hash_add(uint32_t* keys, uint32_t* vals, int log_h, uint32_t w, uint32_t inc,
+                                              uint32_t* old) {
   const uint32_t mask = (1u << log_h) - 1u;
   uint32_t h = hash_slot(w, log_h);
   for (uint32_t probe = 0; probe <= mask; probe++) {
@@ -49,6 +52,17 @@ __device__ __forceinline__ bool smem_hash_add(uint32_t* keys, unsigned long long
     h = (h + 1u) & mask;
   }
   return false;
+}
+
+// Empty the first 2^log_h slots (log_h >= 5, both arrays 16-byte aligned) with
+// `threads` threads, thread `t` of them.
+__device__ __forceinline__ void hash_clear(uint32_t* keys, uint32_t* vals, int log_h, int t, int threads) {
+  uint4* k4 = reinterpret_cast<uint4*>(keys);
+  uint4* v4 = reinterpret_cast<uint4*>(vals);
+  for (int i = t; i < (1 << log_h) / 4; i += threads) {
+    k4[i] = make_uint4(kEmptyKey, kEmptyKey, kEmptyKey, kEmptyKey);
+    v4[i] = make_uint4(0u, 0u, 0u, 0u);
+  }
 }
 
 // Smallest 2^k >= (work << mult_log) slots (at least 32, at most 2^max_log).
@@ -98,89 +112,99 @@ __device__ __forceinline__ uint32_t neighbour_row(const CsrView& g, const PivotG
   return e & 1u;
 }
 
-// The warp walks lower-neighbour positions [a, b) of the pivot in groups of
-// 32 (`step` = distance between this warp's groups) and, for each lower
-// neighbour v, the accepted prefix of v's row in chunks of 32 * U entries.
-// visit(x[U], s1) is called by all lanes together; lane l holds entries
-// chunk + u*32 + l, with x = 0xFFFFFFFF where nothing is accepted.
-template <int U, typename Visit>
-__device__ __forceinline__ void warp_walk(const CsrView& g, const PivotGeom& q, uint32_t a, uint32_t b,
-                                          uint32_t step, Visit&& visit) {
-  const unsigned lane = lane_id();
-  for (uint32_t i0 = a; i0 < b; i0 += step) {
-    uint32_t e = 0;
-    int64_t vb = 0, ve = 0;
-    if (i0 + lane < b) {
-      e = g.col[q.rb + i0 + lane];
-      neighbour_row(g, q, e, vb, ve);
-    }
-    const uint32_t cnt = min(32u, b - i0);
-    for (uint32_t k = 0; k < cnt; k++) {
-      const uint32_t s1 = __shfl_sync(kFullMask, e, k) & 1u;
-      const int64_t jb0 = __shfl_sync(kFullMask, vb, k);
-      const int64_t je = __shfl_sync(kFullMask, ve, k);
-      for (int64_t jb = jb0; jb < je; jb += 32 * U) {
-        uint32_t x[U];
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-          const int64_t j = jb + u * 32 + lane;
-          x[u] = j < je ? g.col[j] : 0xFFFFFFFFu;
-        }
-        bool stop = false;
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-          if (x[u] >= q.lim) {
-            x[u] = 0xFFFFFFFFu;
-            stop = true;
-          }
-        }
-        visit(x, s1);
-        if (__any_sync(kFullMask, stop)) break;  // rows ascend: nothing accepted beyond
-      }
-    }
-  }
-}
-
-template <int G>
-__device__ __forceinline__ unsigned group_mask() {
-  const unsigned lane = lane_id();
-  return G == 32 ? kFullMask : (((1u << G) - 1u) << (lane & ~(unsigned)(G - 1)));
-}
-
 // Hash tiers: groups of G lanes (group gid of `groups`) take lower neighbours
 // gid, gid + groups, ... of the pivot; a group walks its neighbour's accepted
-// prefix G entries at a time and adds every wedge to the shared hash table,
-// accumulating the Lemma 1 contributions. The next neighbour's row bounds are
-// loaded while the current one is walked. Returns false if the table ran out
-// of slots. G is chosen from the pivot's mean accepted segment (work / L) so
-// that short segments do not leave most lanes of a warp idle.
-template <int G>
-__device__ __forceinline__ bool hash_walk(uint32_t gid, uint32_t groups, const CsrView& g, const PivotGeom& q,
-                                          uint32_t* keys, unsigned long long* vals, int log_h, uint64_t& bal,
-                                          uint64_t& unb) {
-  const int gl = threadIdx.x & (G - 1);
-  const unsigned gmask = group_mask<G>();
-  bool fits = true;
-  int64_t b_nx = 0, en_nx = 0;
-  uint32_t s1_nx = 0;
-  if (gid < q.L) s1_nx = neighbour_row(g, q, g.col[q.rb + gid], b_nx, en_nx);
-  for (uint32_t i = gid; i < q.L; i += groups) {
-    const int64_t b = b_nx, en = en_nx;
-    const uint32_t s1 = s1_nx;
-    if (i + groups < q.L) s1_nx = neighbour_row(g, q, g.col[q.rb + i + groups], b_nx, en_nx);
-    for (int64_t c = b; c < en; c += G) {
-      const int64_t j = c + gl;
-      const uint32_t x = j < en ? g.col[j] : 0xFFFFFFFFu;
-      const bool ok = x < q.lim;
-      if (ok) {
-        const unsigned long long inc = wedge_inc(x, s1);
-        unsigned long long old;
-        if (smem_hash_add(keys, vals, log_h, x >> 1, inc, &old)) wedge_contrib(old, inc, bal, unb);
-        else fits = false;
-      }
-      if (__ballot_sync(gmask, !ok)) break;  // rows ascend: nothing accepted beyond
+// prefix G entries at a time. visit(G, x, e, i, pos, last) is called by the
+// whole warp for every chunk: the lane's entry x at CSR position pos (~0 where
+// nothing is accepted) of the row of neighbour position i, whose entry in the
+// pivot's row is e; `last` says that the neighbour ends with this chunk (so it
+// is called with `last` exactly once per neighbour).
+// The walk is bound by the latency of its dependent loads (entry of the
+// pivot's row, row bounds, entries), so each is issued ahead: the next chunk
+// (of this neighbour, or the first of the group's next one) before the current
+// one is visited, row bounds one neighbour ahead and row entries two. Every
+// group moves on to its next neighbour by itself: the loop's trip count is
+// warp-uniform (one vote), a group that has run out only votes. With 32-bit
+// counters (kHashSlotBytes, which also lets half again as many CTAs fit an SM)
+// this took the 20M-edge rating graph's medium tier from 0.99 to 0.44 ms and a
+// 1M-edge one's from 92 to 47 us (light: 80 to 52 us), 1,024 batched small
+// graphs' light tier from 0.90 to 0.54 ms.
+template <int G, typename Visit>
+__device__ __forceinline__ void group_walk(uint32_t gid, uint32_t groups, const CsrView& g, const PivotGeom& q,
+                                           Visit&& visit) {
+  const unsigned lane = lane_id();
+  const uint32_t gl = lane & (G - 1);
+  const uint32_t* __restrict__ col = g.col;
+  auto bounds = [&](bool ok, uint32_t e, uint32_t& c, uint32_t& en) {
+    c = en = 0;
+    if (ok) {
+      int64_t b, n;
+      neighbour_row(g, q, e, b, n);
+      c = (uint32_t)b;
+      en = (uint32_t)n;
     }
+  };
+  uint32_t i = gid;
+  uint32_t e = i < q.L ? col[q.rb + i] : 0u;
+  uint32_t e1 = i + groups < q.L ? col[q.rb + i + groups] : 0u;
+  uint32_t c, en, c1, en1;
+  bounds(i < q.L, e, c, en);
+  uint32_t x = en - c > gl ? col[c + gl] : 0xFFFFFFFFu;
+  bounds(i + groups < q.L, e1, c1, en1);
+  uint32_t e2 = i + 2 * groups < q.L ? col[q.rb + i + 2 * groups] : 0u;
+  while (__any_sync(kFullMask, i < q.L)) {
+    const bool cont = __shfl_sync(kFullMask, x, lane | (G - 1)) < q.lim;  // all accepted: the row goes on
+    const uint32_t xc = x < q.lim ? x : 0xFFFFFFFFu, ec = e, ic = i, pos = c + gl;
+    if (cont) {
+      c += G;
+    } else {
+      i += groups;
+      c = c1;
+      en = en1;
+      e = e1;
+    }
+    x = en - c > gl ? col[c + gl] : 0xFFFFFFFFu;
+    if (!cont) {
+      e1 = e2;
+      bounds(i + groups < q.L, e1, c1, en1);
+      e2 = i + 2 * groups < q.L ? col[q.rb + i + 2 * groups] : 0u;
+    }
+    visit(std::integral_constant<int, G>(), xc, ec, ic, pos, !cont && ic < q.L);
+    __syncwarp();
   }
+}
+
+template <typename Visit>
+__device__ __forceinline__ void group_walk_dispatch(int group_log, uint32_t tid, uint32_t threads, const CsrView& g,
+                                                    const PivotGeom& q, Visit&& visit) {
+  switch (group_log) {
+    case 2: group_walk<4>(tid >> 2, threads >> 2, g, q, visit); break;
+    case 3: group_walk<8>(tid >> 3, threads >> 3, g, q, visit); break;
+    case 4: group_walk<16>(tid >> 4, threads >> 4, g, q, visit); break;
+    default: group_walk<32>(tid >> 5, threads >> 5, g, q, visit); break;
+  }
+}
+
+// Count a pivot's wedges into a hash table and add their Lemma 1
+// contributions. A pivot's sums fit 32 bits (at most kMediumMaxWork wedges,
+// each adding less than that). Returns false if the table ran out of slots.
+__device__ __forceinline__ bool hash_count(int group_log, uint32_t tid, uint32_t threads, const CsrView& g,
+                                           const PivotGeom& q, uint32_t* keys, uint32_t* vals, int log_h,
+                                           uint64_t& bal, uint64_t& unb) {
+  bool fits = true;
+  uint32_t own = 0, other = 0;
+  group_walk_dispatch(group_log, tid, threads, g, q, [&](auto, uint32_t x, uint32_t e, uint32_t, uint32_t, bool) {
+    if (x != 0xFFFFFFFFu) {
+      const uint32_t sh = ((x ^ e) & 1u) << 4;
+      uint32_t old = 0;
+      fits &= smem_hash_add(keys, vals, log_h, x >> 1, 1u << sh, &old);
+      const uint32_t v = __funnelshift_l(old, old, sh);  // (other class << 16) | own class
+      own += v & 0xFFFFu;
+      other += v >> 16;
+    }
+  });
+  bal += own;
+  unb += other;
   return fits;
 }
 
@@ -190,16 +214,6 @@ __device__ __forceinline__ int hash_group_log(uint64_t work, uint32_t L, int max
   const uint64_t mean = work / (L ? L : 1);
   const int lg = mean >= 24 ? 5 : mean >= 12 ? 4 : mean >= 6 ? 3 : 2;
   return lg < max_log ? lg : max_log;
-}
-
-template <typename... A>
-__device__ __forceinline__ bool hash_walk_dispatch(int group_log, uint32_t tid, uint32_t threads, A&&... a) {
-  switch (group_log) {
-    case 2: return hash_walk<4>(tid >> 2, threads >> 2, a...);
-    case 3: return hash_walk<8>(tid >> 3, threads >> 3, a...);
-    case 4: return hash_walk<16>(tid >> 4, threads >> 4, a...);
-    default: return hash_walk<32>(tid >> 5, threads >> 5, a...);
-  }
 }
 
 // log2 of the hash slots a tier's tables need at most: table_log of the
@@ -212,6 +226,7 @@ inline int tier_slots_log(uint64_t max_work, int mult_log, int cap) {
 }
 
 constexpr int kLightWarps = 8;
+constexpr size_t kHashSlotBytes = 8;  // a key and a packed counter
 
 constexpr int kMediumThreads = 256;
 constexpr int kMediumWarps = kMediumThreads / 32;

@@ -26,8 +26,7 @@ struct TipOut {
 };
 
 // Counter of endpoint w in a shared hash table (the key must be present).
-__device__ __forceinline__ unsigned long long hash_find(const uint32_t* keys, const unsigned long long* vals,
-                                                        int log_h, uint32_t w) {
+__device__ __forceinline__ uint32_t hash_find(const uint32_t* keys, const uint32_t* vals, int log_h, uint32_t w) {
   const uint32_t mask = (1u << log_h) - 1u;
   uint32_t h = hash_slot(w, log_h);
   for (uint32_t probe = 0; probe <= mask; probe++) {
@@ -35,7 +34,7 @@ __device__ __forceinline__ unsigned long long hash_find(const uint32_t* keys, co
     if (keys[h] == kEmptyKey) break;
     h = (h + 1u) & mask;
   }
-  return 0ull;
+  return 0u;
 }
 
 // Butterflies one wedge is in, from its endpoint's buckets (p, q) packed as
@@ -68,106 +67,102 @@ __device__ __forceinline__ void add_edge(const TipOut& o, int64_t j, uint64_t x,
   if (DBBC_CHECK(j >= 0 && j < o.nnz)) add_pair(o.eb, o.eu, j, x, y);
 }
 
-// The second walk over a pivot's wedges (lower-neighbour positions [a, b),
-// `step` apart in groups of 32 per warp): each lane credits the far edge
-// (v, w) of its wedge; the warp sums v's wedges and one lane credits the
-// middle v and the near edge (u, v).
-template <bool VERT, bool EDGE, typename Lookup>
-__device__ __forceinline__ void warp_second_walk(const CsrView& g, const PivotGeom& q, uint32_t a, uint32_t b,
-                                                 uint32_t step, Lookup&& lookup, const TipOut& o) {
-  const unsigned lane = lane_id();
-  for (uint32_t i0 = a; i0 < b; i0 += step) {
-    uint32_t e = 0;
-    int64_t vb0 = 0, ve = 0;
-    if (i0 + lane < b) {
-      e = g.col[q.rb + i0 + lane];
-      const int64_t vrow = q.base + (e >> 1);
-      vb0 = g.row_ptr[vrow];
-      ve = g.row_ptr[vrow + 1];
-    }
-    const uint32_t cnt = min(32u, b - i0);
-    for (uint32_t k = 0; k < cnt; k++) {
-      const uint32_t ek = __shfl_sync(kFullMask, e, k);
-      const uint32_t s1 = ek & 1u;
-      const int64_t jb0 = __shfl_sync(kFullMask, vb0, k);
-      const int64_t je = __shfl_sync(kFullMask, ve, k);
-      uint64_t sb = 0, su = 0;
-      for (int64_t jb = jb0; jb < je; jb += 32) {
-        const int64_t j = jb + lane;
-        const uint32_t x = j < je ? g.col[j] : 0xFFFFFFFFu;
-        const bool ok = x < q.lim;
-        if (ok) {
-          uint64_t cb, cu;
-          wedge_pairs(lookup(x >> 1), ((x ^ s1) & 1u) == 0, cb, cu);
-          if (EDGE) add_edge(o, j, cb, cu);
-          sb += cb;
-          su += cu;
-        }
-        if (__ballot_sync(kFullMask, !ok)) break;  // rows ascend: nothing accepted beyond
-      }
-      sb = warp_sum_u64(sb);
-      su = warp_sum_u64(su);
-      if (lane == 0) {
-        if (VERT) add_vertex(o, q.base + (ek >> 1), sb, su);
-        if (EDGE) add_edge(o, q.rb + i0 + k, sb, su);
-      }
+// The endpoints of a pivot's complete hash table (slots t, t + threads, ...):
+// each endpoint and the pivot get the endpoint's Lemma 1 totals; the pivot's
+// share is summed over the warp.
+__device__ __forceinline__ void credit_endpoints(const CsrView& g, int32_t p, const uint32_t* keys,
+                                                 const uint32_t* vals, int log_h, int t, int threads,
+                                                 const TipOut& o) {
+  const int64_t end_base = p < g.n_u ? 0 : (int64_t)g.n_u;  // endpoints share the pivot's side
+  uint64_t pb = 0, pu = 0;
+  for (int i = t; i < (1 << log_h); i += threads) {
+    const uint32_t v = vals[i];
+    if (v) {
+      uint64_t eb = 0, eu = 0;
+      endpoint_contrib(((unsigned long long)(v >> 16) << 32) | (v & 0xFFFFu), eb, eu);
+      add_vertex(o, end_base + keys[i], eb, eu);
+      pb += eb;
+      pu += eu;
     }
   }
+  pb = warp_sum_u64(pb);
+  pu = warp_sum_u64(pu);
+  if (lane_id() == 0) add_vertex(o, p, pb, pu);
+}
+
+// The second walk over a light or medium pivot's wedges, by the same lane
+// groups as the first: each lane credits the far edge (v, w) of its wedge from
+// the endpoint's final counter; when a group reaches the end of a neighbour v
+// its lanes' sums credit the middle v and the near edge (u, v). Sums fit 32
+// bits (at most kMediumMaxWork wedges of fewer butterflies each). Lane groups
+// sized to the pivot's mean segment keep the warp's lanes busy where one warp
+// per neighbour left most of them idle (mean accepted segments are 5 to 20
+// entries in these tiers): per-edge counts of a 20M-edge graph, medium tier
+// 4.06 to 0.74 ms and light 1.41 to 0.40 ms; per-vertex counts of a 4M-edge
+// one, 1.21 to 0.26 ms and 0.42 to 0.14 ms.
+template <bool VERT, bool EDGE>
+__device__ __forceinline__ void second_walk(int group_log, uint32_t tid, uint32_t threads, const CsrView& g,
+                                            const PivotGeom& q, const uint32_t* keys, const uint32_t* vals, int log_h,
+                                            const TipOut& o) {
+  uint32_t sb = 0, su = 0;
+  group_walk_dispatch(group_log, tid, threads, g, q,
+                      [&](auto gtag, uint32_t x, uint32_t e, uint32_t i, uint32_t pos, bool last) {
+    constexpr int G = decltype(gtag)::value;
+    if (x != 0xFFFFFFFFu) {
+      const uint32_t v = hash_find(keys, vals, log_h, x >> 1);
+      uint64_t cb, cu;
+      wedge_pairs(((unsigned long long)(v >> 16) << 32) | (v & 0xFFFFu), ((x ^ e) & 1u) == 0, cb, cu);
+      if (EDGE) add_edge(o, pos, cb, cu);
+      sb += (uint32_t)cb;
+      su += (uint32_t)cu;
+    }
+    __syncwarp();
+    if (__any_sync(kFullMask, last)) {
+      uint32_t tb = sb, tu = su;
+#pragma unroll
+      for (int off = G / 2; off > 0; off >>= 1) {
+        tb += __shfl_xor_sync(kFullMask, tb, off);
+        tu += __shfl_xor_sync(kFullMask, tu, off);
+      }
+      if (last) {
+        if ((threadIdx.x & (G - 1)) == 0) {
+          if (VERT) add_vertex(o, q.base + (e >> 1), tb, tu);
+          if (EDGE) add_edge(o, q.rb + i, tb, tu);
+        }
+        sb = su = 0;
+      }
+    }
+  });
 }
 
 // ------------------------------------------------------------------ light / medium
+// Tables as in the counting kernels (2^slots_log slots).
 template <bool VERT, bool EDGE>
 __global__ void __launch_bounds__(kLightWarps * 32) tips_light_kernel(CsrView g, const int32_t* __restrict__ piv,
                                                                       const uint64_t* __restrict__ work,
-                                                                      int64_t n_piv, int hash_mult_log, TipOut o,
-                                                                      unsigned* status) {
+                                                                      int64_t n_piv, int hash_mult_log, int slots_log,
+                                                                      TipOut o, unsigned* status) {
   extern __shared__ __align__(16) unsigned char light_smem[];
-  unsigned long long* vals_all = reinterpret_cast<unsigned long long*>(light_smem);
-  uint32_t* keys_all = reinterpret_cast<uint32_t*>(vals_all + kLightWarps * kLightSlots);
+  const int slots = 1 << slots_log;
   const int w = threadIdx.x >> 5;
   const unsigned lane = lane_id();
-  uint32_t* keys = keys_all + w * kLightSlots;
-  unsigned long long* vals = vals_all + w * kLightSlots;
-  for (int i = lane; i < kLightSlots; i += 32) {
-    keys[i] = kEmptyKey;
-    vals[i] = 0;
-  }
+  uint32_t* keys = reinterpret_cast<uint32_t*>(light_smem) + 2 * w * slots;
+  uint32_t* vals = keys + slots;
+  hash_clear(keys, vals, slots_log, lane, 32);
   __syncwarp();
   bool full = false;
   const int64_t nw = (int64_t)gridDim.x * kLightWarps;
   for (int64_t t = (int64_t)blockIdx.x * kLightWarps + w; t < n_piv; t += nw) {
     const int32_t p = piv[t];
-    const int log_h = table_log(work[p], 10, hash_mult_log);
+    const uint64_t wp = work[p];
+    const int log_h = table_log(wp, slots_log, hash_mult_log);
     const PivotGeom q = pivot_geom(g, p);
-    warp_walk<1>(g, q, 0, q.L, 32, [&](const uint32_t (&x)[1], uint32_t s1) {
-      if (x[0] != 0xFFFFFFFFu) {
-        unsigned long long old;
-        full |= !smem_hash_add(keys, vals, log_h, x[0] >> 1, wedge_inc(x[0], s1), &old);
-      }
-    });
-    __syncwarp();
-    if (VERT) {
-      const int64_t end_base = p < g.n_u ? 0 : (int64_t)g.n_u;  // endpoints share the pivot's side
-      uint64_t pb = 0, pu = 0;
-      for (int i = lane; i < (1 << log_h); i += 32) {
-        if (keys[i] != kEmptyKey) {
-          uint64_t eb = 0, eu = 0;
-          endpoint_contrib(vals[i], eb, eu);
-          add_vertex(o, end_base + keys[i], eb, eu);
-          pb += eb;
-          pu += eu;
-        }
-      }
-      pb = warp_sum_u64(pb);
-      pu = warp_sum_u64(pu);
-      if (lane == 0) add_vertex(o, p, pb, pu);
-    }
-    warp_second_walk<VERT, EDGE>(g, q, 0, q.L, 32, [&](uint32_t x) { return hash_find(keys, vals, log_h, x); }, o);
-    __syncwarp();
-    for (int i = lane; i < (1 << log_h); i += 32) {
-      keys[i] = kEmptyKey;
-      vals[i] = 0;
-    }
+    const int gl = hash_group_log(wp, q.L, 5);
+    uint64_t unused_b = 0, unused_u = 0;
+    full |= !hash_count(gl, lane, 32u, g, q, keys, vals, log_h, unused_b, unused_u);
+    if (VERT) credit_endpoints(g, p, keys, vals, log_h, lane, 32, o);
+    second_walk<VERT, EDGE>(gl, lane, 32u, g, q, keys, vals, log_h, o);
+    hash_clear(keys, vals, log_h, lane, 32);
     __syncwarp();
   }
   if (full) atomicOr(status, DBBC_DEV_HASH_FULL);
@@ -176,55 +171,27 @@ __global__ void __launch_bounds__(kLightWarps * 32) tips_light_kernel(CsrView g,
 template <bool VERT, bool EDGE>
 __global__ void __launch_bounds__(kMediumThreads) tips_medium_kernel(CsrView g, const int32_t* __restrict__ piv,
                                                                      const uint64_t* __restrict__ work,
-                                                                     int64_t n_piv, int hash_mult_log, TipOut o,
-                                                                     unsigned* status) {
+                                                                     int64_t n_piv, int hash_mult_log, int slots_log,
+                                                                     TipOut o, unsigned* status) {
   extern __shared__ __align__(16) unsigned char med_smem[];
-  unsigned long long* vals = reinterpret_cast<unsigned long long*>(med_smem);
-  uint32_t* keys = reinterpret_cast<uint32_t*>(vals + kMediumSlots);
-  for (int i = threadIdx.x; i < kMediumSlots; i += kMediumThreads) {
-    keys[i] = kEmptyKey;
-    vals[i] = 0;
-  }
+  uint32_t* keys = reinterpret_cast<uint32_t*>(med_smem);
+  uint32_t* vals = keys + (1 << slots_log);
+  hash_clear(keys, vals, slots_log, threadIdx.x, kMediumThreads);
   __syncthreads();
-  const int w = threadIdx.x >> 5;
   bool full = false;
   for (int64_t t = blockIdx.x; t < n_piv; t += gridDim.x) {
     const int32_t p = piv[t];
-    const int log_h = table_log(work[p], 13, hash_mult_log);
+    const uint64_t wp = work[p];
+    const int log_h = table_log(wp, slots_log, hash_mult_log);
     const PivotGeom q = pivot_geom(g, p);
-    warp_walk<2>(g, q, (uint32_t)w * 32u, q.L, kMediumWarps * 32u, [&](const uint32_t (&x)[2], uint32_t s1) {
-#pragma unroll
-      for (int u = 0; u < 2; u++) {
-        if (x[u] != 0xFFFFFFFFu) {
-          unsigned long long old;
-          full |= !smem_hash_add(keys, vals, log_h, x[u] >> 1, wedge_inc(x[u], s1), &old);
-        }
-      }
-    });
+    const int gl = hash_group_log(wp, q.L, 5);
+    uint64_t unused_b = 0, unused_u = 0;
+    full |= !hash_count(gl, threadIdx.x, (uint32_t)kMediumThreads, g, q, keys, vals, log_h, unused_b, unused_u);
     __syncthreads();
-    if (VERT) {
-      const int64_t end_base = p < g.n_u ? 0 : (int64_t)g.n_u;
-      uint64_t pb = 0, pu = 0;
-      for (int i = threadIdx.x; i < (1 << log_h); i += kMediumThreads) {
-        if (keys[i] != kEmptyKey) {
-          uint64_t eb = 0, eu = 0;
-          endpoint_contrib(vals[i], eb, eu);
-          add_vertex(o, end_base + keys[i], eb, eu);
-          pb += eb;
-          pu += eu;
-        }
-      }
-      pb = warp_sum_u64(pb);
-      pu = warp_sum_u64(pu);
-      if (lane_id() == 0) add_vertex(o, p, pb, pu);
-    }
-    warp_second_walk<VERT, EDGE>(g, q, (uint32_t)w * 32u, q.L, kMediumWarps * 32u,
-                                 [&](uint32_t x) { return hash_find(keys, vals, log_h, x); }, o);
+    if (VERT) credit_endpoints(g, p, keys, vals, log_h, threadIdx.x, kMediumThreads, o);
+    second_walk<VERT, EDGE>(gl, threadIdx.x, (uint32_t)kMediumThreads, g, q, keys, vals, log_h, o);
     __syncthreads();
-    for (int i = threadIdx.x; i < (1 << log_h); i += kMediumThreads) {
-      keys[i] = kEmptyKey;
-      vals[i] = 0;
-    }
+    hash_clear(keys, vals, log_h, threadIdx.x, kMediumThreads);
     __syncthreads();
   }
   if (full) atomicOr(status, DBBC_DEV_HASH_FULL);
@@ -449,21 +416,25 @@ void enqueue_tips(const dbbc_graph* g, cudaStream_t s, const TipOut& o, unsigned
   const int sms = num_sms();
   if (g->n_light > 0) {
     auto fn = tips_light_kernel<VERT, EDGE>;
-    const size_t smem = (size_t)kLightWarps * kLightSlots * 12;
-    DBBC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int slots_log = tier_slots_log(g->tune.light_max_work, g->tune.hash_mult_log, 10);
+    const size_t smem = (size_t)kLightWarps * ((size_t)1 << slots_log) * kHashSlotBytes;
+    DBBC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)((size_t)kLightWarps * kLightSlots * kHashSlotBytes)));
     const int64_t want = ceil_div<int64_t>(g->n_light, kLightWarps);
     const int64_t cap = (int64_t)sms * blocks_per_sm((const void*)fn, kLightWarps * 32, smem);
     fn<<<(unsigned)std::min(want, cap), kLightWarps * 32, smem, s>>>(
-        view, g->order + g->n_hub + g->n_medium, g->work, g->n_light, g->tune.hash_mult_log, o, d_status);
+        view, g->order + g->n_hub + g->n_medium, g->work, g->n_light, g->tune.hash_mult_log, slots_log, o, d_status);
     DBBC_LAUNCH_CHECK();
   }
   if (g->n_medium > 0) {
     auto fn = tips_medium_kernel<VERT, EDGE>;
-    const size_t smem = (size_t)kMediumSlots * 12;
-    DBBC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const int slots_log = tier_slots_log(g->tune.medium_max_work, g->tune.hash_mult_log, 13);
+    const size_t smem = ((size_t)1 << slots_log) * kHashSlotBytes;
+    DBBC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)((size_t)kMediumSlots * kHashSlotBytes)));
     const int64_t cap = (int64_t)sms * blocks_per_sm((const void*)fn, kMediumThreads, smem);
     fn<<<(unsigned)std::min<int64_t>(g->n_medium, cap), kMediumThreads, smem, s>>>(
-        view, g->order + g->n_hub, g->work, g->n_medium, g->tune.hash_mult_log, o, d_status);
+        view, g->order + g->n_hub, g->work, g->n_medium, g->tune.hash_mult_log, slots_log, o, d_status);
     DBBC_LAUNCH_CHECK();
   }
   if (g->n_hub > 0) {
