@@ -10,12 +10,22 @@
 namespace dbbc {
 
 // Components of a disjoint union as seen by the kernels: component c owns the
-// side ids (and, after ranking, the side ranks) [uoff[c], uoff[c+1]) of U and
-// [voff[c], voff[c+1]) of V. A plain graph is one component.
+// side ids (and, after ranking, the side ranks) [uo(c), uo(c + 1)) of U and
+// [vo(c), vo(c + 1)) of V. A plain graph is one component and has no arrays.
+__device__ __forceinline__ int32_t component_of(const int64_t* off, int32_t n_graphs, int64_t side_id);
 struct UnionView {
   const int64_t* uoff;
   const int64_t* voff;
   int32_t n_graphs;
+  int64_t n_u, n_v;
+  __device__ __forceinline__ int64_t uo(int32_t c) const { return n_graphs == 1 ? (c ? n_u : 0) : uoff[c]; }
+  __device__ __forceinline__ int64_t vo(int32_t c) const { return n_graphs == 1 ? (c ? n_v : 0) : voff[c]; }
+  __device__ __forceinline__ int32_t comp_u(int64_t id) const {
+    return n_graphs == 1 ? 0 : component_of(uoff, n_graphs, id);
+  }
+  __device__ __forceinline__ int32_t comp_v(int64_t id) const {
+    return n_graphs == 1 ? 0 : component_of(voff, n_graphs, id);
+  }
 };
 
 __device__ __forceinline__ int32_t component_of(const int64_t* off, int32_t n_graphs, int64_t side_id) {
@@ -47,56 +57,6 @@ __device__ __forceinline__ int64_t upper_bound_dev(const T* a, int64_t n, T x) {
   return lo;
 }
 
-__global__ void validate_kernel(const int32_t* __restrict__ u, const int32_t* __restrict__ v,
-                                const int8_t* __restrict__ s, int64_t m, int32_t n_u, int32_t n_v, unsigned* err) {
-  unsigned e = 0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t a = u[i], b = v[i];
-    const int8_t c = s[i];
-    if (a < 0 || a >= n_u) e |= 1u;
-    if (b < 0 || b >= n_v) e |= 2u;
-    if (c != 1 && c != -1) e |= 4u;
-  }
-  e = __reduce_or_sync(kFullMask, e);
-  if (lane_id() == 0 && e) atomicOr(err, e);
-}
-
-__global__ void edge_keys_kernel(const int32_t* __restrict__ u, const int32_t* __restrict__ v, int64_t m, int bits_v,
-                                 uint64_t* __restrict__ key, uint32_t* __restrict__ idx) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    key[i] = ((uint64_t)(uint32_t)u[i] << bits_v) | (uint32_t)v[i];
-    idx[i] = (uint32_t)i;
-  }
-}
-
-// flag[i] = 1 iff i is the last occurrence of its key (keys sorted stably, so
-// the last of a run is the latest input occurrence).
-__global__ void run_last_kernel(const uint64_t* __restrict__ key, int64_t m, uint32_t* __restrict__ flag,
-                                unsigned* dup) {
-  bool any_dup = false;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    const bool last = (i == m - 1) || (key[i] != key[i + 1]);
-    flag[i] = last ? 1u : 0u;
-    any_dup |= !last;
-  }
-  if (__any_sync(kFullMask, any_dup) && lane_id() == 0) atomicOr(dup, 8u);
-}
-
-__global__ void compact_edges_kernel(const uint64_t* __restrict__ key, const uint32_t* __restrict__ idx,
-                                     const uint32_t* __restrict__ flag, const uint32_t* __restrict__ pos,
-                                     const int8_t* __restrict__ sign, int64_t m, int bits_v,
-                                     int32_t* __restrict__ eu, int32_t* __restrict__ ev, int8_t* __restrict__ es) {
-  const uint64_t mask_v = (bits_v >= 64) ? ~0ull : ((1ull << bits_v) - 1);
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    if (!flag[i]) continue;
-    const uint32_t j = pos[i];
-    const uint64_t k = key[i];
-    eu[j] = (int32_t)(k >> bits_v);
-    ev[j] = (int32_t)(k & mask_v);
-    es[j] = sign[idx[i]];
-  }
-}
-
 // deg[id] += 1 for every lane with ok, as one atomic per run of equal ids in
 // consecutive lanes (edges that arrive grouped by an endpoint form long runs).
 __device__ __forceinline__ void add_runs(int32_t* __restrict__ deg, int32_t id, bool ok) {
@@ -110,62 +70,125 @@ __device__ __forceinline__ void add_runs(int32_t* __restrict__ deg, int32_t id, 
   if (ok && head) atomicAdd(&deg[x], len);
 }
 
-// Degrees over unified ids (V ids follow the U ids).
-__global__ void degree_kernel(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev, int64_t m,
-                              int32_t n_u, int32_t* __restrict__ deg) {
+// Validation and degrees in one read of the edges: flags the edges whose ids
+// are out of range or whose sign is not +-1 (every later kernel of the build
+// then returns at once), and counts the others' degrees over unified ids (V
+// ids follow the U ids).
+__global__ void degree_kernel(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
+                              const int8_t* __restrict__ es, int64_t m, int32_t n_u, int32_t n_v,
+                              int32_t* __restrict__ deg, unsigned* flags) {
   constexpr int kRound = 4;  // edges per thread per round, their loads in flight together
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t iters = (m + stride - 1) / stride;  // the same for every lane: the warp votes together
   const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned bad = 0;
   for (int64_t it = 0; it < iters; it += kRound) {
     int32_t a[kRound], b[kRound];
+    int8_t c[kRound];
 #pragma unroll
     for (int j = 0; j < kRound; j++) {
       const int64_t i = (it + j) * stride + t0;
       a[j] = i < m ? eu[i] : 0;
-      b[j] = i < m ? n_u + ev[i] : 0;
+      b[j] = i < m ? ev[i] : 0;
+      c[j] = i < m ? es[i] : (int8_t)1;
     }
 #pragma unroll
     for (int j = 0; j < kRound; j++) {
-      const bool ok = (it + j) * stride + t0 < m;
-      add_runs(deg, a[j], ok);
-      add_runs(deg, b[j], ok);
+      const bool in = (it + j) * stride + t0 < m;
+      const bool ok_u = a[j] >= 0 && a[j] < n_u, ok_v = b[j] >= 0 && b[j] < n_v;
+      if (in) bad |= (ok_u ? 0u : kPrepBadU) | (ok_v ? 0u : kPrepBadV) | (c[j] == 1 || c[j] == -1 ? 0u : kPrepBadSign);
+      add_runs(deg, a[j], in && ok_u);
+      add_runs(deg, ok_v ? n_u + b[j] : 0, in && ok_v);
     }
   }
+  bad = __reduce_or_sync(kFullMask, bad);
+  if (lane_id() == 0 && bad) atomicOr(flags, bad);
 }
 
 // Sort key per vertex: (side, component, degree, id within the component).
 // Ascending order is the Def. 3 priority within each side of each component
 // (V ids follow U ids in the unified space); components occupy contiguous
 // rank ranges, which keeps a component's accepted endpoints together.
-__global__ void vertex_keys_kernel(const int32_t* __restrict__ deg, int64_t n, int32_t n_u, int bits_comp,
-                                   int bits_deg, int bits_id, UnionView un, uint64_t* __restrict__ key) {
+// Degrees of distinct edges fit bits_deg; repeated pairs can push one past it,
+// and is cut off there: such a list is ranked again without the repeats.
+// Counts the digits of the sort (bits_id and up) as it goes.
+__global__ void __launch_bounds__(256) vertex_keys_kernel(const int32_t* __restrict__ deg, int64_t n, int32_t n_u,
+                                                          int bits_comp, int bits_deg, int bits_id, UnionView un,
+                                                          uint64_t* __restrict__ key, int passes, uint32_t* hist,
+                                                          const unsigned* flags) {
+  __shared__ uint32_t h[kRsMaxPasses][256];
+  if (cta_stopped(flags)) return;
+  DigitCounts dc{h, passes, bits_id};
+  dc.start();
+  const uint64_t deg_mask = (1ull << bits_deg) - 1;
   for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
     const uint64_t side = x >= n_u ? 1 : 0;
     const int64_t sid = side ? x - n_u : x;
-    const int64_t* off = side ? un.voff : un.uoff;
-    const int32_t c = component_of(off, un.n_graphs, sid);
-    const uint64_t local = (uint64_t)(sid - off[c]);
-    key[x] = (side << (bits_comp + bits_deg + bits_id)) | ((uint64_t)c << (bits_deg + bits_id)) |
-             ((uint64_t)deg[x] << bits_id) | local;
+    const int32_t c = side ? un.comp_v(sid) : un.comp_u(sid);
+    const uint64_t local = (uint64_t)(sid - (side ? un.vo(c) : un.uo(c)));
+    const uint64_t k = (side << (bits_comp + bits_deg + bits_id)) | ((uint64_t)c << (bits_deg + bits_id)) |
+                       (min((uint64_t)(uint32_t)deg[x], deg_mask) << bits_id) | local;
+    key[x] = k;
+    dc.add(k);
   }
+  dc.finish(hist);
 }
 
-__global__ void ranks_kernel(const uint64_t* __restrict__ skey, int64_t n, int32_t n_u, int bits_comp, int bits_deg,
-                             int bits_id, UnionView un, int32_t* __restrict__ vertex, int32_t* __restrict__ side_rank,
-                             int32_t* __restrict__ rowdeg) {
+// Rows in rank order: vertex, degree and (unions) component of every row, the
+// rank of every vertex, and the row pointers, whose prefix sum runs in the
+// same kernel over tiles of kRowTile rows (tile_prefix). Clears the rows' work.
+constexpr int kRowThreads = 256;
+constexpr int kRowItems = 4;
+constexpr int kRowTile = kRowThreads * kRowItems;
+
+__global__ void __launch_bounds__(kRowThreads) ranks_kernel(const uint64_t* __restrict__ skey, int64_t n, int32_t n_u,
+                                                            int bits_comp, int bits_deg, int bits_id, UnionView un,
+                                                            int32_t* __restrict__ vertex,
+                                                            int32_t* __restrict__ side_rank,
+                                                            int32_t* __restrict__ rowdeg, int64_t* __restrict__ row_ptr,
+                                                            int32_t* __restrict__ component,
+                                                            uint64_t* __restrict__ work, uint64_t* state,
+                                                            unsigned* counter, unsigned* flags) {
+  __shared__ uint64_t tot_sh;
+  const int64_t tile = take_tile(counter, flags);
+  if (tile < 0) return;
   const uint64_t id_mask = (1ull << bits_id) - 1, deg_mask = (1ull << bits_deg) - 1;
   const uint64_t comp_mask = (1ull << bits_comp) - 1;
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
-    const uint64_t k = skey[r];
-    const bool side = (k >> (bits_comp + bits_deg + bits_id)) & 1;
-    const int32_t c = bits_comp ? (int32_t)((k >> (bits_deg + bits_id)) & comp_mask) : 0;
-    const int64_t local = (int64_t)(k & id_mask);
-    const int32_t x = side ? (int32_t)(n_u + un.voff[c] + local) : (int32_t)(un.uoff[c] + local);
-    if (!DBBC_CHECK(x >= 0 && x < n)) continue;
-    vertex[r] = x;
-    side_rank[x] = side ? (int32_t)(r - n_u) : (int32_t)r;
-    rowdeg[r] = (int32_t)((k >> bits_id) & deg_mask);
+  const int64_t r0 = tile * kRowTile + (int64_t)threadIdx.x * kRowItems;
+  uint32_t d[kRowItems];
+  uint64_t sum = 0;
+#pragma unroll
+  for (int j = 0; j < kRowItems; j++) {
+    const int64_t r = r0 + j;
+    d[j] = 0;
+    if (r < n) {
+      const uint64_t k = skey[r];
+      const bool side = (k >> (bits_comp + bits_deg + bits_id)) & 1;
+      const int32_t c = bits_comp ? (int32_t)((k >> (bits_deg + bits_id)) & comp_mask) : 0;
+      const int64_t local = (int64_t)(k & id_mask);
+      const int32_t x = side ? (int32_t)(n_u + un.vo(c) + local) : (int32_t)(un.uo(c) + local);
+      d[j] = (uint32_t)((k >> bits_id) & deg_mask);
+      if (DBBC_CHECK(x >= 0 && x < n)) {
+        vertex[r] = x;
+        side_rank[x] = side ? (int32_t)(r - n_u) : (int32_t)r;
+        rowdeg[r] = (int32_t)d[j];
+        work[r] = 0;
+        if (component) component[r] = c;
+      }
+    }
+    sum += d[j];
+  }
+  uint64_t run = block_excl_scan<uint64_t, kRowThreads>(sum, &tot_sh);
+  __syncthreads();
+  uint64_t prefix;
+  if (!tile_prefix(state, tile, tot_sh, flags, &prefix)) return;
+  run += prefix;
+#pragma unroll
+  for (int j = 0; j < kRowItems; j++) {
+    const int64_t r = r0 + j;
+    if (r < n) row_ptr[r] = (int64_t)run;
+    run += d[j];
+    if (r == n - 1) row_ptr[n] = (int64_t)run;
   }
 }
 
@@ -173,60 +196,115 @@ __global__ void ranks_kernel(const uint64_t* __restrict__ skey, int64_t n, int32
 // ku = (U rank << (bits_v + 1)) | (V rank << 1) | negative; the V rows are the
 // same list re-sorted stably by V rank alone, as
 // kv = (V rank << (bits_u + 1)) | (U rank << 1) | negative, which keeps every
-// V row ascending by U rank.
-__global__ void csr_u_keys_kernel(const int32_t* __restrict__ eu, const int32_t* __restrict__ ev,
-                                  const int8_t* __restrict__ es, int64_t m, int32_t n_u,
-                                  const int32_t* __restrict__ side_rank, int bits_v, uint64_t* __restrict__ ku) {
+// V row ascending by U rank. The last pass of each sort also writes the rows'
+// entries (the low bits of the key).
+__global__ void __launch_bounds__(256) csr_u_keys_kernel(const int32_t* __restrict__ eu,
+                                                         const int32_t* __restrict__ ev,
+                                                         const int8_t* __restrict__ es, int64_t m, int32_t n_u,
+                                                         const int32_t* __restrict__ side_rank, int bits_v,
+                                                         uint64_t* __restrict__ ku, int passes, uint32_t* hist,
+                                                         const unsigned* flags) {
+  __shared__ uint32_t h[kRsMaxPasses][256];
+  if (cta_stopped(flags)) return;
+  DigitCounts dc{h, passes, 1};
+  dc.start();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
     const uint64_t ru = (uint32_t)side_rank[eu[i]];
     const uint64_t rv = (uint32_t)side_rank[n_u + ev[i]];
-    ku[i] = (ru << (bits_v + 1)) | (rv << 1) | (es[i] < 0 ? 1u : 0u);
+    const uint64_t k = (ru << (bits_v + 1)) | (rv << 1) | (es[i] < 0 ? 1u : 0u);
+    ku[i] = k;
+    dc.add(k);
   }
+  dc.finish(hist);
 }
 
-// V keys of the U-sorted list, each with its U position (the edge's position
-// in its U row) as the value the V sort carries along.
-__global__ void csr_v_keys_kernel(const uint64_t* __restrict__ ku, int64_t m, int bits_u, int bits_v,
-                                  uint64_t* __restrict__ kv, uint32_t* __restrict__ upos) {
-  const uint64_t mask_v = (1ull << bits_v) - 1;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    const uint64_t k = ku[i];
-    const uint64_t ru = k >> (bits_v + 1), rv = (k >> 1) & mask_v;
-    kv[i] = (rv << (bits_u + 1)) | (ru << 1) | (k & 1u);
-    upos[i] = (uint32_t)i;
-  }
-}
-
-// Flags a repeated (u, v) pair: U-sorted keys that agree in everything but the
-// sign bit are adjacent.
-__global__ void adjacent_dup_kernel(const uint64_t* __restrict__ key, int64_t m, unsigned* dup) {
-  bool any = false;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i + 1 < m; i += (int64_t)gridDim.x * blockDim.x)
-    any |= (key[i] >> 1) == (key[i + 1] >> 1);
-  if (__any_sync(kFullMask, any) && lane_id() == 0) atomicOr(dup, 1u);
-}
-
-// Row and entry of CSR position i: the first m positions are the U rows, the
-// next m the V rows.
-struct CsrKeys {
-  const uint64_t* ku;
-  const uint64_t* kv;
-  const uint32_t* upos;  // upos[k]: the U position of the edge at V position m + k
-  int64_t m;
-  int32_t n_u;
+// V key of a U key.
+struct VKey {
   int bits_u, bits_v;
-  __device__ __forceinline__ int64_t row(int64_t i) const {
-    return i < m ? (int64_t)(ku[i] >> (bits_v + 1)) : (int64_t)n_u + (int64_t)(kv[i - m] >> (bits_u + 1));
-  }
-  __device__ __forceinline__ uint32_t entry(int64_t i) const {
-    return i < m ? (uint32_t)(ku[i] & ((2ull << bits_v) - 1)) : (uint32_t)(kv[i - m] & ((2ull << bits_u) - 1));
+  __device__ __forceinline__ uint64_t operator()(uint64_t k) const {
+    const uint64_t ru = k >> (bits_v + 1), rv = (k >> 1) & ((1ull << bits_v) - 1);
+    return (rv << (bits_u + 1)) | (ru << 1) | (k & 1u);
   }
 };
 
-__global__ void csr_cols_kernel(CsrKeys ck, int64_t nnz, uint32_t* __restrict__ col) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nnz; i += (int64_t)gridDim.x * blockDim.x)
-    col[i] = ck.entry(i);
+// The first pass of the V sort reads the U-sorted list: V keys, each with its
+// U position (the edge's position in its U row) as the value.
+struct VKeyLoad {
+  const uint64_t* ku;
+  VKey vk;
+  __device__ __forceinline__ uint64_t key(uint32_t i) const { return vk(ku[i]); }
+  __device__ __forceinline__ uint32_t val(uint32_t i) const { return i; }
+};
+
+// Flags a repeated (u, v) pair (U-sorted keys that agree in everything but the
+// sign bit are adjacent) and counts the digits of the V sort.
+__global__ void __launch_bounds__(256) csr_v_digits_kernel(const uint64_t* __restrict__ ku, int64_t m, VKey vk,
+                                                           int passes, uint32_t* hist, unsigned* flags) {
+  __shared__ uint32_t h[kRsMaxPasses][256];
+  if (cta_stopped(flags)) return;
+  DigitCounts dc{h, passes, 1 + vk.bits_u};
+  dc.start();
+  bool dup = false;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+    const uint64_t k = ku[i];
+    if (i + 1 < m) dup |= (k >> 1) == (ku[i + 1] >> 1);
+    dc.add(vk(k));
+  }
+  if (__syncthreads_or(dup)) {
+    if (threadIdx.x == 0) atomicOr(flags, (unsigned)kPrepDup);
+    return;
+  }
+  dc.finish(hist);
 }
+
+// The distinct edges of a U-sorted list with repeated pairs: the last of every
+// run (the sorts are stable, so the latest input occurrence), compacted in one
+// pass over tiles of kRowTile edges. *count gets their number.
+__global__ void __launch_bounds__(kRowThreads) dedup_kernel(const uint64_t* __restrict__ ku, int64_t m, int bits_v,
+                                                            int32_t n_u, const int32_t* __restrict__ vertex,
+                                                            int32_t* __restrict__ eu, int32_t* __restrict__ ev,
+                                                            int8_t* __restrict__ es, uint64_t* count, uint64_t* state,
+                                                            unsigned* counter, unsigned* flags) {
+  __shared__ uint32_t tot_sh;
+  const int64_t tile = take_tile(counter, flags);
+  if (tile < 0) return;
+  const int64_t i0 = tile * kRowTile + (int64_t)threadIdx.x * kRowItems;
+  uint64_t k[kRowItems + 1];
+#pragma unroll
+  for (int j = 0; j <= kRowItems; j++) k[j] = i0 + j < m ? ku[i0 + j] : ~0ull;
+  bool keep[kRowItems];
+  uint32_t sum = 0;
+#pragma unroll
+  for (int j = 0; j < kRowItems; j++) {
+    keep[j] = i0 + j < m && (i0 + j == m - 1 || (k[j] >> 1) != (k[j + 1] >> 1));
+    sum += keep[j] ? 1u : 0u;
+  }
+  const uint32_t ex = block_excl_scan<uint32_t, kRowThreads>(sum, &tot_sh);
+  __syncthreads();
+  uint64_t prefix;
+  if (!tile_prefix(state, tile, tot_sh, flags, &prefix)) return;
+  uint64_t at = prefix + ex;
+#pragma unroll
+  for (int j = 0; j < kRowItems; j++) {
+    if (keep[j]) {
+      const uint64_t ru = k[j] >> (bits_v + 1), rv = (k[j] >> 1) & ((1ull << bits_v) - 1);
+      eu[at] = vertex[ru];
+      ev[at] = vertex[n_u + rv] - n_u;
+      es[at] = (k[j] & 1u) ? (int8_t)-1 : (int8_t)1;
+      at++;
+    }
+    if (i0 + j == m - 1) *count = at;
+  }
+}
+
+// V keys and U positions of the V rows: the edge at V position m + k.
+struct CsrKeys {
+  const uint64_t* kv;
+  const uint32_t* upos;
+  int64_t m;
+  int32_t n_u;
+  int bits_u;
+};
 
 // lower[r] = neighbours of row r with lower Def. 3 priority. A U vertex of
 // degree d is above a V vertex iff deg(v) < d (equal degree: the V id is
@@ -234,19 +312,36 @@ __global__ void csr_cols_kernel(CsrKeys ck, int64_t nnz, uint32_t* __restrict__ 
 // Neighbours lie in the row's own component, whose other-side ranks ascend by
 // degree, and rows list neighbours by ascending side rank, so the lower ones
 // are a prefix.
+// The last CTA instead finds, per side, how many vertices have degree below
+// each of four limits (ranks ascend by degree within a side): below[2k] for U,
+// below[2k + 1] for V.
+struct DegreeLimits {
+  int32_t d[4];
+};
 __global__ void lower_kernel(const int64_t* __restrict__ row_ptr, const uint32_t* __restrict__ col,
                              const int32_t* __restrict__ rowdeg, int64_t n, int32_t n_u, UnionView un,
-                             uint32_t* __restrict__ lower) {
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
+                             uint32_t* __restrict__ lower, DegreeLimits lim, int64_t* below, const unsigned* flags) {
+  if (cta_stopped(flags)) return;
+  if (blockIdx.x == gridDim.x - 1) {
+    const int t = threadIdx.x;
+    if (t < 8) {
+      const bool u = (t & 1) == 0;
+      below[t] = u ? lower_bound_dev<int32_t>(rowdeg, n_u, lim.d[t >> 1])
+                   : lower_bound_dev<int32_t>(rowdeg + n_u, n - n_u, lim.d[t >> 1]);
+    }
+    return;
+  }
+  const int64_t stride = (int64_t)(gridDim.x - 1) * blockDim.x;
+  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += stride) {
     const int32_t d = rowdeg[r];
     int64_t t;  // side rank threshold in the other side
     if (r < n_u) {
-      const int32_t c = component_of(un.uoff, un.n_graphs, r);
-      const int64_t b = un.voff[c], e = un.voff[c + 1];
+      const int32_t c = un.comp_u(r);
+      const int64_t b = un.vo(c), e = un.vo(c + 1);
       t = b + lower_bound_dev<int32_t>(rowdeg + n_u + b, e - b, d);
     } else {
-      const int32_t c = component_of(un.voff, un.n_graphs, r - n_u);
-      const int64_t b = un.uoff[c], e = un.uoff[c + 1];
+      const int32_t c = un.comp_v(r - n_u);
+      const int64_t b = un.uo(c), e = un.uo(c + 1);
       t = b + upper_bound_dev<int32_t>(rowdeg + b, e - b, d);
     }
     const int64_t b = row_ptr[r];
@@ -264,8 +359,9 @@ __global__ void lower_kernel(const int64_t* __restrict__ row_ptr, const uint32_t
 // in V order, 32 consecutive ones per warp: the V rows' sums are merged by a
 // segmented warp sum, the U rows' go to their rows directly.
 __global__ void work_kernel(CsrKeys ck, const int64_t* __restrict__ row_ptr, const uint32_t* __restrict__ lower,
-                            unsigned long long* __restrict__ work) {
+                            unsigned long long* __restrict__ work, const unsigned* flags) {
   constexpr int kRound = 4;  // edges per thread per round, their loads in flight together
+  if (cta_stopped(flags)) return;
   const int64_t m = ck.m;
   const uint64_t mask_u = (1ull << ck.bits_u) - 1;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -316,142 +412,140 @@ __global__ void work_kernel(CsrKeys ck, const int64_t* __restrict__ row_ptr, con
 }
 
 struct PrepStats {
-  unsigned long long wedges, wedges_hub, wedges_medium, wedges_light, max_work;
+  unsigned long long wedges, wedges_hub, wedges_medium, wedges_light;
   unsigned long long n_piv, n_hub, n_medium;
   unsigned long long lower_hub, lower_medium, lower_light;
+  unsigned long long max_work;
+};
+constexpr int kStatSums = 10;  // the sums of PrepStats, in order; max_work follows
+
+// What a build reads back from the device before it sizes the pivots.
+struct PrepResult {
+  PrepStats st;
+  int64_t below[8];         // vertices of degree below four limits (lower_kernel)
+  unsigned long long kept;  // distinct edges (dedup_kernel)
+  unsigned flags;           // kPrep*
 };
 
 // Pivots that can close a butterfly: at least two lower neighbours and at
 // least one accepted wedge. (A pivot with a single lower neighbour v reaches
-// every endpoint w at most once, so all its buckets stay below 2.)
-__global__ void pivot_flags_kernel(const uint64_t* __restrict__ work, const uint32_t* __restrict__ lower, int64_t n,
-                                   uint64_t light_max, uint64_t medium_max, uint32_t* __restrict__ flag,
-                                   PrepStats* st) {
-  uint64_t w_all = 0, w_hub = 0, w_med = 0, w_light = 0, mx = 0, np = 0, nh = 0, nm = 0;
-  uint64_t l_hub = 0, l_med = 0, l_light = 0;
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
-    const uint64_t w = work[r];
-    w_all += w;
-    const bool piv = lower[r] >= 2 && w > 0;
-    flag[r] = piv ? 1u : 0u;
-    if (piv) {
-      np++;
-      mx = w > mx ? w : mx;
-      const uint64_t L = lower[r];
-      if (w > medium_max) { nh++; w_hub += w; l_hub += L; }
-      else if (w > light_max) { nm++; w_med += w; l_med += L; }
-      else { w_light += w; l_light += L; }
+// every endpoint w at most once, so all its buckets stay below 2.) One pass
+// over tiles of kPivotTile rows adds up the statistics, compacts the pivots in
+// row order as sort keys ~work (ascending keys are descending work) with their
+// rows, and counts the digits of that sort.
+constexpr int kPivotItems = 8;
+constexpr int kPivotTile = kRowThreads * kPivotItems;
+
+__global__ void __launch_bounds__(kRowThreads) pivots_kernel(const uint64_t* __restrict__ work,
+                                                             const uint32_t* __restrict__ lower, int64_t n,
+                                                             uint64_t light_max, uint64_t medium_max,
+                                                             uint64_t* __restrict__ key, uint32_t* __restrict__ row,
+                                                             uint32_t* hist, PrepStats* st, uint64_t* state,
+                                                             unsigned* counter, unsigned* flags) {
+  __shared__ uint32_t h[kRsMaxPasses][256];
+  __shared__ uint64_t part[kRowThreads / 32][kStatSums + 1];
+  __shared__ uint32_t tot_sh;
+  const int64_t tile = take_tile(counter, flags);
+  if (tile < 0) return;
+  DigitCounts dc{h, kRsMaxPasses, 0};
+  dc.start();
+  const int64_t r0 = tile * kPivotTile + (int64_t)threadIdx.x * kPivotItems;
+  uint64_t w[kPivotItems];
+  uint64_t s[kStatSums] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+  uint64_t mx = 0;
+  uint32_t mine = 0;
+#pragma unroll
+  for (int j = 0; j < kPivotItems; j++) {
+    const int64_t r = r0 + j;
+    w[j] = r < n ? work[r] : 0;
+    const uint32_t L = r < n ? lower[r] : 0u;
+    s[0] += w[j];
+    if (L >= 2 && w[j] > 0) {
+      mine |= 1u << j;
+      s[4]++;
+      mx = w[j] > mx ? w[j] : mx;
+      const int tier = w[j] > medium_max ? 0 : w[j] > light_max ? 1 : 2;  // hub, medium, light
+      s[1] += tier == 0 ? w[j] : 0;
+      s[2] += tier == 1 ? w[j] : 0;
+      s[3] += tier == 2 ? w[j] : 0;
+      s[5] += tier == 0;
+      s[6] += tier == 1;
+      s[7] += tier == 0 ? L : 0;
+      s[8] += tier == 1 ? L : 0;
+      s[9] += tier == 2 ? L : 0;
     }
   }
-  w_all = warp_sum_u64(w_all);
-  w_hub = warp_sum_u64(w_hub);
-  w_med = warp_sum_u64(w_med);
-  w_light = warp_sum_u64(w_light);
-  np = warp_sum_u64(np);
-  nh = warp_sum_u64(nh);
-  nm = warp_sum_u64(nm);
-  l_hub = warp_sum_u64(l_hub);
-  l_med = warp_sum_u64(l_med);
-  l_light = warp_sum_u64(l_light);
+#pragma unroll
+  for (int k = 0; k < kStatSums; k++) {
+    const uint64_t t = warp_sum_u64(s[k]);
+    if (lane_id() == 0) part[threadIdx.x >> 5][k] = t;
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const uint64_t y = __shfl_xor_sync(kFullMask, mx, o);
     mx = y > mx ? y : mx;
   }
-  if (lane_id() == 0) {
-    if (w_all) atomicAdd(&st->wedges, (unsigned long long)w_all);
-    if (w_hub) atomicAdd(&st->wedges_hub, (unsigned long long)w_hub);
-    if (w_med) atomicAdd(&st->wedges_medium, (unsigned long long)w_med);
-    if (w_light) atomicAdd(&st->wedges_light, (unsigned long long)w_light);
-    if (mx) atomicMax(&st->max_work, (unsigned long long)mx);
-    if (np) atomicAdd(&st->n_piv, (unsigned long long)np);
-    if (nh) atomicAdd(&st->n_hub, (unsigned long long)nh);
-    if (nm) atomicAdd(&st->n_medium, (unsigned long long)nm);
-    if (l_hub) atomicAdd(&st->lower_hub, (unsigned long long)l_hub);
-    if (l_med) atomicAdd(&st->lower_medium, (unsigned long long)l_med);
-    if (l_light) atomicAdd(&st->lower_light, (unsigned long long)l_light);
+  if (lane_id() == 0) part[threadIdx.x >> 5][kStatSums] = mx;
+  const uint32_t ex = block_excl_scan<uint32_t, kRowThreads>(__popc(mine), &tot_sh);
+  __syncthreads();
+  if (threadIdx.x <= kStatSums) {
+    unsigned long long* out = reinterpret_cast<unsigned long long*>(st) + threadIdx.x;
+    uint64_t t = 0;
+    for (int k = 0; k < kRowThreads / 32; k++) {
+      const uint64_t x = part[k][threadIdx.x];
+      t = threadIdx.x < kStatSums ? t + x : x > t ? x : t;
+    }
+    if (t && threadIdx.x < kStatSums) atomicAdd(out, (unsigned long long)t);
+    if (t && threadIdx.x == kStatSums) atomicMax(out, (unsigned long long)t);
   }
-}
-
-// Descending-work sort key for pivot rows: (2^bits - 1 - work) ascending.
-__global__ void pivot_keys_kernel(const uint64_t* __restrict__ work, const uint32_t* __restrict__ flag,
-                                  const uint32_t* __restrict__ pos, int64_t n, int bits, uint64_t* __restrict__ key,
-                                  uint32_t* __restrict__ row) {
-  const uint64_t top = bits >= 64 ? ~0ull : ((1ull << bits) - 1);
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
-    if (!flag[r]) continue;
-    const uint32_t j = pos[r];
-    key[j] = top - work[r];
-    row[j] = (uint32_t)r;
-  }
-}
-
-// Per side, how many vertices have degree below each of four limits (ranks
-// ascend by degree within a side): out[2k] for U, out[2k + 1] for V.
-struct DegreeLimits {
-  int32_t d[4];
-};
-__global__ void narrow_ranks_kernel(const int32_t* __restrict__ rowdeg, int64_t n, int32_t n_u, DegreeLimits lim,
-                                    int64_t* out) {
-  const int t = threadIdx.x;
-  if (t < 8) {
-    const bool u = (t & 1) == 0;
-    out[t] = u ? lower_bound_dev<int32_t>(rowdeg, n_u, lim.d[t >> 1])
-               : lower_bound_dev<int32_t>(rowdeg + n_u, n - n_u, lim.d[t >> 1]);
-  }
-}
-
-// Union of several graphs: graph i's local ids are validated against its own
-// sides and shifted by the sizes of the graphs before it.
-__global__ void union_ids_kernel(const int32_t* __restrict__ u, const int32_t* __restrict__ v,
-                                 const int8_t* __restrict__ s, const int64_t* __restrict__ eoff,
-                                 const int32_t* __restrict__ nu, const int32_t* __restrict__ nv,
-                                 const int64_t* __restrict__ uoff, const int64_t* __restrict__ voff, int32_t n_graphs,
-                                 int32_t* __restrict__ ou, int32_t* __restrict__ ov, int8_t* __restrict__ os,
-                                 unsigned* err) {
-  unsigned e = 0;
-  for (int32_t gi = blockIdx.x; gi < n_graphs; gi += gridDim.x) {
-    const int64_t e0 = eoff[gi], e1 = eoff[gi + 1];
-    const int32_t a = nu[gi], b = nv[gi];
-    const int32_t du = (int32_t)uoff[gi], dv = (int32_t)voff[gi];
-    for (int64_t i = e0 + threadIdx.x; i < e1; i += blockDim.x) {
-      const int32_t x = u[i], y = v[i];
-      const int8_t c = s[i];
-      if (x < 0 || x >= a) e |= 1u;
-      if (y < 0 || y >= b) e |= 2u;
-      if (c != 1 && c != -1) e |= 4u;
-      ou[i] = x + du;
-      ov[i] = y + dv;
-      os[i] = c;
+  uint64_t prefix;
+  if (!tile_prefix(state, tile, tot_sh, flags, &prefix)) return;
+  uint64_t at = prefix + ex;
+#pragma unroll
+  for (int j = 0; j < kPivotItems; j++) {
+    if (mine >> j & 1u) {
+      key[at] = ~w[j];
+      row[at] = (uint32_t)(r0 + j);
+      dc.add(~w[j]);
+      at++;
     }
   }
-  e = __reduce_or_sync(kFullMask, e);
-  if (lane_id() == 0 && e) atomicOr(err, e);
+  dc.finish(hist);
 }
 
-// Component of every row of a union: the graph whose id range holds the
-// row's vertex.
-__global__ void component_kernel(const int32_t* __restrict__ vertex, int64_t n, int32_t n_u_total,
+// Union of several graphs: graph i's local ids are shifted by the sizes of the
+// graphs before it; an id out of its own graph's range becomes -1, which the
+// build's validation finds. Threads take edges grid-wide (one search for the
+// warp's first edge, then a walk over the components its lanes span), so a
+// large graph is not left to one CTA: 200 graphs of 6.3M edges in all took
+// 414 us with a CTA per graph.
+__global__ void union_ids_kernel(const int32_t* __restrict__ u, const int32_t* __restrict__ v,
+                                 const int8_t* __restrict__ s, const int64_t* __restrict__ eoff,
                                  const int64_t* __restrict__ uoff, const int64_t* __restrict__ voff, int32_t n_graphs,
-                                 int32_t* __restrict__ comp) {
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < n; r += (int64_t)gridDim.x * blockDim.x) {
-    const int32_t x = vertex[r];
-    const bool is_u = x < n_u_total;
-    const int64_t key = is_u ? x : (int64_t)x - n_u_total;
-    const int64_t* off = is_u ? uoff : voff;
-    comp[r] = (int32_t)upper_bound_dev<int64_t>(off, (int64_t)n_graphs + 1, key) - 1;
+                                 int64_t m, int32_t* __restrict__ ou, int32_t* __restrict__ ov,
+                                 int8_t* __restrict__ os) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+    int32_t c = component_of(eoff, n_graphs, i - (int64_t)lane_id());
+    while (i >= eoff[c + 1]) c++;
+    const int64_t u0 = uoff[c], v0 = voff[c];
+    const int32_t x = u[i], y = v[i];
+    ou[i] = x >= 0 && x < uoff[c + 1] - u0 ? (int32_t)(u0 + x) : -1;
+    ov[i] = y >= 0 && y < voff[c + 1] - v0 ? (int32_t)(v0 + y) : -1;
+    os[i] = s[i];
   }
 }
 
-__global__ void gather_u32_kernel(const uint32_t* __restrict__ src, const uint32_t* __restrict__ idx, int64_t n,
-                                  uint32_t* __restrict__ dst) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    dst[i] = src[idx[i]];
-}
-__global__ void gather_u64_kernel(const uint64_t* __restrict__ src, const uint32_t* __restrict__ idx, int64_t n,
-                                  uint64_t* __restrict__ dst) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    dst[i] = src[idx[i]];
+// What the hub plan needs of every hub, in pivot order.
+struct HubInfo {
+  uint32_t row, lower;
+  uint64_t work;
+};
+__global__ void hub_info_kernel(const int32_t* __restrict__ order, const uint32_t* __restrict__ lower,
+                                const uint64_t* __restrict__ work, int64_t n_hub, HubInfo* __restrict__ out) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_hub; i += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t r = (uint32_t)order[i];
+    out[i] = HubInfo{r, lower[r], work[r]};
+  }
 }
 
 // ------------------------------------------------------------------ host
@@ -461,12 +555,23 @@ static unsigned grid_for(int64_t n, int threads = 256) {
   return (unsigned)(b < cap ? b : cap);
 }
 
+// For kernels that count digits: one resident wave, so that few CTAs add to
+// the global counts.
+static unsigned count_grid(int64_t n) { return std::min(grid_for(n), (unsigned)kNumSMs * 8u); }
+
 void* graph_alloc(dbbc_graph* g, size_t bytes) {
   void* p = dev_alloc(bytes ? bytes : 16, g->stream);
   if (!p) throw Error{DBBC_ENOMEM, "graph_alloc"};
   g->allocations.push_back(p);
   g->device_bytes += bytes;
   return p;
+}
+
+// Give one of the graph's allocations back.
+static void graph_release(dbbc_graph* g, void* p, size_t bytes) {
+  g->allocations.erase(std::find(g->allocations.begin(), g->allocations.end(), p));
+  g->device_bytes -= bytes;
+  dev_free(p, g->stream);
 }
 
 void free_graph_memory(dbbc_graph* g) {
@@ -483,22 +588,35 @@ static T read_back(const T* d, cudaStream_t s) {
   return h;
 }
 
+// Carves a build's device scratch out of one allocation: run once without a
+// base to size it, then again to place it.
+struct Carver {
+  char* base = nullptr;
+  size_t used = 0;
+  template <typename T>
+  T* get(size_t n) {
+    T* p = reinterpret_cast<T*>(base + used);
+    used += (n * sizeof(T) + 255) / 256 * 256;
+    return p;
+  }
+  RadixState radix(int passes, int64_t n) {
+    RadixState r;
+    r.hist = get<uint32_t>((size_t)passes * 256);
+    r.counters = get<unsigned>((size_t)passes);
+    r.state = get<uint32_t>((size_t)passes * (size_t)radix_tiles(n) * 256);
+    return r;
+  }
+};
+
 static void plan_hubs(dbbc_graph* g, cudaStream_t s, const UnionSpec& un) {
   if (g->n_hub == 0) return;
-  std::vector<uint32_t> rows((size_t)g->n_hub), lows((size_t)g->n_hub);
-  std::vector<uint64_t> works((size_t)g->n_hub);
+  std::vector<HubInfo> hubs((size_t)g->n_hub);
   {
     Scratch sc(s);
-    uint32_t* d_low = sc.get<uint32_t>((size_t)g->n_hub);
-    uint64_t* d_work = sc.get<uint64_t>((size_t)g->n_hub);
-    const uint32_t* d_rows = reinterpret_cast<const uint32_t*>(g->order);
-    gather_u32_kernel<<<grid_for(g->n_hub), 256, 0, s>>>(g->lower, d_rows, g->n_hub, d_low);
+    HubInfo* d = sc.get<HubInfo>(hubs.size());
+    hub_info_kernel<<<grid_for(g->n_hub), 256, 0, s>>>(g->order, g->lower, g->work, g->n_hub, d);
     DBBC_LAUNCH_CHECK();
-    gather_u64_kernel<<<grid_for(g->n_hub), 256, 0, s>>>(g->work, d_rows, g->n_hub, d_work);
-    DBBC_LAUNCH_CHECK();
-    DBBC_CUDA(cudaMemcpyAsync(rows.data(), d_rows, rows.size() * 4, cudaMemcpyDeviceToHost, s));
-    DBBC_CUDA(cudaMemcpyAsync(lows.data(), d_low, lows.size() * 4, cudaMemcpyDeviceToHost, s));
-    DBBC_CUDA(cudaMemcpyAsync(works.data(), d_work, works.size() * 8, cudaMemcpyDeviceToHost, s));
+    DBBC_CUDA(cudaMemcpyAsync(hubs.data(), d, hubs.size() * sizeof(HubInfo), cudaMemcpyDeviceToHost, s));
     DBBC_CUDA(cudaStreamSynchronize(s));
   }
   // Split each hub's accepted ranks [0, sp) into items of roughly equal work.
@@ -513,10 +631,10 @@ static void plan_hubs(dbbc_graph* g, cudaStream_t s, const UnionSpec& un) {
   };
   std::vector<Planned> plan;
   int64_t max_lower = 1;
-  for (size_t h = 0; h < rows.size(); h++) {
-    const int32_t row = (int32_t)rows[h];
-    const uint32_t L = lows[h];
-    const uint64_t W = works[h];
+  for (const HubInfo& hub : hubs) {
+    const int32_t row = (int32_t)hub.row;
+    const uint32_t L = hub.lower;
+    const uint64_t W = hub.work;
     const bool is_u = row < g->n_u;
     const uint64_t sp = is_u ? (uint64_t)row : (uint64_t)(row - g->n_u);
     // the hub's accepted endpoints are the ranks of its own component below it
@@ -613,13 +731,12 @@ static void plan_hubs(dbbc_graph* g, cudaStream_t s, const UnionSpec& un) {
     items[i] = plan[i].it;
     g->sweep_est_host[i] = plan[i].est;
   }
-  g->sweep_items_host = items;
-  g->n_sweep_items = (int64_t)items.size();
+  g->sweep_items_host = std::move(items);
+  const std::vector<SweepItem>& kept = g->sweep_items_host;
+  g->n_sweep_items = (int64_t)kept.size();
   g->sweep_max_lower = max_lower;
-  g->sweep_items = static_cast<SweepItem*>(graph_alloc(g, items.size() * sizeof(SweepItem)));
-  DBBC_CUDA(cudaMemcpyAsync(g->sweep_items, items.data(), items.size() * sizeof(SweepItem), cudaMemcpyHostToDevice,
-                            s));
-  DBBC_CUDA(cudaStreamSynchronize(s));
+  g->sweep_items = static_cast<SweepItem*>(graph_alloc(g, kept.size() * sizeof(SweepItem)));
+  DBBC_CUDA(cudaMemcpyAsync(g->sweep_items, kept.data(), kept.size() * sizeof(SweepItem), cudaMemcpyHostToDevice, s));
 }
 
 void build_graph_multi(dbbc_graph* g, const int32_t* u, const int32_t* v, const int8_t* sgn,
@@ -653,49 +770,32 @@ void build_graph_multi(dbbc_graph* g, const int32_t* u, const int32_t* v, const 
     dv = tv;
     ds = ts;
   }
-  int64_t* d_meta = sc.get<int64_t>((size_t)3 * (n_graphs + 1));
-  int32_t* d_n = sc.get<int32_t>((size_t)2 * n_graphs + 2);
-  std::vector<int32_t> nn((size_t)2 * n_graphs + 2, 0);
-  std::copy(n_u, n_u + n_graphs, nn.begin());
-  std::copy(n_v, n_v + n_graphs, nn.begin() + n_graphs);
-  DBBC_CUDA(cudaMemcpyAsync(d_meta, edge_offsets, (size_t)(n_graphs + 1) * 8, cudaMemcpyHostToDevice, s));
-  DBBC_CUDA(cudaMemcpyAsync(d_meta + n_graphs + 1, uoff.data(), uoff.size() * 8, cudaMemcpyHostToDevice, s));
-  DBBC_CUDA(cudaMemcpyAsync(d_meta + 2 * (n_graphs + 1), voff.data(), voff.size() * 8, cudaMemcpyHostToDevice, s));
-  DBBC_CUDA(cudaMemcpyAsync(d_n, nn.data(), nn.size() * 4, cudaMemcpyHostToDevice, s));
+  // edge, U and V offsets in one upload
+  const size_t k = (size_t)n_graphs + 1;
+  std::vector<int64_t> meta(3 * k);
+  std::copy(edge_offsets, edge_offsets + k, meta.begin());
+  std::copy(uoff.begin(), uoff.end(), meta.begin() + (ptrdiff_t)k);
+  std::copy(voff.begin(), voff.end(), meta.begin() + (ptrdiff_t)(2 * k));
+  int64_t* d_meta = sc.get<int64_t>(meta.size());
+  DBBC_CUDA(cudaMemcpyAsync(d_meta, meta.data(), meta.size() * 8, cudaMemcpyHostToDevice, s));
   int32_t* ou = sc.get<int32_t>((size_t)std::max<int64_t>(m, 1));
   int32_t* ov = sc.get<int32_t>((size_t)std::max<int64_t>(m, 1));
   int8_t* os = sc.get<int8_t>((size_t)std::max<int64_t>(m, 1));
-  unsigned* d_err = sc.get<unsigned>(1);
-  DBBC_CUDA(cudaMemsetAsync(d_err, 0, sizeof(unsigned), s));
-  if (n_graphs > 0 && m > 0) {
-    union_ids_kernel<<<(unsigned)std::min<int32_t>(n_graphs, 65535), 256, 0, s>>>(
-        du, dv, ds, d_meta, d_n, d_n + n_graphs, d_meta + n_graphs + 1, d_meta + 2 * (n_graphs + 1), n_graphs, ou, ov,
-        os, d_err);
+  if (m > 0) {
+    union_ids_kernel<<<grid_for(m), 256, 0, s>>>(du, dv, ds, d_meta, d_meta + k, d_meta + 2 * k, n_graphs, m, ou, ov,
+                                                 os);
     DBBC_LAUNCH_CHECK();
-    if (read_back(d_err, s) != 0) throw Error{DBBC_EINVAL, "invalid edge id or sign"};
   }
   UnionSpec un;
   un.n_graphs = std::max<int32_t>(n_graphs, 1);
   un.uoff = n_graphs > 0 ? uoff : std::vector<int64_t>{0, 0};
   un.voff = n_graphs > 0 ? voff : std::vector<int64_t>{0, 0};
-  un.d_uoff = n_graphs > 0 ? d_meta + n_graphs + 1 : nullptr;
-  un.d_voff = n_graphs > 0 ? d_meta + 2 * (n_graphs + 1) : nullptr;
+  un.d_uoff = d_meta + k;
+  un.d_voff = d_meta + 2 * k;
   for (int32_t i = 0; i < n_graphs; i++) un.max_side = std::max<int64_t>(un.max_side, std::max(n_u[i], n_v[i]));
-  if (n_graphs == 0) {
-    int64_t* d = sc.get<int64_t>(4);
-    DBBC_CUDA(cudaMemsetAsync(d, 0, 32, s));
-    un.d_uoff = d;
-    un.d_voff = d + 2;
-  }
-  build_graph(g, ou, ov, os, m, true, reject_duplicates, s, &un);
   g->n_components = n_graphs;
-  g->component = static_cast<int32_t*>(graph_alloc(g, (size_t)std::max<int64_t>(g->n, 1) * 4));
-  if (g->n > 0) {
-    component_kernel<<<grid_for(g->n), 256, 0, s>>>(g->vertex, g->n, g->n_u, d_meta + n_graphs + 1,
-                                                    d_meta + 2 * (n_graphs + 1), n_graphs, g->component);
-    DBBC_LAUNCH_CHECK();
-  }
-  DBBC_CUDA(cudaStreamSynchronize(s));
+  g->component = static_cast<int32_t*>(graph_alloc(g, (size_t)std::max<int64_t>((int64_t)g->n_u + g->n_v, 1) * 4));
+  build_graph(g, ou, ov, os, m, true, reject_duplicates, s, &un);
 }
 
 void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const int8_t* s_in, int64_t m,
@@ -705,7 +805,6 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
   g->n = n;
   g->m_input = m;
   g->tune = current_tuning();
-  Scratch sc(s);
   // a plain graph is a union of one component
   UnionSpec plain;
   const UnionSpec* un = union_spec;
@@ -713,39 +812,9 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
     plain.uoff = {0, (int64_t)n_u};
     plain.voff = {0, (int64_t)n_v};
     plain.max_side = std::max<int64_t>(n_u, n_v);
-    int64_t* d = sc.get<int64_t>(4);
-    DBBC_CUDA(cudaMemcpyAsync(d, plain.uoff.data(), 16, cudaMemcpyHostToDevice, s));
-    DBBC_CUDA(cudaMemcpyAsync(d + 2, plain.voff.data(), 16, cudaMemcpyHostToDevice, s));
-    plain.d_uoff = d;
-    plain.d_voff = d + 2;
     un = &plain;
   }
-  const UnionView uv{un->d_uoff, un->d_voff, un->n_graphs};
-
-  // ---- inputs on the device
-  const int32_t* du = u_in;
-  const int32_t* dv = v_in;
-  const int8_t* ds = s_in;
-  if (!on_device && m > 0) {
-    int32_t* tu = sc.get<int32_t>((size_t)m);
-    int32_t* tv = sc.get<int32_t>((size_t)m);
-    int8_t* ts = sc.get<int8_t>((size_t)m);
-    DBBC_CUDA(cudaMemcpyAsync(tu, u_in, (size_t)m * 4, cudaMemcpyHostToDevice, s));
-    DBBC_CUDA(cudaMemcpyAsync(tv, v_in, (size_t)m * 4, cudaMemcpyHostToDevice, s));
-    DBBC_CUDA(cudaMemcpyAsync(ts, s_in, (size_t)m, cudaMemcpyHostToDevice, s));
-    du = tu;
-    dv = tv;
-    ds = ts;
-  }
-  unsigned* d_flags = sc.get<unsigned>(4);
-  DBBC_CUDA(cudaMemsetAsync(d_flags, 0, 4 * sizeof(unsigned), s));
-
-  // ---- a1: validate
-  if (m > 0) {
-    validate_kernel<<<grid_for(m), 256, 0, s>>>(du, dv, ds, m, n_u, n_v, d_flags);
-    DBBC_LAUNCH_CHECK();
-    if (read_back(d_flags, s) != 0) throw Error{DBBC_EINVAL, "invalid edge id or sign"};
-  }
+  const UnionView uv{un->d_uoff, un->d_voff, un->n_graphs, n_u, n_v};
 
   const int bits_u = bits_for(n_u > 0 ? (uint64_t)(n_u - 1) : 0);
   const int bits_v = bits_for(n_v > 0 ? (uint64_t)(n_v - 1) : 0);
@@ -754,125 +823,193 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
   const int bits_lid = std::max(1, bits_for(un->max_side > 0 ? (uint64_t)(un->max_side - 1) : 0));
   const int bits_deg = std::max(1, bits_for((uint64_t)un->max_side));
   if (1 + bits_comp + bits_deg + bits_lid > 64) throw Error{DBBC_EINVAL, "union too large for 64-bit rank keys"};
-  int32_t* deg = sc.get<int32_t>((size_t)n);
-  int32_t* side_rank = sc.get<int32_t>((size_t)n);
-  int32_t* rowdeg = sc.get<int32_t>((size_t)n);
-  uint64_t* vk0 = sc.get<uint64_t>((size_t)n);
-  uint64_t* vk1 = sc.get<uint64_t>((size_t)n);
-  uint64_t* ck0 = sc.get<uint64_t>((size_t)(2 * m));
-  uint64_t* ck1 = sc.get<uint64_t>((size_t)(2 * m));
+  // keys are generated in (side, component, local id) order, so a stable sort
+  // on (side, component, degree) alone leaves equal degrees by id; the edge
+  // sorts skip bit 0 (the sign), so repeated pairs stay in input order
+  const int rank_end = 1 + bits_comp + bits_deg + bits_lid;
+  const int passes_r = radix_passes(bits_lid, rank_end);
+  const int passes_u = radix_passes(1, 1 + bits_v + bits_u);
+  const int passes_v = radix_passes(1 + bits_u, 1 + bits_u + bits_v);
+
+  // ---- scratch, one allocation: what has to start at zero comes first
+  struct Layout {
+    PrepResult* res;
+    RadixState rank, su, sv, piv;
+    uint64_t *row_state, *pivot_state, *dedup_state;
+    unsigned* counters;  // tiles of the row, pivot and dedup kernels
+    int32_t* deg;
+    size_t zeroed;
+    int32_t *side_rank, *rowdeg;
+    uint64_t *vk0, *vk1, *ck0, *ck1;  // vertex / pivot keys, edge keys
+    uint32_t *up0, *up1, *pr0, *pr1;  // U positions, pivot rows
+    int32_t *tu, *tv;                 // host inputs; distinct edges
+    int8_t* ts;
+  };
+  auto place = [&](Carver& c) {
+    Layout l;
+    const size_t mm = (size_t)m, nn = (size_t)n;
+    l.res = c.get<PrepResult>(1);
+    l.rank = c.radix(passes_r, n);
+    l.su = c.radix(passes_u, m);
+    l.sv = c.radix(passes_v, m);
+    l.piv = c.radix(kRsMaxPasses, n);
+    l.row_state = c.get<uint64_t>((size_t)ceil_div<int64_t>(n, kRowTile) + 1);
+    l.pivot_state = c.get<uint64_t>((size_t)ceil_div<int64_t>(n, kPivotTile) + 1);
+    l.dedup_state = c.get<uint64_t>((size_t)ceil_div<int64_t>(m, kRowTile) + 1);
+    l.counters = c.get<unsigned>(3);
+    l.deg = c.get<int32_t>(nn);
+    l.zeroed = c.used;
+    l.side_rank = c.get<int32_t>(nn);
+    l.rowdeg = c.get<int32_t>(nn);
+    l.vk0 = c.get<uint64_t>(nn);
+    l.vk1 = c.get<uint64_t>(nn);
+    l.ck0 = c.get<uint64_t>(mm);
+    l.ck1 = c.get<uint64_t>(mm);
+    l.up0 = c.get<uint32_t>(mm);
+    l.up1 = c.get<uint32_t>(mm);
+    l.pr0 = c.get<uint32_t>(nn);
+    l.pr1 = c.get<uint32_t>(nn);
+    l.tu = l.tv = nullptr;
+    l.ts = nullptr;
+    if (!on_device) {
+      l.tu = c.get<int32_t>(mm);
+      l.tv = c.get<int32_t>(mm);
+      l.ts = c.get<int8_t>(mm);
+    }
+    return l;
+  };
+  Scratch sc(s);
+  Carver carver;
+  place(carver);
+  carver.base = sc.get<char>(carver.used);
+  carver.used = 0;
+  const Layout l = place(carver);
+  unsigned* d_flags = &l.res->flags;
+
+  // ---- inputs on the device
+  const int32_t* du = u_in;
+  const int32_t* dv = v_in;
+  const int8_t* ds = s_in;
+  if (!on_device && m > 0) {
+    DBBC_CUDA(cudaMemcpyAsync(l.tu, u_in, (size_t)m * 4, cudaMemcpyHostToDevice, s));
+    DBBC_CUDA(cudaMemcpyAsync(l.tv, v_in, (size_t)m * 4, cudaMemcpyHostToDevice, s));
+    DBBC_CUDA(cudaMemcpyAsync(l.ts, s_in, (size_t)m, cudaMemcpyHostToDevice, s));
+    du = l.tu;
+    dv = l.tv;
+    ds = l.ts;
+  }
   g->vertex = static_cast<int32_t*>(graph_alloc(g, (size_t)n * 4));
   g->row_ptr = static_cast<int64_t*>(graph_alloc(g, (size_t)(n + 1) * 8));
+  g->lower = static_cast<uint32_t*>(graph_alloc(g, (size_t)n * 4));
+  g->work = static_cast<uint64_t*>(graph_alloc(g, (size_t)n * 8));
+  if (n == 0) DBBC_CUDA(cudaMemsetAsync(g->row_ptr, 0, 8, s));
 
-  // a2 + a3 for an edge list: degrees, Def. 3 ranks per side, and the CSR
-  // keys of both sides (CsrKeys: U rows sorted by (U rank, V rank), V rows
-  // by (V rank, U rank)) with the sign in bit 0. Returns the keys and whether
-  // any (u, v) pair occurs twice (adjacent U keys).
-  auto csr_from_edges = [&](const int32_t* eu, const int32_t* ev, const int8_t* es, int64_t me,
-                            bool* dup) -> CsrKeys {
-    DBBC_CUDA(cudaMemsetAsync(deg, 0, (size_t)n * 4, s));
+  // a1-a4 for an edge list, without a wait: validation and degrees, Def. 3
+  // ranks per side, the CSR of both sides, accepted wedges per pivot and the
+  // pivots. When an edge is invalid, a (u, v) pair occurs twice or a wait gave
+  // up, the kernels that follow return at once and the flags say why. *ku_out
+  // gets the U-sorted keys.
+  const uint64_t* ku = nullptr;
+  auto build_from_edges = [&](const int32_t* eu, const int32_t* ev, const int8_t* es, int64_t me) -> PrepResult {
+    DBBC_CUDA(cudaMemsetAsync(l.res, 0, l.zeroed, s));
+    g->col = static_cast<uint32_t*>(graph_alloc(g, (size_t)(2 * me) * 4));
     if (me > 0) {
-      degree_kernel<<<grid_for(me), 256, 0, s>>>(eu, ev, me, n_u, deg);
+      degree_kernel<<<grid_for(me), 256, 0, s>>>(eu, ev, es, me, n_u, n_v, l.deg, d_flags);
       DBBC_LAUNCH_CHECK();
     }
     if (n > 0) {
-      vertex_keys_kernel<<<grid_for(n), 256, 0, s>>>(deg, n, n_u, bits_comp, bits_deg, bits_lid, uv, vk0);
+      vertex_keys_kernel<<<count_grid(n), 256, 0, s>>>(l.deg, n, n_u, bits_comp, bits_deg, bits_lid, uv, l.vk0, passes_r,
+                                                     l.rank.hist, d_flags);
       DBBC_LAUNCH_CHECK();
-      // keys are generated in (side, component, local id) order, so a stable
-      // sort on (side, component, degree) alone leaves equal degrees by id
-      const bool alt = radix_sort<uint64_t, uint32_t, false>(vk0, vk1, nullptr, nullptr, n, bits_lid,
-                                                             1 + bits_comp + bits_deg + bits_lid, s, sc);
-      ranks_kernel<<<grid_for(n), 256, 0, s>>>(alt ? vk1 : vk0, n, n_u, bits_comp, bits_deg, bits_lid, uv,
-                                               g->vertex, side_rank, rowdeg);
+      uint64_t *in = l.vk0, *out = l.vk1;
+      for (int p = 0; p < passes_r; p++, std::swap(in, out))
+        radix_pass<PlainLoad, false, true, false>(PlainLoad{in, nullptr}, PassOut{out, nullptr, nullptr, 0}, n,
+                                                  bits_lid, p, l.rank, d_flags, s);
+      ranks_kernel<<<(unsigned)ceil_div<int64_t>(n, kRowTile), kRowThreads, 0, s>>>(
+          in, n, n_u, bits_comp, bits_deg, bits_lid, uv, g->vertex, l.side_rank, l.rowdeg, g->row_ptr, g->component,
+          g->work, l.row_state, l.counters, d_flags);
       DBBC_LAUNCH_CHECK();
     }
-    *dup = false;
-    CsrKeys k{ck0, ck0 + me, nullptr, me, n_u, bits_u, bits_v};
-    if (me == 0) return k;
-    // the halves of ck0 / ck1 hold the U keys and the V keys; the sorts skip
-    // bit 0 (the sign), so repeated pairs stay in input order
-    csr_u_keys_kernel<<<grid_for(me), 256, 0, s>>>(eu, ev, es, me, n_u, side_rank, bits_v, ck0);
-    DBBC_LAUNCH_CHECK();
-    const bool alt_u = radix_sort<uint64_t, uint32_t, false>(ck0, ck1, nullptr, nullptr, me, 1, 1 + bits_v + bits_u,
-                                                             s, sc);
-    k.ku = alt_u ? ck1 : ck0;
-    DBBC_CUDA(cudaMemsetAsync(d_flags + 3, 0, sizeof(unsigned), s));
-    adjacent_dup_kernel<<<grid_for(me), 256, 0, s>>>(k.ku, me, d_flags + 3);
-    DBBC_LAUNCH_CHECK();
-    uint32_t* up0 = sc.get<uint32_t>((size_t)me);
-    uint32_t* up1 = sc.get<uint32_t>((size_t)me);
-    csr_v_keys_kernel<<<grid_for(me), 256, 0, s>>>(k.ku, me, bits_u, bits_v, ck0 + me, up0);
-    DBBC_LAUNCH_CHECK();
-    const bool alt_v = radix_sort<uint64_t, uint32_t, true>(ck0 + me, ck1 + me, up0, up1, me, 1 + bits_u,
-                                                            1 + bits_u + bits_v, s, sc);
-    k.kv = alt_v ? ck1 + me : ck0 + me;
-    k.upos = alt_v ? up1 : up0;
-    *dup = read_back(d_flags + 3, s) != 0;
-    return k;
+    CsrKeys ck{nullptr, nullptr, me, n_u, bits_u};
+    if (me > 0) {
+      csr_u_keys_kernel<<<count_grid(me), 256, 0, s>>>(eu, ev, es, me, n_u, l.side_rank, bits_v, l.ck0, passes_u,
+                                                     l.su.hist, d_flags);
+      DBBC_LAUNCH_CHECK();
+      uint64_t *in = l.ck0, *out = l.ck1;
+      for (int p = 0; p < passes_u; p++, std::swap(in, out)) {
+        const PassOut po{out, nullptr, g->col, (2ull << bits_v) - 1};
+        if (p + 1 < passes_u)
+          radix_pass<PlainLoad, false, true, false>(PlainLoad{in, nullptr}, po, me, 1, p, l.su, d_flags, s);
+        else
+          radix_pass<PlainLoad, false, true, true>(PlainLoad{in, nullptr}, po, me, 1, p, l.su, d_flags, s);
+      }
+      ku = in;
+      const VKey vk{bits_u, bits_v};
+      csr_v_digits_kernel<<<count_grid(me), 256, 0, s>>>(ku, me, vk, passes_v, l.sv.hist, d_flags);
+      DBBC_LAUNCH_CHECK();
+      uint32_t *vin = l.up0, *vout = l.up1;
+      for (int p = 0; p < passes_v; p++, std::swap(in, out), std::swap(vin, vout)) {
+        const PassOut po{out, vout, g->col + me, (2ull << bits_u) - 1};
+        const bool last = p + 1 == passes_v;
+        const VKeyLoad first{ku, vk};
+        const PlainLoad next{in, vin};
+        if (p == 0 && last) radix_pass<VKeyLoad, true, true, true>(first, po, me, 1 + bits_u, p, l.sv, d_flags, s);
+        else if (p == 0) radix_pass<VKeyLoad, true, true, false>(first, po, me, 1 + bits_u, p, l.sv, d_flags, s);
+        else if (last) radix_pass<PlainLoad, true, true, true>(next, po, me, 1 + bits_u, p, l.sv, d_flags, s);
+        else radix_pass<PlainLoad, true, true, false>(next, po, me, 1 + bits_u, p, l.sv, d_flags, s);
+      }
+      ck.kv = in;
+      ck.upos = vin;
+    }
+    if (n > 0) {
+      const DegreeLimits lim{{kNarrowCountLimit, kTinyCountLimit, kQuarterCountLimit, 1}};
+      lower_kernel<<<grid_for(n) + 1, 256, 0, s>>>(g->row_ptr, g->col, l.rowdeg, n, n_u, uv, g->lower, lim,
+                                                   l.res->below, d_flags);
+      DBBC_LAUNCH_CHECK();
+      if (me > 0) {
+        work_kernel<<<grid_for(me), 256, 0, s>>>(ck, g->row_ptr, g->lower,
+                                                 reinterpret_cast<unsigned long long*>(g->work), d_flags);
+        DBBC_LAUNCH_CHECK();
+      }
+      pivots_kernel<<<(unsigned)ceil_div<int64_t>(n, kPivotTile), kRowThreads, 0, s>>>(
+          g->work, g->lower, n, g->tune.light_max_work, g->tune.medium_max_work, l.vk0, l.pr0, l.piv.hist,
+          &l.res->st, l.pivot_state, l.counters + 1, d_flags);
+      DBBC_LAUNCH_CHECK();
+    }
+    const PrepResult r = read_back(l.res, s);
+    if (r.flags & kPrepInvalid) throw Error{DBBC_EINVAL, "invalid edge id or sign"};
+    if (r.flags & kPrepTimeout) throw Error{DBBC_ETIMEOUT, "a bounded wait of the build gave up"};
+    return r;
   };
 
-  // ---- a1-a3: build straight from the input; only when some (u, v) pair
-  // repeats, drop all but its latest occurrence (stable sort on (u, v), keep
-  // the last of every run) and build again from the distinct edges.
-  bool dup = false;
+  // ---- build straight from the input; only when some (u, v) pair repeats,
+  // keep the latest occurrence of every pair (the last of its run in the
+  // U-sorted list) and build again from the distinct edges.
   int64_t mu = m;
-  CsrKeys ck = csr_from_edges(du, dv, ds, m, &dup);
-  if (dup) {
+  PrepResult r = build_from_edges(du, dv, ds, m);
+  if (r.flags & kPrepDup) {
     if (reject_duplicates) throw Error{DBBC_EINVAL, "duplicate edge under DBBC_DUP_REJECT"};
-    uint64_t* k0 = ck0;  // reuse the CSR key buffers (2m entries each) for the (u, v) sort
-    uint64_t* k1 = ck1;
-    uint32_t* i0 = sc.get<uint32_t>((size_t)m);
-    uint32_t* i1 = sc.get<uint32_t>((size_t)m);
-    edge_keys_kernel<<<grid_for(m), 256, 0, s>>>(du, dv, m, bits_v, k0, i0);
+    int32_t* eu = sc.get<int32_t>((size_t)m);
+    int32_t* ev = sc.get<int32_t>((size_t)m);
+    int8_t* es = sc.get<int8_t>((size_t)m);
+    DBBC_CUDA(cudaMemsetAsync(d_flags, 0, sizeof(unsigned), s));
+    dedup_kernel<<<(unsigned)ceil_div<int64_t>(m, kRowTile), kRowThreads, 0, s>>>(
+        ku, m, bits_v, n_u, g->vertex, eu, ev, es, reinterpret_cast<uint64_t*>(&l.res->kept), l.dedup_state,
+        l.counters + 2, d_flags);
     DBBC_LAUNCH_CHECK();
-    const bool alt = radix_sort<uint64_t, uint32_t, true>(k0, k1, i0, i1, m, 0, bits_u + bits_v, s, sc);
-    const uint64_t* ks = alt ? k1 : k0;
-    const uint32_t* is = alt ? i1 : i0;
-    uint32_t* flag = alt ? i0 : i1;  // the free index buffer
-    uint32_t* pos = sc.get<uint32_t>((size_t)m);
-    run_last_kernel<<<grid_for(m), 256, 0, s>>>(ks, m, flag, d_flags + 1);
-    DBBC_LAUNCH_CHECK();
-    exclusive_scan<uint32_t, uint32_t>(flag, pos, m, s, sc, reinterpret_cast<uint32_t*>(d_flags + 2));
-    mu = read_back(d_flags + 2, s);
-    int32_t* eu = sc.get<int32_t>((size_t)mu);
-    int32_t* ev = sc.get<int32_t>((size_t)mu);
-    int8_t* es = sc.get<int8_t>((size_t)mu);
-    compact_edges_kernel<<<grid_for(m), 256, 0, s>>>(ks, is, flag, pos, ds, m, bits_v, eu, ev, es);
-    DBBC_LAUNCH_CHECK();
-    ck = csr_from_edges(eu, ev, es, mu, &dup);
-    if (dup) throw Error{DBBC_EINTERNAL, "duplicates left after deduplication"};
+    const PrepResult d = read_back(l.res, s);
+    if (d.flags & kPrepTimeout) throw Error{DBBC_ETIMEOUT, "a bounded wait of the build gave up"};
+    mu = (int64_t)d.kept;
+    graph_release(g, g->col, (size_t)(2 * m) * 4);
+    g->col = nullptr;
+    r = build_from_edges(eu, ev, es, mu);
+    if (r.flags & kPrepDup) throw Error{DBBC_EINTERNAL, "duplicates left after deduplication"};
   }
   g->m = mu;
   g->nnz = 2 * mu;
-  g->col = static_cast<uint32_t*>(graph_alloc(g, (size_t)g->nnz * 4));
-  g->lower = static_cast<uint32_t*>(graph_alloc(g, (size_t)n * 4));
-  g->work = static_cast<uint64_t*>(graph_alloc(g, (size_t)n * 8));
-  exclusive_scan<int32_t, int64_t>(rowdeg, g->row_ptr, n, s, sc, g->row_ptr + n);
-  DBBC_CUDA(cudaMemsetAsync(g->work, 0, (size_t)n * 8, s));
-  if (g->nnz > 0) {
-    csr_cols_kernel<<<grid_for(g->nnz), 256, 0, s>>>(ck, g->nnz, g->col);
-    DBBC_LAUNCH_CHECK();
-  }
-  if (n > 0) {
-    lower_kernel<<<grid_for(n), 256, 0, s>>>(g->row_ptr, g->col, rowdeg, n, n_u, uv, g->lower);
-    DBBC_LAUNCH_CHECK();
-  }
 
-  // ---- a4: accepted wedges per pivot and the counting tiers
-  if (g->nnz > 0) {
-    work_kernel<<<grid_for(g->m), 256, 0, s>>>(ck, g->row_ptr, g->lower,
-                                               reinterpret_cast<unsigned long long*>(g->work));
-    DBBC_LAUNCH_CHECK();
-  }
-  PrepStats* d_st = sc.get<PrepStats>(1);
-  DBBC_CUDA(cudaMemsetAsync(d_st, 0, sizeof(PrepStats), s));
-  uint32_t* pflag = sc.get<uint32_t>((size_t)std::max<int64_t>(n, 1));
-  if (n > 0) {
-    pivot_flags_kernel<<<grid_for(n), 256, 0, s>>>(g->work, g->lower, n, g->tune.light_max_work,
-                                                   g->tune.medium_max_work, pflag, d_st);
-    DBBC_LAUNCH_CHECK();
-  }
-  const PrepStats st = read_back(d_st, s);
+  // ---- the counting tiers: pivots in descending work, ties by row
+  const PrepStats& st = r.st;
   g->wedges = st.wedges;
   g->wedges_hub = st.wedges_hub;
   g->wedges_medium = st.wedges_medium;
@@ -886,40 +1023,30 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
   g->lower_light = (int64_t)st.lower_light;
   g->order = static_cast<int32_t*>(graph_alloc(g, (size_t)std::max<int64_t>(g->n_piv, 1) * 4));
   if (g->n_piv > 0) {
-    uint32_t* ppos = sc.get<uint32_t>((size_t)n);
-    exclusive_scan<uint32_t, uint32_t>(pflag, ppos, n, s, sc);
-    const int wbits = std::max(1, bits_for(st.max_work));
-    uint64_t* pk0 = sc.get<uint64_t>((size_t)g->n_piv);
-    uint64_t* pk1 = sc.get<uint64_t>((size_t)g->n_piv);
-    uint32_t* pr0 = reinterpret_cast<uint32_t*>(g->order);
-    uint32_t* pr1 = sc.get<uint32_t>((size_t)g->n_piv);
-    pivot_keys_kernel<<<grid_for(n), 256, 0, s>>>(g->work, pflag, ppos, n, wbits, pk0, pr0);
-    DBBC_LAUNCH_CHECK();
-    const bool alt = radix_sort<uint64_t, uint32_t, true>(pk0, pk1, pr0, pr1, g->n_piv, 0, wbits, s, sc);
-    if (alt)
-      DBBC_CUDA(cudaMemcpyAsync(pr0, pr1, (size_t)g->n_piv * 4, cudaMemcpyDeviceToDevice, s));
+    const int passes = radix_passes(0, bits_for(st.max_work));
+    uint64_t *kin = l.vk0, *kout = l.vk1;
+    uint32_t *vin = l.pr0, *vout = l.pr1;
+    for (int p = 0; p < passes; p++, std::swap(kin, kout), std::swap(vin, vout)) {
+      const PlainLoad in{kin, vin};
+      if (p + 1 == passes)
+        radix_pass<PlainLoad, true, false, false>(
+            in, PassOut{nullptr, reinterpret_cast<uint32_t*>(g->order), nullptr, 0}, g->n_piv, 0, p, l.piv, d_flags, s);
+      else
+        radix_pass<PlainLoad, true, true, false>(in, PassOut{kout, vout, nullptr, 0}, g->n_piv, 0, p, l.piv, d_flags,
+                                                 s);
+    }
   }
   // per side: how many vertices have degree < 2^16, < 2^8, < 2^4 and 0
-  // (ranks ascend by degree)
-  {
-    int64_t* d_t = sc.get<int64_t>(8);
-    const DegreeLimits lim{{kNarrowCountLimit, kTinyCountLimit, kQuarterCountLimit, 1}};
-    narrow_ranks_kernel<<<1, 32, 0, s>>>(rowdeg, n, n_u, lim, d_t);
-    DBBC_LAUNCH_CHECK();
-    int64_t ht[8];
-    DBBC_CUDA(cudaMemcpyAsync(ht, d_t, sizeof(ht), cudaMemcpyDeviceToHost, s));
-    DBBC_CUDA(cudaStreamSynchronize(s));
-    g->narrow_ranks_u = ht[0];
-    g->narrow_ranks_v = ht[1];
-    g->tiny_ranks_u = ht[2];
-    g->tiny_ranks_v = ht[3];
-    g->quarter_ranks_u = ht[4];
-    g->quarter_ranks_v = ht[5];
-    g->zero_ranks_u = ht[6];
-    g->zero_ranks_v = ht[7];
-  }
+  g->narrow_ranks_u = r.below[0];
+  g->narrow_ranks_v = r.below[1];
+  g->tiny_ranks_u = r.below[2];
+  g->tiny_ranks_v = r.below[3];
+  g->quarter_ranks_u = r.below[4];
+  g->quarter_ranks_v = r.below[5];
+  g->zero_ranks_u = r.below[6];
+  g->zero_ranks_v = r.below[7];
   plan_hubs(g, s, *un);
-  DBBC_CUDA(cudaStreamSynchronize(s));
+  if (read_back(d_flags, s) & kPrepTimeout) throw Error{DBBC_ETIMEOUT, "a bounded wait of the build gave up"};
 }
 
 }  // namespace dbbc

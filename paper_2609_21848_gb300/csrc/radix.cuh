@@ -1,17 +1,65 @@
-// In-repo device primitives: exclusive scan and a stable LSD radix sort
-// (8-bit digits, per-tile histograms, warp-ballot ranking, shared-memory staging
-// so that the scatter writes whole digit runs). Written for sm_103a; no CUB.
+// In-repo device primitives: single-pass prefix sums over tiles and a stable
+// LSD radix sort with one kernel per digit. Written for sm_103a; no CUB.
+//
+// Both chain their tiles by decoupled look-back (Merrill and Garland,
+// "Single-pass Parallel Prefix Scan with Decoupled Look-back", 2016): a tile
+// publishes its own sum, adds up what the tiles before it have published until
+// it meets one whose running total is known, and publishes its own running
+// total. Tiles are numbered by a counter in the order in which their CTAs
+// start, so every tile that one waits for is running or done. Each wait is
+// bounded all the same: a tile that polls kSpinLimit times sets kPrepTimeout in
+// the pass's flag word and returns, every other wait then ends at once, and
+// the kernels that follow see the flag and return.
 #pragma once
+
+#include <algorithm>
 
 #include "common.cuh"
 
 namespace dbbc {
 
-// ------------------------------------------------------------------ scans
-constexpr int kScanThreads = 256;
-constexpr int kScanItems = 8;
-constexpr int kScanTile = kScanThreads * kScanItems;
+// Bits of a build's device flag word. kPrepStop: the kernels after the one
+// that set it have nothing valid to work on and return.
+enum : unsigned {
+  kPrepBadU = 1u,
+  kPrepBadV = 2u,
+  kPrepBadSign = 4u,
+  kPrepInvalid = kPrepBadU | kPrepBadV | kPrepBadSign,
+  kPrepDup = 8u,       // a (u, v) pair occurs twice
+  kPrepTimeout = 16u,  // a bounded wait gave up
+  kPrepStop = kPrepInvalid | kPrepDup | kPrepTimeout,
+};
 
+constexpr uint32_t kSpinLimit = 1u << 22;  // polls of one wait (seconds; a wait normally takes microseconds)
+
+__device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
+  uint32_t v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint64_t ld_relaxed(const uint64_t* p) {
+  uint64_t v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ void st_relaxed(uint32_t* p, uint32_t v) {
+  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_relaxed(uint64_t* p, uint64_t v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
+}
+
+// True when a wait that has polled `polls` times has to end: it reached its
+// limit (which sets the flag), or another one did.
+__device__ __forceinline__ bool wait_over(uint32_t polls, unsigned* flags) {
+  if (polls >= kSpinLimit) {
+    atomicOr(flags, (unsigned)kPrepTimeout);
+    return true;
+  }
+  return (polls & 63u) == 63u && (ld_relaxed(flags) & kPrepTimeout) != 0;
+}
+
+// ------------------------------------------------------------------ scans
 // Inclusive warp scan.
 template <typename T>
 __device__ __forceinline__ T warp_incl_scan(T x) {
@@ -43,272 +91,326 @@ __device__ __forceinline__ T block_excl_scan(T x, T* total) {
   return warp_tot[w] + inc - x;
 }
 
-template <typename TI, typename TO>
-__global__ void __launch_bounds__(kScanThreads) scan_reduce_kernel(const TI* in, int64_t n, TO* tile_sums) {
-  const int64_t base = (int64_t)blockIdx.x * kScanTile;
-  TO s = 0;
-  for (int i = threadIdx.x; i < kScanTile; i += kScanThreads) {
-    const int64_t k = base + i;
-    if (k < n) s += (TO)in[k];
-  }
-  __shared__ TO tot;
-  block_excl_scan<TO, kScanThreads>(s, &tot);
-  if (threadIdx.x == 0) tile_sums[blockIdx.x] = tot;
+// Whether this CTA has to return at once (kPrepStop), the same answer in every
+// thread although other CTAs may be setting the flag. Contains __syncthreads.
+__device__ __forceinline__ bool cta_stopped(const unsigned* flags) {
+  return __syncthreads_or(threadIdx.x == 0 && (ld_relaxed(flags) & kPrepStop) != 0) != 0;
 }
 
-// In-place exclusive scan of the tile sums by one block of 1024 threads.
-template <typename TO>
-__global__ void __launch_bounds__(1024) scan_top_kernel(TO* sums, int64_t n, TO* grand_total) {
-  __shared__ TO tot;
-  TO carry = 0;
-  for (int64_t base = 0; base < n; base += 1024) {
-    const int64_t k = base + threadIdx.x;
-    TO x = k < n ? sums[k] : TO(0);
-    TO ex = block_excl_scan<TO, 1024>(x, &tot);
-    if (k < n) sums[k] = carry + ex;
-    carry += tot;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0 && grand_total) *grand_total = carry;
+// The number of this CTA's tile, the same in every thread, or -1 when the CTA
+// has to return (kPrepStop). Contains __syncthreads.
+__device__ __forceinline__ int64_t take_tile(unsigned* counter, const unsigned* flags) {
+  __shared__ int64_t tile_sh;
+  if (threadIdx.x == 0) tile_sh = (ld_relaxed(flags) & kPrepStop) != 0 ? -1 : (int64_t)atomicAdd(counter, 1u);
+  __syncthreads();
+  return tile_sh;
 }
 
-template <typename TI, typename TO>
-__global__ void __launch_bounds__(kScanThreads) scan_down_kernel(const TI* in, int64_t n, const TO* tile_off,
-                                                                 TO* out) {
-  const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
-  TO v[kScanItems];
-  TO s = 0;
-#pragma unroll
-  for (int j = 0; j < kScanItems; j++) {
-    v[j] = (base + j < n) ? (TO)in[base + j] : TO(0);
-    s += v[j];
-  }
-  __shared__ TO tot;
-  TO run = block_excl_scan<TO, kScanThreads>(s, &tot) + tile_off[blockIdx.x];
-#pragma unroll
-  for (int j = 0; j < kScanItems; j++) {
-    if (base + j < n) out[base + j] = run;
-    run += v[j];
-  }
-}
+// Exclusive prefix of `sum` over the tiles before this one (sums below 2^62).
+// Called by all threads; `state` (one zeroed word per tile) holds 0 (nothing
+// yet), kTileSum | sum or kTileTotal | running total. Warp 0 looks at 32
+// earlier tiles at a time. Returns false when a wait gave up.
+constexpr uint64_t kTileSum = 1ull << 62, kTileTotal = 2ull << 62, kTileValue = kTileSum - 1;
 
-// out[i] = sum_{k<i} in[k]; optionally the grand total into device *total.
-// `out` may alias `in`.
-template <typename TI, typename TO>
-void exclusive_scan(const TI* in, TO* out, int64_t n, cudaStream_t s, Scratch& scratch, TO* total = nullptr) {
-  if (n <= 0) {
-    if (total) DBBC_CUDA(cudaMemsetAsync(total, 0, sizeof(TO), s));
-    return;
+__device__ __forceinline__ bool tile_prefix(uint64_t* state, int64_t tile, uint64_t sum, unsigned* flags,
+                                            uint64_t* prefix) {
+  __shared__ uint64_t pre_sh;
+  __shared__ int ok_sh;
+  if (threadIdx.x < 32) {
+    const unsigned lane = lane_id();
+    if (lane == 0) st_relaxed(&state[tile], (tile == 0 ? kTileTotal : kTileSum) | sum);
+    uint64_t pre = 0;
+    bool ok = true;
+    int64_t end = tile;  // the tiles [end, tile) are in `pre`
+    uint32_t polls = 0;
+    while (end > 0) {
+      const int64_t t = end - 1 - (int64_t)lane;
+      const uint64_t s = t >= 0 ? ld_relaxed(&state[t]) : kTileTotal;
+      // lanes up to the first running total count, if all before it are there
+      const unsigned total = __ballot_sync(kFullMask, (s & kTileTotal) != 0);
+      const unsigned none = __ballot_sync(kFullMask, (s & (kTileTotal | kTileSum)) == 0);
+      const unsigned upto = total ? (total & (0u - total)) : 0u;            // its bit
+      const unsigned need = total ? (upto | (upto - 1u)) : kFullMask;       // lanes 0 .. first total
+      const unsigned miss = none & need;
+      const unsigned take = miss ? ((miss & (0u - miss)) - 1u) : need;      // lanes before the first gap
+      pre += warp_sum_u64((take >> lane) & 1u ? (s & kTileValue) : 0ull);
+      if (total && !miss) break;
+      end -= __popc(take);
+      if (take == 0u) {
+        const bool over = __any_sync(kFullMask, lane == 0 && wait_over(++polls, flags));
+        if (over) {
+          ok = false;
+          break;
+        }
+      }
+    }
+    if (lane == 0) {
+      if (ok && tile > 0) st_relaxed(&state[tile], kTileTotal | (pre + sum));
+      pre_sh = pre;
+      ok_sh = ok ? 1 : 0;
+    }
   }
-  const int64_t tiles = ceil_div<int64_t>(n, kScanTile);
-  TO* sums = scratch.get<TO>((size_t)tiles);
-  scan_reduce_kernel<TI, TO><<<(unsigned)tiles, kScanThreads, 0, s>>>(in, n, sums);
-  DBBC_LAUNCH_CHECK();
-  scan_top_kernel<TO><<<1, 1024, 0, s>>>(sums, tiles, total);
-  DBBC_LAUNCH_CHECK();
-  scan_down_kernel<TI, TO><<<(unsigned)tiles, kScanThreads, 0, s>>>(in, n, sums, out);
-  DBBC_LAUNCH_CHECK();
+  __syncthreads();
+  *prefix = pre_sh;
+  return ok_sh != 0;
 }
 
 // ------------------------------------------------------------------ radix sort
-constexpr int kRsThreads = 256;
-constexpr int kRsWarps = kRsThreads / 32;
+// Keys are 64-bit, values 32-bit, digits 8 bits. The caller's key kernel
+// writes the keys and counts every digit of the sort at once (DigitCounts);
+// each digit is then one pass over the keys and one launch, where a histogram
+// kernel, a three-kernel scan of the per-tile histograms and a scatter kernel
+// took two reads and five launches. Whole builds on GB300, with the first
+// pass, the digit counts and the row entries fused as in prep.cu: 20k edges
+// 424 -> 188 us, 2M with repeated pairs 1.55 -> 0.84 ms, 20M 3.72 -> 3.02 ms,
+// 300M 47.5 -> 41.4 ms. Tiles of 512 threads x 8 keys, two CTAs per SM, were
+// the best of 256 x 8, 256 x 12, 256 x 16, 384 x 8 and 512 x 8 with one CTA
+// (20M: 3.21, 3.10, 3.06, 3.18 and 3.50 ms).
+#ifndef DBBC_RS_THREADS
+#define DBBC_RS_THREADS 512
+#endif
 #ifndef DBBC_RS_ITEMS
 #define DBBC_RS_ITEMS 8
 #endif
-#ifndef DBBC_RS_MATCH
-#define DBBC_RS_MATCH 0
+#ifndef DBBC_RS_CTAS
+#define DBBC_RS_CTAS 2
 #endif
+constexpr int kRsThreads = DBBC_RS_THREADS;
+constexpr int kRsWarps = kRsThreads / 32;
 constexpr int kRsItems = DBBC_RS_ITEMS;         // keys per thread
-constexpr int kRsTile = kRsThreads * kRsItems;  // keys per tile (2048 by default)
+constexpr int kRsTile = kRsThreads * kRsItems;  // keys per tile
+constexpr int kRsMaxPasses = 8;
+static_assert(kRsThreads >= 256, "one thread per digit");
 
-template <typename K>
-__device__ __forceinline__ uint32_t rs_digit(K key, int shift) {
-  return (uint32_t)(key >> shift) & 0xFFu;
+__device__ __forceinline__ uint32_t rs_digit(uint64_t key, int shift) { return (uint32_t)(key >> shift) & 0xFFu; }
+
+inline int radix_passes(int begin_bit, int end_bit) {
+  return std::max(1, ceil_div(end_bit - begin_bit, 8));
 }
+inline int64_t radix_tiles(int64_t n) { return ceil_div<int64_t>(std::max<int64_t>(n, 1), kRsTile); }
 
-// The lanes of the warp whose d (a digit, or 256 for "no key") equals this
-// lane's: one ballot per bit of d, each lane keeping the lanes that agree with
-// it on that bit. Nine ballots and a few logic operations per key run the
-// digit passes faster than one warp match instruction per key (the Chung-Lu
-// 1M x 200k x 20M build: 4.08 -> 3.70 ms). DBBC_RS_MATCH=1 builds the match
-// form.
-__device__ __forceinline__ unsigned rs_peers(uint32_t d) {
-#if DBBC_RS_MATCH
-  return __match_any_sync(kFullMask, d);
-#else
-  unsigned peers = kFullMask;
+// Zeroed device words of one sort: digit counts of every pass, tile counters
+// and tile states (see radix_pass_kernel).
+struct RadixState {
+  uint32_t* hist;      // [passes][256]
+  unsigned* counters;  // [passes]
+  uint32_t* state;     // [passes][tiles][256]
+};
+
+// Counts of all digits of a sort, kept in shared memory by the kernel that
+// makes the keys. Every thread of the CTA calls start and finish.
+struct DigitCounts {
+  uint32_t (*h)[256];
+  int passes, begin_bit;
+  __device__ __forceinline__ void start() {
+    for (int i = threadIdx.x; i < passes * 256; i += blockDim.x) (&h[0][0])[i] = 0;
+    __syncthreads();
+  }
+  __device__ __forceinline__ void add(uint64_t key) {
+    for (int p = 0; p < passes; p++) atomicAdd(&h[p][rs_digit(key, begin_bit + 8 * p)], 1u);
+  }
+  __device__ __forceinline__ void finish(uint32_t* hist) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < passes * 256; i += blockDim.x) {
+      const uint32_t c = (&h[0][0])[i];
+      if (c) atomicAdd(&hist[i], c);
+    }
+  }
+};
+
+// Where a pass's keys (and values) come from: the arrays of the pass before,
+// or a transformation of another list (see prep.cu).
+struct PlainLoad {
+  const uint64_t* kin;
+  const uint32_t* vin;
+  __device__ __forceinline__ uint64_t key(uint32_t i) const { return kin[i]; }
+  __device__ __forceinline__ uint32_t val(uint32_t i) const { return vin[i]; }
+};
+
+// What a pass writes: keys and / or values, and with AUX (key & aux_mask) as a
+// 32-bit word per key.
+struct PassOut {
+  uint64_t* key;
+  uint32_t* val;
+  uint32_t* aux;
+  uint64_t aux_mask;
+};
+
+// The lanes of the warp whose digit d equals this lane's, among the lanes of
+// `valid`: one ballot per bit of d, each lane keeping the lanes that agree with
+// it on that bit (a warp match instruction per key runs slower).
+__device__ __forceinline__ unsigned rs_peers(uint32_t d, unsigned valid) {
+  unsigned peers = valid;
 #pragma unroll
-  for (int b = 0; b < 9; b++) {
+  for (int b = 0; b < 8; b++) {
     const bool bit = (d >> b) & 1u;
     const unsigned bal = __ballot_sync(kFullMask, bit);
     peers &= bit ? bal : ~bal;
   }
   return peers;
-#endif
 }
 
-// Per-tile digit counts, digit-major: hist[d * ntiles + tile]. Every thread
-// loads its kRsItems keys before counting any, so that each warp has kRsItems
-// loads in flight at once.
-template <typename K>
-__global__ void __launch_bounds__(kRsThreads) radix_hist_kernel(const K* __restrict__ keys, int64_t n, int shift,
-                                                                 uint32_t* hist, int64_t ntiles) {
-  __shared__ uint32_t h[kRsWarps][256];
-  const int w = threadIdx.x >> 5;
-  const int64_t base = (int64_t)blockIdx.x * kRsTile + threadIdx.x;
-  K key[kRsItems];
-#pragma unroll
-  for (int j = 0; j < kRsItems; j++) {
-    const int64_t k = base + j * kRsThreads;
-    key[j] = k < n ? keys[k] : K(0);
-  }
-  for (int i = threadIdx.x; i < kRsWarps * 256; i += kRsThreads) (&h[0][0])[i] = 0;
-  __syncthreads();
-#pragma unroll
-  for (int j = 0; j < kRsItems; j++) {
-    const uint32_t d = base + j * kRsThreads < n ? rs_digit(key[j], shift) : 256u;
-    const unsigned peers = rs_peers(d);
-    if (d < 256u && (int)lane_id() == 31 - __clz(peers)) h[w][d] += __popc(peers);
-    __syncwarp();
-  }
-  __syncthreads();
-  uint32_t c = 0;
-#pragma unroll
-  for (int ww = 0; ww < kRsWarps; ww++) c += h[ww][threadIdx.x];
-  hist[(int64_t)threadIdx.x * ntiles + blockIdx.x] = c;
-}
+// One digit pass of the stable sort, one tile per CTA. The tile's keys are
+// loaded, kRsItems per thread in flight together; each warp ranks its keys in
+// input order (digit peers per key, per-warp digit counters); the tile's digit
+// counts are published, the tile is staged in shared memory in digit order,
+// and thread d looks back over the earlier tiles for digit d, four of them per
+// round of loads. The tile is then written out as whole digit runs. A tile
+// state is one word per digit: 0 (nothing yet), 1 + the tile's count, or
+// kDigitTotal | the running total (totals are below 2^31). A pass over 20M keys
+// takes 157 us (1.76 TB/s; the two kernels it replaces, 70 + 100 us and their
+// scan 25): 52% of the issue slots, half of them the digit ballots, the rest
+// waits at the tile's barriers with 32 warps per SM.
+constexpr uint32_t kDigitTotal = 0x80000000u;
 
-// One digit pass of the stable sort. A tile's keys (and values) are loaded
-// first, all kRsItems per thread in flight together; each warp then ranks its
-// 256 keys in input order (digit peers per key, per-warp digit counters), the
-// block turns the per-warp counts into tile positions, the tile is staged in
-// shared memory in digit order, and written out as whole digit runs at the
-// offsets of the scanned digit-major histogram.
-template <typename K, typename V, bool HAS_V>
-__global__ void __launch_bounds__(kRsThreads) radix_scatter_kernel(const K* __restrict__ kin, const V* __restrict__ vin,
-                                                                    K* __restrict__ kout, V* __restrict__ vout,
-                                                                    int64_t n, int shift, const uint32_t* offs,
-                                                                    int64_t ntiles) {
+template <class Load, bool HAS_V, bool WRITE_K, bool AUX>
+__global__ void __launch_bounds__(kRsThreads, DBBC_RS_CTAS) radix_pass_kernel(Load load, PassOut out, int64_t n, int shift,
+                                                                const uint32_t* __restrict__ hist, uint32_t* state,
+                                                                unsigned* counter, unsigned* flags) {
   extern __shared__ __align__(16) unsigned char rs_smem[];
-  K* sk = reinterpret_cast<K*>(rs_smem);
-  V* sv = reinterpret_cast<V*>(sk + kRsTile);
-  uint32_t* wh = reinterpret_cast<uint32_t*>(HAS_V ? (void*)(sv + kRsTile) : (void*)(sk + kRsTile));
-  uint32_t* bstart = wh + kRsWarps * 256;
-  uint32_t* gofs = bstart + 256;
+  // warp digit counters first, then the staged tile, in the same memory
+  uint32_t* wh = reinterpret_cast<uint32_t*>(rs_smem);
+  uint64_t* sk = reinterpret_cast<uint64_t*>(rs_smem);
+  uint32_t* sv = reinterpret_cast<uint32_t*>(sk + kRsTile);
+  __shared__ uint32_t bstart[256], gofs[256];
   __shared__ uint32_t tot_sh;
-
+  __shared__ int ok_sh;
+  const int64_t tile = take_tile(counter, flags);
+  if (tile < 0) return;
   const int w = threadIdx.x >> 5;
   const unsigned lane = lane_id();
-  const int64_t tile_base = (int64_t)blockIdx.x * kRsTile;
-  const int64_t wbase = tile_base + (int64_t)w * (kRsItems * 32);
-  K key[kRsItems];
-  V val[kRsItems];
+  const uint32_t nk = (uint32_t)n;  // below 2^31, so tiles end below 2^32
+  const uint32_t tile_base = (uint32_t)tile * kRsTile;
+  const uint32_t wbase = tile_base + (uint32_t)w * (kRsItems * 32) + lane;
+  uint64_t key[kRsItems];
+  uint32_t val[kRsItems];
 #pragma unroll
   for (int j = 0; j < kRsItems; j++) {
-    const int64_t i = wbase + j * 32 + lane;
-    const bool valid = i < n;
-    key[j] = valid ? kin[i] : K(0);
-    if (HAS_V) val[j] = valid ? vin[i] : V(0);
+    const uint32_t i = wbase + j * 32;
+    const bool valid = i < nk;
+    key[j] = valid ? load.key(i) : 0ull;
+    if (HAS_V) val[j] = valid ? load.val(i) : 0u;
   }
+  // exclusive prefix of the digit's count over smaller digits
+  const uint32_t digit_base =
+      block_excl_scan<uint32_t, kRsThreads>(threadIdx.x < 256 ? hist[threadIdx.x] : 0u, &tot_sh);
   for (int i = threadIdx.x; i < kRsWarps * 256; i += kRsThreads) wh[i] = 0;
-  gofs[threadIdx.x] = offs[(int64_t)threadIdx.x * ntiles + blockIdx.x];
+  if (threadIdx.x == 0) ok_sh = 1;
   __syncthreads();
 
-  // digits (256 = past the end) and their warp peers, independent per item
-  unsigned peers[kRsItems];
-#pragma unroll
-  for (int j = 0; j < kRsItems; j++) {
-    const uint32_t d = wbase + j * 32 + lane < n ? rs_digit(key[j], shift) : 256u;
-    peers[j] = rs_peers(d);
-  }
   // rank within the warp, item by item in input order
   const unsigned lt_mask = (1u << lane) - 1u;
   uint32_t loc[kRsItems];
 #pragma unroll
   for (int j = 0; j < kRsItems; j++) {
-    const uint32_t d = wbase + j * 32 + lane < n ? rs_digit(key[j], shift) : 256u;
+    const bool ok = wbase + j * 32 < nk;
+    const unsigned valid = __ballot_sync(kFullMask, ok);
+    const uint32_t d = rs_digit(key[j], shift);
+    const unsigned peers = rs_peers(d, valid);
     uint32_t pre = 0;
-    if (d < 256u) pre = wh[w * 256 + d];
+    if (ok) pre = wh[w * 256 + d];
     __syncwarp();
-    loc[j] = pre + __popc(peers[j] & lt_mask);
-    if (d < 256u && (int)lane == 31 - __clz(peers[j])) wh[w * 256 + d] = pre + __popc(peers[j]);
+    loc[j] = pre + __popc(peers & lt_mask);
+    if (ok && (int)lane == 31 - __clz(peers)) wh[w * 256 + d] = pre + __popc(peers);
     __syncwarp();
   }
   __syncthreads();
   {  // per digit: exclusive prefix over warps, then over digits
     const int d = threadIdx.x;
     uint32_t run = 0;
+    if (d < 256) {
 #pragma unroll
-    for (int ww = 0; ww < kRsWarps; ww++) {
-      const uint32_t c = wh[ww * 256 + d];
-      wh[ww * 256 + d] = run;
-      run += c;
+      for (int ww = 0; ww < kRsWarps; ww++) {
+        const uint32_t c = wh[ww * 256 + d];
+        wh[ww * 256 + d] = run;
+        run += c;
+      }
+      st_relaxed(&state[tile * 256 + d], tile == 0 ? kDigitTotal | run : 1u + run);
     }
     const uint32_t ex = block_excl_scan<uint32_t, kRsThreads>(run, &tot_sh);
-    bstart[d] = ex;
-  }
-  __syncthreads();
-#pragma unroll
-  for (int j = 0; j < kRsItems; j++) {
-    const bool valid = wbase + j * 32 + lane < n;
-    const uint32_t d = valid ? rs_digit(key[j], shift) : 256u;
-    const uint32_t pos = valid ? bstart[d] + wh[w * 256 + d] + loc[j] : 0u;
-    if (valid && DBBC_CHECK(pos < (uint32_t)kRsTile)) {
-      sk[pos] = key[j];
-      if (HAS_V) sv[pos] = val[j];
+    if (d < 256) {
+      bstart[d] = ex;
+      gofs[d] = run;  // the tile's count, until the look-back
     }
   }
   __syncthreads();
-  const int64_t rem = n - tile_base;
-  const int cnt = rem < kRsTile ? (int)rem : kRsTile;
 #pragma unroll
   for (int j = 0; j < kRsItems; j++) {
-    const int i = threadIdx.x + j * kRsThreads;
+    const uint32_t d = rs_digit(key[j], shift);
+    loc[j] += bstart[d] + wh[w * 256 + d];
+  }
+  __syncthreads();  // the counters' memory is free
+#pragma unroll
+  for (int j = 0; j < kRsItems; j++) {
+    if (wbase + j * 32 < nk && DBBC_CHECK(loc[j] < (uint32_t)kRsTile)) {
+      sk[loc[j]] = key[j];
+      if (HAS_V) sv[loc[j]] = val[j];
+    }
+  }
+  if (threadIdx.x < 256) {  // look back for digit d
+    const int d = threadIdx.x;
+    const uint32_t count = gofs[d];
+    uint32_t before = 0, polls = 0;
+    bool ok = true;
+    for (int64_t t = tile - 1; t >= 0;) {
+      uint32_t s[4];
+#pragma unroll
+      for (int k = 0; k < 4; k++) s[k] = t - k >= 0 ? ld_relaxed(&state[(t - k) * 256 + d]) : kDigitTotal;
+      int used = 0;
+      bool done = false;
+#pragma unroll
+      for (int k = 0; k < 4; k++) {
+        if (!done && used == k && s[k] != 0u) {
+          used = k + 1;
+          done = (s[k] & kDigitTotal) != 0u;
+          before += done ? s[k] & ~kDigitTotal : s[k] - 1u;
+        }
+      }
+      if (done) break;
+      t -= used;
+      if (used == 0 && wait_over(++polls, flags)) {
+        ok = false;
+        break;
+      }
+    }
+    if (ok) {
+      if (tile > 0) st_relaxed(&state[tile * 256 + d], kDigitTotal | (before + count));
+    } else {
+      ok_sh = 0;
+    }
+    gofs[d] = digit_base + before - bstart[d];
+  }
+  __syncthreads();
+  if (!ok_sh) return;
+  const uint32_t cnt = min(nk - tile_base, (uint32_t)kRsTile);
+#pragma unroll
+  for (int j = 0; j < kRsItems; j++) {
+    const uint32_t i = threadIdx.x + j * kRsThreads;
     if (i < cnt) {
-      const K k = sk[i];
-      const uint32_t d = rs_digit(k, shift);
-      const int64_t g = (int64_t)gofs[d] + (i - (int64_t)bstart[d]);
-      if (DBBC_CHECK(g >= 0 && g < n)) {
-        kout[g] = k;
-        if (HAS_V) vout[g] = sv[i];
+      const uint64_t k = sk[i];
+      const uint32_t g = gofs[rs_digit(k, shift)] + i;
+      if (g < nk) {
+        if (WRITE_K) out.key[g] = k;
+        if (HAS_V) out.val[g] = sv[i];
+        if (AUX) out.aux[g] = (uint32_t)(k & out.aux_mask);
       }
     }
   }
 }
 
-template <typename K, typename V, bool HAS_V>
-size_t radix_scatter_smem() {
-  return (size_t)kRsTile * (sizeof(K) + (HAS_V ? sizeof(V) : 0)) + (size_t)(kRsWarps * 256 + 512) * 4;
-}
-
-// Stable sort of keys (and values) by bits [begin_bit, end_bit). Sorts between
-// the two buffers of each pair; returns true when the result ended in the
-// *_alt buffers. n < 2^32.
-template <typename K, typename V, bool HAS_V>
-bool radix_sort(K* keys, K* keys_alt, V* vals, V* vals_alt, int64_t n, int begin_bit, int end_bit, cudaStream_t s,
-                Scratch& scratch) {
-  if (n <= 1 || end_bit <= begin_bit) return false;
-  const int64_t ntiles = ceil_div<int64_t>(n, kRsTile);
-  uint32_t* hist = scratch.get<uint32_t>((size_t)ntiles * 256);
-  const size_t smem = radix_scatter_smem<K, V, HAS_V>();
-  DBBC_CUDA(cudaFuncSetAttribute(radix_scatter_kernel<K, V, HAS_V>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem));
-  bool alt = false;
-  for (int shift = begin_bit; shift < end_bit; shift += 8) {
-    const K* kin = alt ? keys_alt : keys;
-    K* kout = alt ? keys : keys_alt;
-    const V* vin = alt ? vals_alt : vals;
-    V* vout = alt ? vals : vals_alt;
-    radix_hist_kernel<K><<<(unsigned)ntiles, kRsThreads, 0, s>>>(kin, n, shift, hist, ntiles);
-    DBBC_LAUNCH_CHECK();
-    exclusive_scan<uint32_t, uint32_t>(hist, hist, ntiles * 256, s, scratch);
-    radix_scatter_kernel<K, V, HAS_V><<<(unsigned)ntiles, kRsThreads, smem, s>>>(kin, vin, kout, vout, n, shift,
-                                                                                  hist, ntiles);
-    DBBC_LAUNCH_CHECK();
-    alt = !alt;
-  }
-  return alt;
+// Launch one pass (pass number `pass` of the sort: digit counts, tile counter
+// and states of `st`).
+template <class Load, bool HAS_V, bool WRITE_K, bool AUX>
+void radix_pass(const Load& load, const PassOut& out, int64_t n, int begin_bit, int pass, const RadixState& st,
+                unsigned* flags, cudaStream_t s) {
+  auto fn = radix_pass_kernel<Load, HAS_V, WRITE_K, AUX>;
+  const size_t staged = (size_t)kRsTile * (8 + (HAS_V ? 4 : 0)), counters = (size_t)kRsWarps * 256 * 4;
+  const size_t smem = std::max(staged, counters);
+  DBBC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  const int64_t tiles = radix_tiles(n);
+  fn<<<(unsigned)tiles, kRsThreads, smem, s>>>(load, out, n, begin_bit + 8 * pass, st.hist + 256 * pass,
+                                               st.state + (size_t)pass * tiles * 256, st.counters + pass, flags);
+  DBBC_LAUNCH_CHECK();
 }
 
 }  // namespace dbbc
