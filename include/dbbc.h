@@ -59,7 +59,7 @@ typedef enum {
   DBBC_EINVAL = 1,    /* bad argument or input (id out of range, sign not +-1, m < 0, duplicate under DUP_REJECT) */
   DBBC_ENOMEM = 2,    /* a device allocation failed */
   DBBC_ECUDA = 3,     /* a CUDA runtime call or kernel launch failed */
-  DBBC_ETIMEOUT = 4,  /* a bounded wait of a build's prefix-sum kernels gave up (none of its tiles waits on a later one) */
+  DBBC_ETIMEOUT = 4,  /* reserved: no kernel of this library waits on another, so no call returns it */
   DBBC_EOVERFLOW = 5, /* a count or an internal capacity exceeded its type */
   DBBC_EINTERNAL = 6  /* an internal consistency check failed (a bug: please report) */
 } dbbc_status;
@@ -80,8 +80,7 @@ enum {
  *   out        : receives a new handle on success.
  * Synchronous with respect to `cuda_stream` (it reads sizes back to the host).
  * Errors: DBBC_EINVAL (any id out of range, any sign not +-1, bad sizes or
- * flags, duplicates under DBBC_DUP_REJECT), DBBC_ENOMEM, DBBC_ECUDA,
- * DBBC_ETIMEOUT. */
+ * flags, duplicates under DBBC_DUP_REJECT), DBBC_ENOMEM, DBBC_ECUDA. */
 DBBC_API dbbc_status dbbc_graph_from_coo(const int32_t* u, const int32_t* v, const int8_t* sign, int64_t m, int32_t n_u,
                                 int32_t n_v, uint32_t flags, void* cuda_stream, dbbc_graph** out);
 

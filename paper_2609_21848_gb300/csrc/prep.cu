@@ -978,7 +978,7 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
     }
     const PrepResult r = read_back(l.res, s);
     if (r.flags & kPrepInvalid) throw Error{DBBC_EINVAL, "invalid edge id or sign"};
-    if (r.flags & kPrepTimeout) throw Error{DBBC_ETIMEOUT, "a bounded wait of the build gave up"};
+    if (r.flags & kPrepTimeout) throw Error{DBBC_EINTERNAL, "a bounded wait of the build gave up"};
     return r;
   };
 
@@ -998,7 +998,7 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
         l.counters + 2, d_flags);
     DBBC_LAUNCH_CHECK();
     const PrepResult d = read_back(l.res, s);
-    if (d.flags & kPrepTimeout) throw Error{DBBC_ETIMEOUT, "a bounded wait of the build gave up"};
+    if (d.flags & kPrepTimeout) throw Error{DBBC_EINTERNAL, "a bounded wait of the build gave up"};
     mu = (int64_t)d.kept;
     graph_release(g, g->col, (size_t)(2 * m) * 4);
     g->col = nullptr;
@@ -1046,7 +1046,7 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
   g->zero_ranks_u = r.below[6];
   g->zero_ranks_v = r.below[7];
   plan_hubs(g, s, *un);
-  if (read_back(d_flags, s) & kPrepTimeout) throw Error{DBBC_ETIMEOUT, "a bounded wait of the build gave up"};
+  if (read_back(d_flags, s) & kPrepTimeout) throw Error{DBBC_EINTERNAL, "a bounded wait of the build gave up"};
 }
 
 }  // namespace dbbc
