@@ -121,6 +121,10 @@ constexpr int16_t kItemFirst = 8;
 constexpr int32_t kTinyCountLimit = 256;
 constexpr int32_t kQuarterCountLimit = 16;
 
+// Bytes allocated past the CSR's last entry: the hub sweep reads rows in
+// aligned chunks of up to 128 entries, the last of which may pass the end.
+constexpr size_t kColPad = 512;
+
 // Read-only view of the device CSR passed to kernels by value.
 // Rows [0, n_u) are U vertices in ascending Def. 3 priority, rows [n_u, n)
 // V vertices in ascending priority. A row lists its neighbours by ascending
@@ -194,7 +198,7 @@ void build_graph_multi(dbbc_graph* g, const int32_t* u, const int32_t* v, const 
                        const int64_t* edge_offsets, const int32_t* n_u, const int32_t* n_v, int32_t n_graphs,
                        bool on_device, bool reject_duplicates, cudaStream_t stream);
 void free_graph_memory(dbbc_graph* g);
-void* graph_alloc(dbbc_graph* g, size_t bytes);
+void* graph_alloc(dbbc_graph* g, size_t bytes, size_t pad = 0);  // pad: slack past the end, not counted
 
 // Event brackets around tiers of one count (profiled counts only).
 struct CountProfiler {

@@ -559,8 +559,8 @@ static unsigned grid_for(int64_t n, int threads = 256) {
 // the global counts.
 static unsigned count_grid(int64_t n) { return std::min(grid_for(n), (unsigned)kNumSMs * 8u); }
 
-void* graph_alloc(dbbc_graph* g, size_t bytes) {
-  void* p = dev_alloc(bytes ? bytes : 16, g->stream);
+void* graph_alloc(dbbc_graph* g, size_t bytes, size_t pad) {
+  void* p = dev_alloc((bytes ? bytes : 16) + pad, g->stream);
   if (!p) throw Error{DBBC_ENOMEM, "graph_alloc"};
   g->allocations.push_back(p);
   g->device_bytes += bytes;
@@ -912,7 +912,7 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
   const uint64_t* ku = nullptr;
   auto build_from_edges = [&](const int32_t* eu, const int32_t* ev, const int8_t* es, int64_t me) -> PrepResult {
     DBBC_CUDA(cudaMemsetAsync(l.res, 0, l.zeroed, s));
-    g->col = static_cast<uint32_t*>(graph_alloc(g, (size_t)(2 * me) * 4));
+    g->col = static_cast<uint32_t*>(graph_alloc(g, (size_t)(2 * me) * 4, kColPad));
     if (me > 0) {
       degree_kernel<<<grid_for(me), 256, 0, s>>>(eu, ev, es, me, n_u, n_v, l.deg, d_flags);
       DBBC_LAUNCH_CHECK();
