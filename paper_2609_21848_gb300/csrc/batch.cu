@@ -8,6 +8,7 @@
 #include <algorithm>
 #include <numeric>
 
+#include "radix.cuh"
 #include "sweep_device.cuh"
 
 namespace dbbc {
@@ -64,12 +65,6 @@ __global__ void gather_component_pivots_kernel(const int32_t* __restrict__ order
     if (i < n_medium) med[i] = bp;
     else light[i - n_medium] = bp;
   }
-}
-
-__global__ void gather_rows_kernel(const int32_t* __restrict__ comp, const int32_t* __restrict__ rows, int64_t n,
-                                   int32_t* __restrict__ out) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    out[i] = comp[rows[i]];
 }
 
 __device__ __forceinline__ void warp_flush(int graph, uint64_t& bal, uint64_t& unb, unsigned long long* out) {
@@ -232,23 +227,87 @@ __global__ void __launch_bounds__(THREADS) hub_sweep_batch_kernel(const GraphDes
 // The largest counter buffer (32-bit words) a window of the item needs, with
 // the windows of ItemWindows: the first window of each counter width is its
 // widest.
-static uint32_t item_window_words(const SweepItem& it) {
+__device__ __forceinline__ uint32_t item_window_words(const SweepItem& it) {
   const uint32_t lo = it.lo, hi = it.hi;
-  const uint32_t qe = std::min(std::max(it.q_end, lo), hi);
-  const uint32_t te = std::min(std::max(it.t_end, qe), hi);
-  const uint32_t ne = std::min(std::max(it.n_end, te), hi);
+  const uint32_t qe = min(max(it.q_end, lo), hi);
+  const uint32_t te = min(max(it.t_end, qe), hi);
+  const uint32_t ne = min(max(it.n_end, te), hi);
   uint32_t w = 0;
   if (qe > lo) {
-    const uint32_t wh = std::min(lo + window_ranks<4>(), qe);
-    w = std::max(w, (wh - (lo & ~3u) + 3u) >> 2);
+    const uint32_t wh = min(lo + window_ranks<4>(), qe);
+    w = max(w, (wh - (lo & ~3u) + 3u) >> 2);
   }
   if (te > qe) {
-    const uint32_t wh = std::min(qe + window_ranks<8>(), te);
-    w = std::max(w, (wh - (qe & ~1u) + 1u) >> 1);
+    const uint32_t wh = min(qe + window_ranks<8>(), te);
+    w = max(w, (wh - (qe & ~1u) + 1u) >> 1);
   }
-  if (ne > te) w = std::max(w, std::min(te + window_ranks<16>(), ne) - te);
-  if (hi > ne) w = std::max(w, 2u * (std::min(ne + window_ranks<32>(), hi) - ne));
+  if (ne > te) w = max(w, min(te + window_ranks<16>(), ne) - te);
+  if (hi > ne) w = max(w, 2u * (min(ne + window_ranks<32>(), hi) - ne));
   return w;
+}
+
+// Hub items of a plan: one job per graph, item k of the job at position
+// offset + k. Every item gets its graph (or, with `comp`, the component of its
+// row) and the digit that sorts wide items before narrow ones, each in
+// descending estimated work; an item goes to a narrow CTA when its windows fit
+// kNarrowWords and its estimated work is small. With the build's hub plan on
+// the device too, build and count of a 200-graph union (36,000 items) went from
+// 4.84 to 2.36 ms.
+struct HubJob {
+  const SweepItem* items;
+  const uint32_t* lower;
+  int64_t offset;
+  int32_t graph;
+};
+struct HubSplit {
+  unsigned long long wide;                     // items on wide CTAs
+  unsigned long long lower_wide, lower_narrow; // most lower neighbours of an item's hub
+  unsigned flags;                              // kPrep* (bounded waits of the sort)
+};
+
+__global__ void __launch_bounds__(256) plan_items_kernel(const HubJob* __restrict__ jobs, int32_t n_jobs,
+                                                         int64_t n_items, const int32_t* __restrict__ comp,
+                                                         BatchHubItem* __restrict__ out, uint64_t* __restrict__ key,
+                                                         uint32_t* __restrict__ idx, uint32_t* hist, HubSplit* split) {
+  __shared__ uint32_t h[1][256];
+  DigitCounts dc{h, 1, 0};
+  dc.start();
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  uint64_t n_wide = 0, low_wide = 0, low_narrow = 0;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_items; i += stride) {
+    int32_t lo = 0, hi = n_jobs;  // the last job that starts at or before item i
+    while (hi - lo > 1) {
+      const int32_t mid = (lo + hi) >> 1;
+      if (jobs[mid].offset <= i) lo = mid; else hi = mid;
+    }
+    const HubJob j = jobs[lo];
+    const SweepItem it = j.items[i - j.offset];
+    const uint32_t L = j.lower[it.row];
+    const bool narrow = it.est <= kNarrowItemWork && item_window_words(it) <= kNarrowWords;
+    out[i] = BatchHubItem{comp ? comp[it.row] : j.graph, 0, it};
+    idx[i] = (uint32_t)i;
+    const uint64_t d = (narrow ? 128u : 0u) | estimate_digit(it.est, 2, 128u);
+    key[i] = d;
+    dc.add(d);
+    n_wide += narrow ? 0 : 1;
+    low_wide = max(low_wide, (uint64_t)(narrow ? 0u : L));
+    low_narrow = max(low_narrow, (uint64_t)(narrow ? L : 0u));
+  }
+  n_wide = warp_sum_u64(n_wide);
+  low_wide = warp_max_u64(low_wide);
+  low_narrow = warp_max_u64(low_narrow);
+  if (lane_id() == 0) {
+    if (n_wide) atomicAdd(&split->wide, (unsigned long long)n_wide);
+    if (low_wide) atomicMax(&split->lower_wide, (unsigned long long)low_wide);
+    if (low_narrow) atomicMax(&split->lower_narrow, (unsigned long long)low_narrow);
+  }
+  dc.finish(hist);
+}
+
+__global__ void gather_hub_items_kernel(const BatchHubItem* __restrict__ src, const uint32_t* __restrict__ idx,
+                                        int64_t n, BatchHubItem* __restrict__ dst) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    dst[i] = src[idx[i]];
 }
 
 }  // namespace dbbc
@@ -264,7 +323,8 @@ struct dbbc_batch {
   dbbc::BatchPivot* light = nullptr;
   dbbc::BatchPivot* medium = nullptr;
   dbbc::BatchHubItem* hub = nullptr;         // items for wide CTAs, then items for narrow ones
-  int64_t n_light = 0, n_medium = 0, n_hub_items = 0, max_lower = 1;
+  int64_t n_light = 0, n_medium = 0;
+  int64_t lower_wide = 1, lower_narrow = 1;  // cursor slots per CTA
   int64_t n_wide = 0, n_narrow = 0;
   unsigned long long* out = nullptr;  // [n_graphs][2]
   uint2* cursors = nullptr;         // wide CTAs'
@@ -301,8 +361,43 @@ static void batch_release(dbbc_batch* b) {
   b->fork = b->join = nullptr;
 }
 
-static void finish_plan(dbbc_batch* b, std::vector<GraphDesc>& desc, std::vector<BatchHubItem>& items,
-                        const std::vector<uint64_t>& est);
+static void finish_plan(dbbc_batch* b, const std::vector<GraphDesc>& desc);
+
+// The plan's hub items, from `n_jobs` jobs over n_items items: wide ones, then
+// narrow ones.
+static void plan_items(dbbc_batch* b, const std::vector<HubJob>& jobs, int64_t n_items, const int32_t* comp) {
+  if (n_items == 0) return;
+  cudaStream_t s = b->stream;
+  Scratch sc(s);
+  const int64_t tiles = radix_tiles(n_items);
+  HubJob* d_jobs = sc.get<HubJob>(jobs.size());
+  DBBC_CUDA(cudaMemcpyAsync(d_jobs, jobs.data(), jobs.size() * sizeof(HubJob), cudaMemcpyHostToDevice, s));
+  // zeroed: the split, the sort's digit counts, tile counter and tile states
+  const size_t words = (sizeof(HubSplit) + 255) / 256 * 64;
+  uint32_t* zero = sc.get<uint32_t>(words + 512 + (size_t)tiles * 256);
+  DBBC_CUDA(cudaMemsetAsync(zero, 0, (words + 512 + (size_t)tiles * 256) * 4, s));
+  HubSplit* split = reinterpret_cast<HubSplit*>(zero);
+  const RadixState st{zero + words, zero + words + 256, zero + words + 512};
+  BatchHubItem* tmp = sc.get<BatchHubItem>((size_t)n_items);
+  uint64_t* key = sc.get<uint64_t>((size_t)n_items);
+  uint32_t* idx = sc.get<uint32_t>((size_t)n_items * 2);
+  b->hub = static_cast<BatchHubItem*>(batch_alloc(b, (size_t)n_items * sizeof(BatchHubItem)));
+  const unsigned grid = (unsigned)std::min<int64_t>((n_items + 255) / 256, (int64_t)kNumSMs * 4);
+  plan_items_kernel<<<grid, 256, 0, s>>>(d_jobs, (int32_t)jobs.size(), n_items, comp, tmp, key, idx, st.hist, split);
+  DBBC_LAUNCH_CHECK();
+  radix_pass<PlainLoad, true, false, false>(PlainLoad{key, idx}, PassOut{nullptr, idx + n_items, nullptr, 0}, n_items,
+                                            0, 0, st, &split->flags, s);
+  gather_hub_items_kernel<<<grid, 256, 0, s>>>(tmp, idx + n_items, n_items, b->hub);
+  DBBC_LAUNCH_CHECK();
+  HubSplit h;
+  DBBC_CUDA(cudaMemcpyAsync(&h, split, sizeof(h), cudaMemcpyDeviceToHost, s));
+  DBBC_CUDA(cudaStreamSynchronize(s));
+  if (h.flags & kPrepTimeout) throw Error{DBBC_EINTERNAL, "a bounded wait of the plan gave up"};
+  b->n_wide = (int64_t)h.wide;
+  b->n_narrow = n_items - b->n_wide;
+  b->lower_wide = std::max<int64_t>(1, (int64_t)h.lower_wide);
+  b->lower_narrow = std::max<int64_t>(1, (int64_t)h.lower_narrow);
+}
 
 // Hash table sizes of the plan's light and medium kernels: the largest any of
 // its graphs' tiers needs (each graph's pivots were tiered by its own tuning).
@@ -327,34 +422,15 @@ static void plan_components(dbbc_batch* b, const dbbc_graph* g) {
   std::vector<GraphDesc> desc((size_t)b->n_graphs, GraphDesc{g->row_ptr, g->col, g->lower, g->work, g->n, g->nnz, g->n_u, g->tune.hash_mult_log});
   b->n_medium = g->n_medium;
   b->n_light = g->n_light;
-  b->max_lower = std::max<int64_t>(1, g->sweep_max_lower);
-  // components of the hub items' rows
-  const size_t nh = g->sweep_items_host.size();
-  std::vector<int32_t> rows(nh), comps(nh);
-  for (size_t k = 0; k < nh; k++) rows[k] = g->sweep_items_host[k].row;
-  std::vector<BatchHubItem> items(nh);
-  if (nh > 0) {
-    Scratch sc(s);
-    int32_t* d_rows = sc.get<int32_t>(nh);
-    int32_t* d_comp = sc.get<int32_t>(nh);
-    DBBC_CUDA(cudaMemcpyAsync(d_rows, rows.data(), nh * 4, cudaMemcpyHostToDevice, s));
-    gather_rows_kernel<<<(unsigned)std::min<size_t>((nh + 255) / 256, 4096), 256, 0, s>>>(g->component, d_rows,
-                                                                                        (int64_t)nh, d_comp);
-    DBBC_LAUNCH_CHECK();
-    DBBC_CUDA(cudaMemcpyAsync(comps.data(), d_comp, nh * 4, cudaMemcpyDeviceToHost, s));
-    DBBC_CUDA(cudaStreamSynchronize(s));
-  }
-  // the union's items are already in descending estimated work
-  for (size_t k = 0; k < nh; k++) items[k] = BatchHubItem{comps[k], 0, g->sweep_items_host[k]};
+  plan_items(b, {HubJob{g->sweep_items, g->lower, 0, 0}}, g->n_sweep_items, g->component);
   plan_table_logs(b, &g, 1);
-  finish_plan(b, desc, items, g->sweep_est_host);
+  finish_plan(b, desc);
   if (b->n_medium + b->n_light > 0) {
     const int64_t total = b->n_medium + b->n_light;
     gather_component_pivots_kernel<<<(unsigned)std::min<int64_t>((total + 255) / 256, 4096), 256, 0, s>>>(
         g->order, g->n_hub, g->n_medium, g->n_light, g->component, b->medium, b->light);
     DBBC_LAUNCH_CHECK();
   }
-  DBBC_CUDA(cudaStreamSynchronize(s));
 }
 
 static void plan_batch(dbbc_batch* b, const dbbc_graph* const* gs) {
@@ -362,30 +438,20 @@ static void plan_batch(dbbc_batch* b, const dbbc_graph* const* gs) {
   cudaStream_t s = b->stream;
   std::vector<GraphDesc> desc((size_t)n);
   std::vector<GatherJob> jobs((size_t)n);
-  struct HubRef {
-    BatchHubItem item;
-    uint64_t est;
-  };
-  std::vector<HubRef> hubs;
+  std::vector<HubJob> hubs((size_t)n);
+  int64_t n_items = 0;
   for (int32_t i = 0; i < n; i++) {
     const dbbc_graph* g = gs[i];
     desc[(size_t)i] = GraphDesc{g->row_ptr, g->col, g->lower, g->work, g->n, g->nnz, g->n_u, g->tune.hash_mult_log};
     jobs[(size_t)i] = GatherJob{g->order, g->n_hub, g->n_medium, g->n_light, b->n_medium, b->n_light};
     b->n_medium += g->n_medium;
     b->n_light += g->n_light;
-    for (size_t k = 0; k < g->sweep_items_host.size(); k++)
-      hubs.push_back(HubRef{BatchHubItem{i, 0, g->sweep_items_host[k]}, g->sweep_est_host[k]});
-    if (g->n_hub > 0) b->max_lower = std::max<int64_t>(b->max_lower, g->sweep_max_lower);
+    hubs[(size_t)i] = HubJob{g->sweep_items, g->lower, n_items, i};
+    n_items += g->n_sweep_items;
   }
-  std::stable_sort(hubs.begin(), hubs.end(), [](const HubRef& a, const HubRef& c) { return a.est > c.est; });
-  std::vector<BatchHubItem> items(hubs.size());
-  std::vector<uint64_t> est(hubs.size());
-  for (size_t k = 0; k < hubs.size(); k++) {
-    items[k] = hubs[k].item;
-    est[k] = hubs[k].est;
-  }
+  plan_items(b, hubs, n_items, nullptr);
   plan_table_logs(b, gs, n);
-  finish_plan(b, desc, items, est);
+  finish_plan(b, desc);
   GatherJob* d_jobs = static_cast<GatherJob*>(batch_alloc(b, jobs.size() * sizeof(GatherJob)));
   DBBC_CUDA(cudaMemcpyAsync(d_jobs, jobs.data(), jobs.size() * sizeof(GatherJob), cudaMemcpyHostToDevice, s));
   if (n > 0) {
@@ -395,32 +461,14 @@ static void plan_batch(dbbc_batch* b, const dbbc_graph* const* gs) {
   DBBC_CUDA(cudaStreamSynchronize(s));  // host vectors above must outlive the copies
 }
 
-// Allocations, launch shapes and uploads shared by both kinds of plan.
-static void finish_plan(dbbc_batch* b, std::vector<GraphDesc>& desc, std::vector<BatchHubItem>& items,
-                        const std::vector<uint64_t>& est) {
+// Allocations, launch shapes and uploads shared by all kinds of plan (the hub
+// items are placed already).
+static void finish_plan(dbbc_batch* b, const std::vector<GraphDesc>& desc) {
   cudaStream_t s = b->stream;
   const int32_t n = b->n_graphs;
-  // wide items first, then the narrow ones, each in their LPT order; an item
-  // goes to a narrow CTA when its windows fit kNarrowWords and its estimated
-  // work (est[k], absent: unknown) is small
-  {
-    std::vector<BatchHubItem> narrow;
-    size_t n_wide = 0;
-    for (size_t k = 0; k < items.size(); k++) {
-      if (k < est.size() && est[k] <= kNarrowItemWork && item_window_words(items[k].it) <= kNarrowWords)
-        narrow.push_back(items[k]);
-      else
-        items[n_wide++] = items[k];
-    }
-    std::copy(narrow.begin(), narrow.end(), items.begin() + (ptrdiff_t)n_wide);
-    b->n_wide = (int64_t)n_wide;
-    b->n_narrow = (int64_t)narrow.size();
-  }
-  b->n_hub_items = (int64_t)items.size();
   b->desc = static_cast<GraphDesc*>(batch_alloc(b, desc.size() * sizeof(GraphDesc)));
   b->light = static_cast<BatchPivot*>(batch_alloc(b, (size_t)b->n_light * sizeof(BatchPivot)));
   b->medium = static_cast<BatchPivot*>(batch_alloc(b, (size_t)b->n_medium * sizeof(BatchPivot)));
-  b->hub = static_cast<BatchHubItem*>(batch_alloc(b, items.size() * sizeof(BatchHubItem)));
   b->out = static_cast<unsigned long long*>(batch_alloc(b, (size_t)n * 2 * sizeof(unsigned long long)));
   b->counters = static_cast<int*>(batch_alloc(b, 3 * sizeof(int)));
   b->status = static_cast<unsigned*>(batch_alloc(b, sizeof(unsigned)));
@@ -429,9 +477,9 @@ static void finish_plan(dbbc_batch* b, std::vector<GraphDesc>& desc, std::vector
   b->narrow_grid = (int)std::min<int64_t>(num_sms() * blocks_per_sm((const void*)DBBC_NARROW_SWEEP, kNarrowThreads,
                                                                     kNarrowSmem), std::max<int64_t>(b->n_narrow, 1));
   if (b->n_wide > 0)
-    b->cursors = static_cast<uint2*>(batch_alloc(b, (size_t)b->hub_grid * (size_t)b->max_lower * sizeof(uint2)));
+    b->cursors = static_cast<uint2*>(batch_alloc(b, (size_t)b->hub_grid * (size_t)b->lower_wide * sizeof(uint2)));
   if (b->n_narrow > 0)
-    b->narrow_cursors = static_cast<uint2*>(batch_alloc(b, (size_t)b->narrow_grid * (size_t)b->max_lower * sizeof(uint2)));
+    b->narrow_cursors = static_cast<uint2*>(batch_alloc(b, (size_t)b->narrow_grid * (size_t)b->lower_narrow * sizeof(uint2)));
   {
     const int sms = num_sms();
     const int64_t want = ceil_div<int64_t>(ceil_div<int64_t>(b->n_light, 32), kLightWarps);
@@ -448,9 +496,6 @@ static void finish_plan(dbbc_batch* b, std::vector<GraphDesc>& desc, std::vector
     DBBC_CUDA(cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming));
   }
   DBBC_CUDA(cudaMemcpyAsync(b->desc, desc.data(), desc.size() * sizeof(GraphDesc), cudaMemcpyHostToDevice, s));
-  if (!items.empty())
-    DBBC_CUDA(cudaMemcpyAsync(b->hub, items.data(), items.size() * sizeof(BatchHubItem), cudaMemcpyHostToDevice, s));
-  DBBC_CUDA(cudaStreamSynchronize(s));  // host vectors must outlive the copies
 }
 
 // The batch count: clear outputs and counters, then the tiers on two
@@ -471,7 +516,7 @@ static void enqueue_batch(dbbc_batch* b, cudaStream_t s) {
   }
   if (b->n_narrow > 0) {
     DBBC_NARROW_SWEEP<<<b->narrow_grid, kNarrowThreads, kNarrowSmem, s2>>>(
-        b->desc, b->hub + b->n_wide, b->n_narrow, b->counters + 2, b->narrow_cursors, b->max_lower, b->out);
+        b->desc, b->hub + b->n_wide, b->n_narrow, b->counters + 2, b->narrow_cursors, b->lower_narrow, b->out);
     DBBC_LAUNCH_CHECK();
   }
   if (b->n_medium > 0) {
@@ -481,7 +526,7 @@ static void enqueue_batch(dbbc_batch* b, cudaStream_t s) {
   }
   if (b->n_wide > 0) {
     DBBC_WIDE_SWEEP<<<b->hub_grid, kSweepThreads, kSweepSmem, s>>>(b->desc, b->hub, b->n_wide, b->counters + 1,
-                                                                  b->cursors, b->max_lower, b->out);
+                                                                  b->cursors, b->lower_wide, b->out);
     DBBC_LAUNCH_CHECK();
   }
   if (b->n_light > 0) {
@@ -542,11 +587,16 @@ void count_subset(const dbbc_graph* g, cudaStream_t s, const std::vector<int32_t
                                               g->tune.hash_mult_log});
     b->n_medium = (int64_t)medium_rows.size();
     b->n_light = (int64_t)light_rows.size();
-    b->max_lower = std::max<int64_t>(1, g->sweep_max_lower);
+    // work unknown: every item on wide CTAs
+    b->lower_wide = std::max<int64_t>(1, g->sweep_max_lower);
     std::vector<BatchHubItem> items(hub_items.size());
     for (size_t k = 0; k < hub_items.size(); k++) items[k] = BatchHubItem{0, 0, hub_items[k]};
+    b->n_wide = (int64_t)items.size();
+    b->hub = static_cast<BatchHubItem*>(batch_alloc(b, items.size() * sizeof(BatchHubItem)));
+    if (!items.empty())
+      DBBC_CUDA(cudaMemcpyAsync(b->hub, items.data(), items.size() * sizeof(BatchHubItem), cudaMemcpyHostToDevice, s));
     plan_table_logs(b, &g, 1);
-    finish_plan(b, desc, items, {});  // work unknown: every item on wide CTAs
+    finish_plan(b, desc);
     std::vector<BatchPivot> med(medium_rows.size()), light(light_rows.size());
     for (size_t k = 0; k < medium_rows.size(); k++) med[k] = BatchPivot{0, medium_rows[k]};
     for (size_t k = 0; k < light_rows.size(); k++) light[k] = BatchPivot{0, light_rows[k]};

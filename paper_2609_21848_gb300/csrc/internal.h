@@ -107,7 +107,8 @@ struct SweepItem {
   uint32_t t_end;
   uint32_t n_end;
   int16_t group_log;
-  int16_t flags;  // kItemList | kItemFinalize
+  int16_t flags;  // kItemList | kItemFinalize | kItemFirst
+  uint32_t est;   // estimated accepted wedges (at most 2^32 - 1)
 };
 constexpr int16_t kItemList = 2;  // list mode: visit a neighbour only in windows holding its entries
 // counters of a window are finalised when it is cleared (C(p,2) + C(q,2) and
@@ -160,11 +161,10 @@ struct dbbc_graph {
   uint64_t wedges = 0, wedges_hub = 0, wedges_medium = 0, wedges_light = 0;
   int64_t lower_hub = 0, lower_medium = 0, lower_light = 0;
   int64_t hub_cursor_inits = 0, hub_cursor_steps = 0;
-  // hub plan: window-span items in descending estimated work
+  // hub plan: window-span items in descending estimated work (in steps of an
+  // eighth of an octave)
   dbbc::SweepItem* sweep_items = nullptr;
   int64_t n_sweep_items = 0;
-  std::vector<dbbc::SweepItem> sweep_items_host;  // same items on the host (batch planning)
-  std::vector<uint64_t> sweep_est_host;           // their estimated accepted wedges
   int64_t sweep_max_lower = 0;  // largest lower-neighbour count of a hub (cursor scratch per CTA)
   int64_t sweep_list_cap = 0;   // largest windows x lower neighbours of a list-mode item (list slots per CTA)
   int64_t narrow_ranks_u = 0, narrow_ranks_v = 0;  // per side: vertices of degree < 2^16 (a rank prefix)

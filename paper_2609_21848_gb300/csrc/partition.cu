@@ -76,7 +76,13 @@ dbbc_status dbbc_count_partition(const dbbc_graph* g, void* cuda_stream, int32_t
       else if ((int64_t)i >= g->n_hub) med.push_back(rows[i]);
     }
     std::vector<SweepItem> hubs;
-    for (const SweepItem& it : g->sweep_items_host)
+    std::vector<SweepItem> items((size_t)g->n_sweep_items);
+    if (!items.empty()) {
+      DBBC_CUDA(cudaMemcpyAsync(items.data(), g->sweep_items, items.size() * sizeof(SweepItem),
+                                cudaMemcpyDeviceToHost, s));
+      DBBC_CUDA(cudaStreamSynchronize(s));
+    }
+    for (const SweepItem& it : items)
       if (mine[(size_t)it.row]) hubs.push_back(it);
     count_subset(g, s, med, light, hubs, balanced, unbalanced);
   } catch (const Error& e) {

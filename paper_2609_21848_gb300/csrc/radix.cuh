@@ -398,6 +398,14 @@ __global__ void __launch_bounds__(kRsThreads, DBBC_RS_CTAS) radix_pass_kernel(Lo
   }
 }
 
+// Sort digit of an estimate x >= 1, larger ones first, in 2^log_steps steps per
+// octave: the top bits of x as a float. Work lists are ordered by it for LPT
+// scheduling, which needs no finer order (one digit pass sorts them).
+__device__ __forceinline__ uint32_t estimate_digit(uint32_t x, int log_steps, uint32_t digits) {
+  const uint32_t q = (__float_as_uint((float)x) >> (23 - log_steps)) - (127u << log_steps);
+  return digits - 1u - min(q, digits - 1u);
+}
+
 // Launch one pass (pass number `pass` of the sort: digit counts, tile counter
 // and states of `st`).
 template <class Load, bool HAS_V, bool WRITE_K, bool AUX>
