@@ -11,19 +11,6 @@
 
 namespace dbbc {
 
-// Lemma 1 contribution of one wedge, from its endpoint counter just before the
-// increment (sym = p, asym = q): adding a symmetric wedge to (p, q) closes p
-// new balanced pairs (C(p+1,2) - C(p,2) = p) and q unbalanced ones ((p+1)q - pq);
-// an asymmetric wedge closes q balanced and p unbalanced ones. Summed over all
-// wedges this equals C(p,2) + C(q,2) and p*q per endpoint.
-__device__ __forceinline__ void wedge_contrib(unsigned long long old, unsigned long long inc, uint64_t& bal,
-                                              uint64_t& unb) {
-  const uint64_t p = old & 0xFFFFFFFFull, q = old >> 32;
-  const bool sym = inc == 1ull;
-  bal += sym ? p : q;
-  unb += sym ? q : p;
-}
-
 // Hash counters of the light and medium tiers: one 32-bit word per endpoint,
 // (asym << 16) | sym. A count never exceeds the pivot's accepted wedges, and
 // those are at most kMediumMaxWork in these tiers. One 32-bit shared atomic
@@ -243,7 +230,6 @@ constexpr int kMediumWarps = kMediumThreads / 32;
 // (asym << 16) | sym when the hub has fewer than 2^16 lower neighbours (no
 // count can exceed that), else (asym << 32) | sym.
 constexpr int kSweepThreads = DBBC_SWEEP_THREADS;
-constexpr int kSweepUnroll = DBBC_SWEEP_UNROLL;
 static_assert(kSweepWindow16 % 4 == 0, "window buffers are cleared 16 bytes at a time");
 
 // Clear the first `words` 32-bit words of a window (16 bytes per store; the
@@ -253,17 +239,6 @@ __device__ __forceinline__ void zero_words(uint32_t* w, uint32_t words) {
   uint4* q = reinterpret_cast<uint4*>(w);
   const uint32_t quads = (words + 3) >> 2;
   for (uint32_t j = threadIdx.x; j < quads; j += THREADS) q[j] = make_uint4(0u, 0u, 0u, 0u);
-}
-
-// x[u] = entry at position c + u*G + gl of a row ending at en, or ~0 past it.
-template <int G>
-__device__ __forceinline__ void load_chunk(const uint32_t* col, uint32_t c, uint32_t en, int gl,
-                                           uint32_t (&x)[kSweepUnroll]) {
-#pragma unroll
-  for (int u = 0; u < kSweepUnroll; u++) {
-    const uint32_t off = (uint32_t)(u * G + gl);
-    x[u] = en - c > off ? __ldg(col + c + off) : 0xFFFFFFFFu;
-  }
 }
 
 // Counter widths of a window. CW = 16: one 32-bit word per endpoint packing
@@ -278,23 +253,17 @@ __host__ __device__ constexpr uint32_t window_ranks() {
   return CW == 4 ? 4 * kSweepWindow16 : CW == 8 ? 2 * kSweepWindow16 : CW == 16 ? kSweepWindow16 : kSweepWindow32;
 }
 
-template <int CW>
-__device__ __forceinline__ uint32_t window_words(uint32_t ranks) {  // 32-bit words holding `ranks` counters
-  return CW == 8 ? (ranks + 1) >> 1 : CW == 16 ? ranks : 2 * ranks;
-}
-
 // The windows of a work item: quarter ones over [lo, qe), tiny ones over
 // [qe, te), narrow ones over [te, ne), wide ones over [ne, hi), numbered in
-// rank order. `quarter` false folds the quarter part into the tiny one (for
-// sweeps that have no 4-bit counters).
+// rank order.
 struct ItemWindows {
   uint32_t lo, qe, te, ne, hi;
   uint32_t rq, rt, rn, rw;
   ItemWindows() = default;
-  __device__ __forceinline__ explicit ItemWindows(const SweepItem& it, bool quarter = true) {
+  __device__ __forceinline__ explicit ItemWindows(const SweepItem& it) {
     lo = it.lo;
     hi = it.hi;
-    qe = quarter ? min(max(it.q_end, lo), hi) : lo;
+    qe = min(max(it.q_end, lo), hi);
     te = min(max(it.t_end, qe), hi);
     ne = min(max(it.n_end, te), hi);
     rq = (qe - lo + window_ranks<4>() - 1) / window_ranks<4>();
@@ -331,97 +300,6 @@ struct ItemWindows {
     return rq + rt + rn + (x - ne) / window_ranks<32>();
   }
 };
-
-// Add one wedge (endpoint counter k, asym = the two edge signs differ) when
-// `ok`, and accumulate its Lemma 1 contribution from the counter's old value:
-// the old count of the wedge's own class (B1 for a symmetric wedge, B2 for an
-// asymmetric one) closes balanced butterflies and the other class unbalanced
-// ones. Packed counters are rotated for an asymmetric wedge so that its own
-// class sits in the low half. Narrow widths sum into 32-bit accumulators (a
-// segment adds fewer than 2^32 to each); the 64-bit width adds directly.
-template <int CW>
-__device__ __forceinline__ void add_wedge(bool ok, uint32_t k, uint32_t asym, uint32_t* c16, unsigned long long* c32,
-                                          uint32_t& acc_same, uint32_t& acc_other, uint64_t& bal, uint64_t& unb) {
-  if (ok && !DBBC_CHECK(k < window_ranks<CW>())) ok = false;
-  if (CW == 8) {
-    const uint32_t wsh = (k & 1u) << 4;  // which half of the word
-    uint32_t old = 0;
-    if (ok) old = atomicAdd(&c16[k >> 1], (asym ? 0x100u : 1u) << wsh);
-    const uint32_t v = (old >> wsh) & 0xFFFFu;            // (asym << 8) | sym
-    const uint32_t r = ((v << 16) | v) >> (asym << 3);  // own class in the low byte
-    acc_same += r & 0xFFu;
-    acc_other += (r >> 8) & 0xFFu;
-  } else if (CW == 16) {
-    const uint32_t sh = asym << 4;
-    uint32_t old = 0;
-    if (ok) old = atomicAdd(&c16[k], 1u << sh);
-    const uint32_t v = __funnelshift_l(old, old, sh);  // (other class << 16) | own class
-    acc_same += v & 0xFFFFu;
-    acc_other += v >> 16;
-  } else {
-    const unsigned long long inc = asym ? (1ull << 32) : 1ull;
-    unsigned long long old = 0;
-    if (ok) old = atomicAdd(&c32[k], inc);
-    wedge_contrib(old, inc, bal, unb);  // adds nothing when old == 0
-  }
-}
-
-// A group of G lanes walks one neighbour's entries inside the window [lo,
-// hl >> 1) from cursor c (the first chunk already in x) and returns the cursor
-// past the window. Entries of the window are a prefix of what is left of the
-// row, so the group stops at the first chunk that is not full. All groups of a
-// warp run the loop in lockstep until the last of them is done (warp-wide
-// votes, the atomic the only predicated step), which keeps the warp converged;
-// a group that is not `active` (no neighbour) only votes. Contributions of
-// the narrow widths are summed per segment in 32 bits (add_wedge).
-template <int G, int CW>
-__device__ __forceinline__ uint32_t walk_segment(const uint32_t* col, uint32_t c, uint32_t en, uint32_t s1,
-                                                 uint32_t (&x)[kSweepUnroll], uint32_t lo2, uint32_t hl, int gl,
-                                                 bool active, uint32_t* c16, unsigned long long* c32,
-                                                 uint64_t& bal, uint64_t& unb) {
-  const unsigned gshift = lane_id() & ~(unsigned)(G - 1);
-  const unsigned gbits = G == 32 ? kFullMask : (1u << G) - 1u;
-  uint32_t acc_same = 0, acc_other = 0;
-  for (;;) {
-    int n_ok = 0;
-#pragma unroll
-    for (int u = 0; u < kSweepUnroll; u++) {
-      const bool ok = active && x[u] < hl;
-      const uint32_t asym = (x[u] ^ s1) & 1u;
-      const uint32_t k = (x[u] - lo2) >> 1;
-      add_wedge<CW>(ok, k, asym, c16, c32, acc_same, acc_other, bal, unb);
-      n_ok += __popc((__ballot_sync(kFullMask, ok) >> gshift) & gbits);
-    }
-    c += (uint32_t)n_ok;
-    active = active && n_ok == G * kSweepUnroll;
-    if (!__any_sync(kFullMask, active)) break;
-    if (active) load_chunk<G>(col, c, en, gl, x);
-  }
-  bal += acc_same;
-  unb += acc_other;
-  return c;
-}
-
-// Cursors of an item: the first entry of each lower neighbour's row at or
-// after rank `lo_rank`, and the row end.
-__device__ __forceinline__ void init_cursor(const CsrView& g, const PivotGeom& q, uint32_t i, uint32_t lo_rank,
-                                            uint32_t* cur, uint32_t& b_out, uint32_t& en_out) {
-  int64_t b, en;
-  neighbour_row(g, q, g.col[q.rb + i], b, en);
-  const uint32_t first = lo_rank << 1;
-  if (first) {  // lower_bound of `first` in the row
-    int64_t lo = b, hi = en;
-    while (lo < hi) {
-      const int64_t mid = (lo + hi) >> 1;
-      if (g.col[mid] < first) lo = mid + 1; else hi = mid;
-    }
-    b = lo;
-  }
-  b_out = (uint32_t)b;
-  en_out = (uint32_t)en;
-  cur[2 * i] = b_out;
-  cur[2 * i + 1] = en_out;
-}
 
 inline int blocks_per_sm(const void* fn, int threads, size_t smem) {
   int b = 0;

@@ -26,11 +26,6 @@ constexpr int kMediumSlots = 8192;
 #ifndef DBBC_SWEEP_THREADS
 #define DBBC_SWEEP_THREADS 1024
 #endif
-// entries per lane per chunk of the per-vertex / per-edge window walks (4
-// measured 5% faster than 2 on GB300)
-#ifndef DBBC_SWEEP_UNROLL
-#define DBBC_SWEEP_UNROLL 4
-#endif
 constexpr uint32_t kSweepWindow16 = DBBC_SWEEP_WINDOW16;     // 32-bit counters packing two 16-bit halves
 constexpr uint32_t kSweepWindow32 = DBBC_SWEEP_WINDOW16 / 2;  // 64-bit counters packing two 32-bit halves
 constexpr uint64_t kSweepItemWork = 1u << 20;  // target accepted wedges per work item
@@ -167,10 +162,7 @@ struct dbbc_graph {
   int64_t n_sweep_items = 0;
   int64_t sweep_max_lower = 0;  // largest lower-neighbour count of a hub (cursor scratch per CTA)
   int64_t sweep_list_cap = 0;   // largest windows x lower neighbours of a list-mode item (list slots per CTA)
-  int64_t narrow_ranks_u = 0, narrow_ranks_v = 0;  // per side: vertices of degree < 2^16 (a rank prefix)
-  int64_t tiny_ranks_u = 0, tiny_ranks_v = 0;      // per side: vertices of degree < 2^8 (a rank prefix)
-  int64_t quarter_ranks_u = 0, quarter_ranks_v = 0;  // per side: vertices of degree < 2^4 (a rank prefix)
-  int64_t zero_ranks_u = 0, zero_ranks_v = 0;      // per side: vertices of degree 0 (a rank prefix; no row lists them)
+  int64_t max_deg_u = 0, max_deg_v = 0;            // largest degree of each side
   // disjoint union of several graphs (dbbc_graph_from_coo_multi): component
   // of every row, 0 for a plain handle (n_components == 1)
   int32_t n_components = 1;

@@ -314,13 +314,15 @@ struct CsrKeys {
 // are a prefix.
 // The last CTA instead finds, per side, how many vertices have degree below
 // each of four limits (ranks ascend by degree within a side): below[2k] for U,
-// below[2k + 1] for V.
+// below[2k + 1] for V; and the largest degree, that of some component's last
+// rank.
 struct DegreeLimits {
   int32_t d[4];
 };
 __global__ void lower_kernel(const int64_t* __restrict__ row_ptr, const uint32_t* __restrict__ col,
                              const int32_t* __restrict__ rowdeg, int64_t n, int32_t n_u, UnionView un,
-                             uint32_t* __restrict__ lower, DegreeLimits lim, int64_t* below, const unsigned* flags) {
+                             uint32_t* __restrict__ lower, DegreeLimits lim, int64_t* below,
+                             unsigned* max_deg, const unsigned* flags) {
   if (cta_stopped(flags)) return;
   if (blockIdx.x == gridDim.x - 1) {
     const int t = threadIdx.x;
@@ -328,6 +330,10 @@ __global__ void lower_kernel(const int64_t* __restrict__ row_ptr, const uint32_t
       const bool u = (t & 1) == 0;
       below[t] = u ? lower_bound_dev<int32_t>(rowdeg, n_u, lim.d[t >> 1])
                    : lower_bound_dev<int32_t>(rowdeg + n_u, n - n_u, lim.d[t >> 1]);
+    }
+    for (int32_t c = t; c < un.n_graphs; c += blockDim.x) {
+      if (un.uo(c + 1) > un.uo(c)) atomicMax(&max_deg[0], (unsigned)rowdeg[un.uo(c + 1) - 1]);
+      if (un.vo(c + 1) > un.vo(c)) atomicMax(&max_deg[1], (unsigned)rowdeg[n_u + un.vo(c + 1) - 1]);
     }
     return;
   }
@@ -429,6 +435,7 @@ struct PrepResult {
   PrepStats st;
   HubStats hubs;
   int64_t below[8];         // vertices of degree below four limits (lower_kernel)
+  unsigned max_deg[2];      // largest degree of each side (lower_kernel)
   unsigned long long kept;  // distinct edges (dedup_kernel)
   unsigned flags;           // kPrep*
 };
@@ -1036,7 +1043,7 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
     if (n > 0) {
       const DegreeLimits lim{{kNarrowCountLimit, kTinyCountLimit, kQuarterCountLimit, 1}};
       lower_kernel<<<grid_for(n) + 1, 256, 0, s>>>(g->row_ptr, g->col, l.rowdeg, n, n_u, uv, g->lower, lim,
-                                                   l.res->below, d_flags);
+                                                   l.res->below, l.res->max_deg, d_flags);
       DBBC_LAUNCH_CHECK();
       if (me > 0) {
         work_kernel<<<grid_for(me), 256, 0, s>>>(ck, g->row_ptr, g->lower,
@@ -1108,15 +1115,8 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
                                                  s);
     }
   }
-  // per side: how many vertices have degree < 2^16, < 2^8, < 2^4 and 0
-  g->narrow_ranks_u = r.below[0];
-  g->narrow_ranks_v = r.below[1];
-  g->tiny_ranks_u = r.below[2];
-  g->tiny_ranks_v = r.below[3];
-  g->quarter_ranks_u = r.below[4];
-  g->quarter_ranks_v = r.below[5];
-  g->zero_ranks_u = r.below[6];
-  g->zero_ranks_v = r.below[7];
+  g->max_deg_u = r.max_deg[0];
+  g->max_deg_v = r.max_deg[1];
   plan_hubs(g, s, uv, l.res, sc);
   if (read_back(d_flags, s) & kPrepTimeout) throw Error{DBBC_EINTERNAL, "a bounded wait of the build gave up"};
 }

@@ -13,15 +13,15 @@
 // are final. Vertex results are accumulated per CSR row and mapped to unified
 // ids at the end; edge results per CSR position (an edge has one position in
 // each of its two rows), summed over both positions when an edge is queried.
-#include "count_device.cuh"
+#include "sweep_device.cuh"
 
 namespace dbbc {
 
 struct TipOut {
   unsigned long long* vb = nullptr;  // [n] per row (vertex counts)
   unsigned long long* vu = nullptr;
-  unsigned long long* eb = nullptr;  // [nnz] per CSR position (edge counts)
-  unsigned long long* eu = nullptr;
+  unsigned long long* eb = nullptr;  // [nnz] per CSR position (edge counts); when no edge can be in 2^32
+  unsigned long long* eu = nullptr;  // butterflies, eu is null and eb holds (unbalanced << 32) | balanced
   int64_t n = 0, nnz = 0;            // their lengths
 };
 
@@ -64,7 +64,9 @@ __device__ __forceinline__ void add_vertex(const TipOut& o, int64_t r, uint64_t 
   if (DBBC_CHECK(r >= 0 && r < o.n)) add_pair(o.vb, o.vu, r, x, y);
 }
 __device__ __forceinline__ void add_edge(const TipOut& o, int64_t j, uint64_t x, uint64_t y) {
-  if (DBBC_CHECK(j >= 0 && j < o.nnz)) add_pair(o.eb, o.eu, j, x, y);
+  if (!DBBC_CHECK(j >= 0 && j < o.nnz)) return;
+  if (o.eu) add_pair(o.eb, o.eu, j, x, y);
+  else if (x | y) atomicAdd(&o.eb[j], (unsigned long long)(x | (y << 32)));
 }
 
 // The endpoints of a pivot's complete hash table (slots t, t + threads, ...):
@@ -198,79 +200,177 @@ __global__ void __launch_bounds__(kMediumThreads) tips_medium_kernel(CsrView g, 
 }
 
 // ------------------------------------------------------------------ hub windows
-// Counter k of a window of width CW (see add_wedge) as (asym << 32) | sym.
+// A hub window runs in three passes over shared-memory counters: the window is
+// counted (the counting sweep's walk without returned values), its endpoints
+// are credited, and the segments just counted are walked again for the middles
+// and the edges. The first pass lists the segments it finds, so the last one
+// visits only neighbours with entries in the window. Per-edge counts of the
+// 20M-edge rating graph: sweep 31.4 -> 19.8 ms (half of it from both counts of
+// an edge sharing one word, see dbbc_count_edges); it is bound by the latency
+// of its loads and of the far edges' adds, 1.2e9 sectors to L2. Per-vertex
+// counts of a 4M-edge one: 3.34 -> 2.26 ms, bound by issue slots (63%).
+
+// A neighbour's segment [c, end) inside the current window; e: its entry in
+// the hub's row, i: its position there.
+struct Segment {
+  uint32_t c, end, e, i;
+};
+
+// Shared byte address of the counter word of entry x's endpoint (see Win).
 template <int CW>
-__device__ __forceinline__ unsigned long long window_value(const uint32_t* c16, const unsigned long long* c32,
-                                                           uint32_t k) {
-  if (CW == 8) {
-    const uint32_t v = (c16[k >> 1] >> ((k & 1u) << 4)) & 0xFFFFu;
-    return ((unsigned long long)(v >> 8) << 32) | (v & 0xFFu);
-  }
-  if (CW == 16) {
-    const uint32_t v = c16[k];
-    return ((unsigned long long)(v >> 16) << 32) | (v & 0xFFFFu);
-  }
-  return c32[k];
+__device__ __forceinline__ uint32_t counter_addr(uint32_t x, uint32_t wb) {
+  return CW == 4 ? wb + ((x >> 1) & ~3u) : CW == 8 ? wb + (x & ~3u) : CW == 16 ? wb + ((x >> 1) << 2)
+                                                                               : wb + ((x >> 1) << 3);
+}
+__device__ __forceinline__ uint32_t lds_u32(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+  return v;
 }
 
-// One window of a hub item, in three passes over the item's lower
-// neighbours (lane groups of G as in the counting sweep, moving in warp
-// lockstep): count the window's wedges (each neighbour's cursor moves past
-// the window, its old value kept in `prev`), credit endpoints and the pivot
-// from the complete window, then walk every neighbour's segment
-// [prev, cursor) again for the middles and edges.
-template <int G, int CW, bool VERT, bool EDGE>
-__device__ __forceinline__ void tips_window(const CsrView& g, const PivotGeom& q, uint32_t* cur, uint32_t* prev, uint32_t lo,
-                            uint32_t hi, uint32_t* c16, unsigned long long* c32, const TipOut& o, uint64_t& pb,
-                            uint64_t& pu) {
-  const uint32_t hl = hi << 1, lo2 = lo << 1;
-  const int gl = threadIdx.x & (G - 1);
-  const uint32_t gid = threadIdx.x / G;
-  constexpr uint32_t groups = kSweepThreads / G;
-  const uint32_t* col = g.col;
-  uint64_t unused_b = 0, unused_u = 0;
-  for (uint32_t i = gid; __any_sync(kFullMask, i < q.L); i += groups) {
-    const bool active = i < q.L;
-    const uint32_t c = active ? cur[2 * i] : 0u, en = active ? cur[2 * i + 1] : 0u;
-    const uint32_t s1 = active ? col[q.rb + i] & 1u : 0u;
-    uint32_t x[kSweepUnroll];
-    load_chunk<G>(col, c, en, gl, x);
-    const uint32_t cn = walk_segment<G, CW>(col, c, en, s1, x, lo2, hl, gl, active, c16, c32, unused_b, unused_u);
-    if (active && gl == 0) {
-      prev[i] = c;
-      cur[2 * i] = cn;
+// Final counts of entry x's endpoint: of the wedge's own class and of the
+// other one.
+template <int CW>
+__device__ __forceinline__ void counter_pair(uint32_t x, uint32_t s1, const Win& w, uint32_t& own, uint32_t& other) {
+  const uint32_t addr = counter_addr<CW>(x, w.wb);
+  own = 1u;  // checked builds: an address outside the window credits nothing
+  other = 0u;
+#if DBBC_CHECKED
+  if (!DBBC_CHECK(x >= w.l && x < w.h && addr >= w.s_lo && addr + (CW == 32 ? 8u : 4u) <= w.s_hi)) return;
+#endif
+  if constexpr (CW == 32) {
+    const uint32_t asym = ((x ^ s1) & 1u) << 2;
+    own = lds_u32(addr + asym);
+    other = lds_u32(addr + (asym ^ 4u));
+  } else {
+    const uint32_t v = lds_u32(addr);
+    if constexpr (CW == 4) {
+      const uint32_t sel = (x ^ s1) & 7u;
+      own = (v >> (sel << 2)) & 0xFu;
+      other = (v >> ((sel ^ 1u) << 2)) & 0xFu;
+    } else if constexpr (CW == 8) {
+      const uint32_t sel = (x ^ s1) & 3u;
+      own = (v >> (sel << 3)) & 0xFFu;
+      other = (v >> ((sel ^ 1u) << 3)) & 0xFFu;
+    } else {
+      const uint32_t r = __funnelshift_l(v, v, ((x ^ s1) & 1u) << 4);
+      own = r & 0xFFFFu;
+      other = r >> 16;
     }
   }
-  __syncthreads();
-  if (VERT) {
-    const int64_t end_base = q.base == 0 ? (int64_t)g.n_u : 0;  // endpoints share the pivot's side
-    for (uint32_t k = threadIdx.x; k < hi - lo; k += kSweepThreads) {
-      const unsigned long long v = window_value<CW>(c16, c32, k);
-      if (v) {
-        uint64_t eb = 0, eu = 0;
-        endpoint_contrib(v, eb, eu);
-        add_vertex(o, end_base + lo + k, eb, eu);
-        pb += eb;
-        pu += eu;
+}
+
+// Second pass: every endpoint of the window, and the pivot, get the endpoint's
+// Lemma 1 totals. A thread takes whole counter words, most of which hold no
+// endpoint in a butterfly (an endpoint is in one from two wedges on).
+template <int CW>
+__device__ __forceinline__ void credit_window(const uint32_t* words, const Win& w, uint32_t wlo, uint32_t whi,
+                                              int64_t end_base, const TipOut& o, uint64_t& pb, uint64_t& pu) {
+  auto endpoint = [&](uint32_t rank, uint32_t p, uint32_t q) {
+    if (p + q < 2u) return;
+    uint64_t eb, eu;
+    if (CW <= 8) {
+      eb = (p * (p - (p > 0u)) + q * (q - (q > 0u))) >> 1;
+      eu = p * q;
+    } else {
+      eb = eu = 0;
+      endpoint_contrib(((unsigned long long)q << 32) | p, eb, eu);
+    }
+    add_vertex(o, end_base + rank, eb, eu);
+    pb += eb;
+    pu += eu;
+  };
+  if constexpr (CW == 32) {
+    for (uint32_t k = threadIdx.x; k < whi - wlo; k += kSweepThreads) endpoint(wlo + k, words[2 * k], words[2 * k + 1]);
+  } else {
+    const uint32_t first = CW == 4 ? wlo & ~3u : CW == 8 ? wlo & ~1u : wlo;  // rank of word 0's first counter
+    for (uint32_t k = threadIdx.x; k < w.words; k += kSweepThreads) {
+      const uint32_t v = words[k];
+      if (v == 0u) continue;
+      if constexpr (CW == 16) {
+        endpoint(first + k, v & 0xFFFFu, v >> 16);
+      } else if constexpr (CW == 8) {
+        endpoint(first + 2 * k, v & 0xFFu, (v >> 8) & 0xFFu);
+        endpoint(first + 2 * k + 1, (v >> 16) & 0xFFu, v >> 24);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; j++) endpoint(first + 4 * k + j, (v >> (8 * j)) & 0xFu, (v >> (8 * j + 4)) & 0xFu);
       }
     }
   }
-  for (uint32_t i = gid; __any_sync(kFullMask, i < q.L); i += groups) {
-    const bool active = i < q.L;
-    const uint32_t c0 = active ? prev[i] : 0u, c1 = active ? cur[2 * i] : 0u;
-    const uint32_t e = active ? col[q.rb + i] : 0u;
-    const uint32_t s1 = e & 1u;
-    const uint32_t trips = __reduce_max_sync(kFullMask, (c1 - c0 + G - 1) / G);
-    uint64_t sb = 0, su = 0;
-    for (uint32_t t = 0; t < trips; t++) {
-      const uint32_t pos = c0 + t * G + gl;
-      if (pos < c1) {
-        const uint32_t xx = col[pos];
-        uint64_t cb, cu;
-        wedge_pairs(window_value<CW>(c16, c32, (xx - lo2) >> 1), ((xx ^ s1) & 1u) == 0, cb, cu);
-        if (EDGE) add_edge(o, pos, cb, cu);
-        sb += cb;
-        su += cu;
+}
+
+// First pass: count all L neighbours' entries in the window; every neighbour
+// that has some moves its slot past them and joins the segment list.
+template <int G, int CW>
+__device__ __forceinline__ void tips_count(const CsrView& g, const PivotGeom& q, uint2* slots, uint32_t* next,
+                                           Segment* seg, uint32_t* n_seg, const Win& w) {
+  const int gl = threadIdx.x & (G - 1);
+  uint64_t unused_b = 0, unused_u = 0;
+  SlotBatch sb;
+  LaneBatch b;
+  slot_fetch<G>(slots, q.L, next, sb);
+  batch_load<G>(g.col, sb, b);
+  while (b.base < q.L) {  // warp-uniform
+    const uint32_t i = b.base + lane_id() / G;
+    const uint32_t en = b.e.x + (b.e.y & 0x7FFFFFFFu);
+    uint32_t cn, xn;
+    if (lean_walk<G, CW, false>(g.col, b.e.x, en, b.e.y >> 31, b.x, w, gl, i < q.L, unused_b, unused_u, cn, xn) &&
+        i < q.L && cn != b.e.x) {
+      slots[i] = lean_slot(cn, en, b.e.y >> 31);
+      const uint32_t k = atomicAdd(n_seg, 1u);
+      if (DBBC_CHECK(k < q.L)) seg[k] = Segment{b.e.x, cn, g.col[q.rb + i], i};
+    }
+    __syncwarp();
+    slot_fetch<G>(slots, q.L, next, sb);
+    batch_load<G>(g.col, sb, b);
+  }
+}
+
+// Last pass: walk the n listed segments again. A wedge with own-class count p
+// and other-class count q is in p - 1 balanced and q unbalanced butterflies.
+// Sums of one segment fit 32 bits in the narrow widths (see lean_walk).
+template <int G, int CW, bool VERT, bool EDGE>
+__device__ __forceinline__ void tips_credit(const CsrView& g, const PivotGeom& q, const Segment* seg, uint32_t n,
+                                            uint32_t* next, const Win& w, const TipOut& o) {
+  using Sum = typename std::conditional<CW == 32, uint64_t, uint32_t>::type;
+  const uint32_t gl = threadIdx.x & (G - 1);
+  for (;;) {
+    uint32_t base = 0;
+    if (lane_id() == 0) base = atomicAdd(next, 32u / G);
+    base = __shfl_sync(kFullMask, base, 0);
+    if (base >= n) break;  // warp-uniform
+    const uint32_t k = base + lane_id() / G;
+    Segment t{0u, 0u, 0u, 0u};
+    if (k < n) t = seg[k];
+    const uint32_t s1 = t.e & 1u, len = t.end - t.c, start = t.c & ~3u;
+    const uint32_t chunks = (t.end - start + 4u * G - 1u) / (4u * G);
+    const uint32_t trips = __reduce_max_sync(kFullMask, chunks);
+    Sum sb = 0, su = 0;
+    // Edges: the group's lanes take consecutive entries, so that the adds to
+    // the far edges of G lanes fall into G / 4 sectors (four entries per lane
+    // would spread them over G sectors: 28.5 instead of 19.8 ms of sweep on the
+    // 20M-edge rating graph). Vertices: four entries per lane by one load.
+    constexpr uint32_t kLane = EDGE ? 1u : 4u, kItem = EDGE ? (uint32_t)G : 1u;
+    for (uint32_t j = 0; j < trips; j++) {
+      const uint32_t pos = start + j * (4u * G) + gl * kLane;
+      uint32_t x[kLU] = {0u, 0u, 0u, 0u};
+      if constexpr (EDGE) {
+#pragma unroll
+        for (int u = 0; u < kLU; u++)
+          if (pos + u * kItem < t.end) x[u] = __ldg(g.col + pos + u * kItem);
+      } else {
+        if (pos < t.end) lean_load(g.col, pos, x);
+      }
+#pragma unroll
+      for (int u = 0; u < kLU; u++) {
+        if (pos + u * kItem - t.c < len) {
+          uint32_t own, other;
+          counter_pair<CW>(x[u], s1, w, own, other);
+          if (EDGE) add_edge(o, pos + u * kItem, own - 1u, other);
+          sb += own - 1u;
+          su += other;
+        }
       }
     }
 #pragma unroll
@@ -278,44 +378,65 @@ __device__ __forceinline__ void tips_window(const CsrView& g, const PivotGeom& q
       sb += __shfl_xor_sync(kFullMask, sb, off);
       su += __shfl_xor_sync(kFullMask, su, off);
     }
-    if (active && gl == 0) {
-      if (VERT) add_vertex(o, q.base + (e >> 1), sb, su);
-      if (EDGE) add_edge(o, q.rb + i, sb, su);
+    if (k < n && gl == 0) {
+      if (VERT) add_vertex(o, q.base + (t.e >> 1), sb, su);
+      if (EDGE) add_edge(o, q.rb + t.i, sb, su);
     }
   }
+}
+
+// Block-uniform counters of the window being swept, in shared memory.
+struct TipsShared {
+  uint32_t next_count, next_credit, n_seg;
+};
+
+template <int G, int CW, bool VERT, bool EDGE>
+__device__ __forceinline__ void tips_window(const CsrView& g, const PivotGeom& q, uint2* slots, Segment* seg,
+                                            TipsShared& sh, uint32_t lo, uint32_t hi, uint32_t sbase, uint32_t* words,
+                                            const TipOut& o, uint64_t& pb, uint64_t& pu) {
+  const Win w = make_win(CW, lo, hi, sbase);
+  tips_count<G, CW>(g, q, slots, &sh.next_count, seg, &sh.n_seg, w);
   __syncthreads();
-  zero_words(c16, window_words<CW>(hi - lo));
+  if (VERT) {
+    credit_window<CW>(words, w, lo, hi, q.base == 0 ? (int64_t)g.n_u : 0, o, pb, pu);  // endpoints share the pivot's side
+  }
+  const uint32_t n = DBBC_CHECK(sh.n_seg <= q.L) ? sh.n_seg : q.L;
+  tips_credit<G, CW, VERT, EDGE>(g, q, seg, n, &sh.next_credit, w, o);
+  __syncthreads();
+  zero_words(words, w.words);
+  if (threadIdx.x == 0) sh = TipsShared{0u, 0u, 0u};
   __syncthreads();
 }
 
-template <int CW, bool VERT, bool EDGE>
-__device__ __forceinline__ void tips_window_dispatch(int group_log, const CsrView& g, const PivotGeom& q,
-                                                     uint32_t* cur, uint32_t* prev, uint32_t lo, uint32_t hi,
-                                                     uint32_t* c16, unsigned long long* c32, const TipOut& o,
-                                                     uint64_t& pb, uint64_t& pu) {
+template <int CW, bool VERT, bool EDGE, typename... A>
+__device__ __forceinline__ void tips_window_dispatch(int group_log, A&&... a) {
   switch (group_log) {
-    case 0: tips_window<1, CW, VERT, EDGE>(g, q, cur, prev, lo, hi, c16, c32, o, pb, pu); break;
-    case 2: tips_window<4, CW, VERT, EDGE>(g, q, cur, prev, lo, hi, c16, c32, o, pb, pu); break;
-    case 3: tips_window<8, CW, VERT, EDGE>(g, q, cur, prev, lo, hi, c16, c32, o, pb, pu); break;
-    case 4: tips_window<16, CW, VERT, EDGE>(g, q, cur, prev, lo, hi, c16, c32, o, pb, pu); break;
-    default: tips_window<32, CW, VERT, EDGE>(g, q, cur, prev, lo, hi, c16, c32, o, pb, pu); break;
+    case 0: tips_window<1, CW, VERT, EDGE>(a...); break;
+    case 2: tips_window<4, CW, VERT, EDGE>(a...); break;
+    case 3: tips_window<8, CW, VERT, EDGE>(a...); break;
+    case 4: tips_window<16, CW, VERT, EDGE>(a...); break;
+    default: tips_window<32, CW, VERT, EDGE>(a...); break;
   }
 }
 
+// Per CTA: cur_cap neighbour slots and cur_cap segments of scratch.
 template <bool VERT, bool EDGE>
 __global__ void __launch_bounds__(kSweepThreads, 1) tips_sweep_kernel(CsrView g, const SweepItem* __restrict__ items,
                                                                    int64_t n_items, int* next_item,
-                                                                   uint32_t* __restrict__ cursors, int64_t cur_cap,
+                                                                   uint2* __restrict__ cursors,
+                                                                   Segment* __restrict__ segments, int64_t cur_cap,
                                                                    TipOut o) {
   extern __shared__ __align__(16) unsigned char sweep_smem[];
-  uint32_t* c16 = reinterpret_cast<uint32_t*>(sweep_smem);
-  unsigned long long* c32 = reinterpret_cast<unsigned long long*>(sweep_smem);
+  uint32_t* words = reinterpret_cast<uint32_t*>(sweep_smem);
+  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sweep_smem);
   __shared__ int item_sh;
+  __shared__ TipsShared sh;
   __shared__ unsigned long long red[2][kSweepThreads / 32];
   const int tid = threadIdx.x;
-  zero_words(c16, kSweepWindow16);
-  uint32_t* cur = cursors + (int64_t)blockIdx.x * cur_cap * 3;  // [cur_cap][2] cursor and row end
-  uint32_t* prev = cur + 2 * cur_cap;                              // [cur_cap] cursor before the window
+  zero_words(words, kSweepWords);
+  if (tid == 0) sh = TipsShared{0u, 0u, 0u};
+  uint2* cur = cursors + (int64_t)blockIdx.x * cur_cap;
+  Segment* seg = segments + (int64_t)blockIdx.x * cur_cap;
   for (;;) {
     if (tid == 0) item_sh = atomicAdd(next_item, 1);
     __syncthreads();
@@ -325,10 +446,11 @@ __global__ void __launch_bounds__(kSweepThreads, 1) tips_sweep_kernel(CsrView g,
     const SweepItem item = items[it];
     PivotGeom q = pivot_geom(g, item.row);
     if (!DBBC_CHECK((int64_t)q.L <= cur_cap)) q.L = 0;  // checked builds: cursor capacity
-    const ItemWindows iw(item, false);  // this sweep has no 4-bit counters
+    const ItemWindows iw(item);
     for (uint32_t i = tid; i < q.L; i += kSweepThreads) {
-      uint32_t b, en;
-      init_cursor(g, q, i, (item.flags & kItemFirst) ? 0u : item.lo, cur, b, en);
+      uint32_t b, en, s1;
+      lean_cursor_start(g, q, i, (item.flags & kItemFirst) ? 0u : item.lo, b, en, s1);
+      cur[i] = lean_slot(b, en, s1);
     }
     __syncthreads();
     uint64_t pb = 0, pu = 0;
@@ -336,9 +458,11 @@ __global__ void __launch_bounds__(kSweepThreads, 1) tips_sweep_kernel(CsrView g,
       uint32_t lo, hi;
       int cw;
       iw.window(r, lo, hi, cw);
-      if (cw == 8) tips_window_dispatch<8, VERT, EDGE>(item.group_log, g, q, cur, prev, lo, hi, c16, c32, o, pb, pu);
-      else if (cw == 16) tips_window_dispatch<16, VERT, EDGE>(item.group_log, g, q, cur, prev, lo, hi, c16, c32, o, pb, pu);
-      else tips_window_dispatch<32, VERT, EDGE>(item.group_log, g, q, cur, prev, lo, hi, c16, c32, o, pb, pu);
+      const int gl = item.group_log;
+      if (cw == 4) tips_window_dispatch<4, VERT, EDGE>(gl, g, q, cur, seg, sh, lo, hi, sbase, words, o, pb, pu);
+      else if (cw == 8) tips_window_dispatch<8, VERT, EDGE>(gl, g, q, cur, seg, sh, lo, hi, sbase, words, o, pb, pu);
+      else if (cw == 16) tips_window_dispatch<16, VERT, EDGE>(gl, g, q, cur, seg, sh, lo, hi, sbase, words, o, pb, pu);
+      else tips_window_dispatch<32, VERT, EDGE>(gl, g, q, cur, seg, sh, lo, hi, sbase, words, o, pb, pu);
     }
     if (VERT) {  // the pivot's share of this item
       pb = warp_sum_u64(pb);
@@ -401,7 +525,12 @@ __global__ void edge_query_kernel(CsrView g, const int32_t* __restrict__ row_of,
       const int64_t p2 = find_in_row(g.col, g.row_ptr[rv], g.row_ptr[rv + 1], (uint32_t)ru);
       if (p1 >= 0 && p2 >= 0) {
         xb = eb[p1] + eb[p2];
-        xu = eu[p1] + eu[p2];
+        if (eu) {
+          xu = eu[p1] + eu[p2];
+        } else {  // both counts in one word, each below 2^32
+          xu = xb >> 32;
+          xb &= 0xFFFFFFFFull;
+        }
       }
     }
     ob[i] = xb;
@@ -439,14 +568,15 @@ void enqueue_tips(const dbbc_graph* g, cudaStream_t s, const TipOut& o, unsigned
   }
   if (g->n_hub > 0) {
     auto fn = tips_sweep_kernel<VERT, EDGE>;
-    const size_t smem = (size_t)kSweepWindow16 * 4;
+    const size_t smem = kSweepSmem;
     DBBC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     const int grid = sms * blocks_per_sm((const void*)fn, kSweepThreads, smem);
-    uint32_t* cursors = sc.get<uint32_t>((size_t)grid * (size_t)g->sweep_max_lower * 3);
+    uint2* cursors = sc.get<uint2>((size_t)grid * (size_t)g->sweep_max_lower);
+    Segment* segments = sc.get<Segment>((size_t)grid * (size_t)g->sweep_max_lower);
     int* next = sc.get<int>(1);
     DBBC_CUDA(cudaMemsetAsync(next, 0, sizeof(int), s));
-    fn<<<grid, kSweepThreads, smem, s>>>(view, g->sweep_items, g->n_sweep_items, next, cursors, g->sweep_max_lower,
-                                         o);
+    fn<<<grid, kSweepThreads, smem, s>>>(view, g->sweep_items, g->n_sweep_items, next, cursors, segments,
+                                         g->sweep_max_lower, o);
     DBBC_LAUNCH_CHECK();
   }
 }
@@ -505,14 +635,17 @@ extern "C" dbbc_status dbbc_count_edges(const dbbc_graph* g, void* cuda_stream, 
   try {
     Scratch sc(s);
     const int64_t n = g->n, nnz = g->nnz;
-    unsigned long long* acc = sc.get<unsigned long long>((size_t)(2 * nnz));
+    // an edge (u, v) is in at most (deg(u) - 1)(deg(v) - 1) butterflies: when
+    // that fits 32 bits for the largest degrees, both counts share a word
+    const size_t words = (uint64_t)g->max_deg_u * (uint64_t)g->max_deg_v >> 32 ? 2 : 1;
+    unsigned long long* acc = sc.get<unsigned long long>(words * (size_t)nnz);
     unsigned* d_status = sc.get<unsigned>(2);  // [0] device checks, [1] ids out of range
     int32_t* row_of = sc.get<int32_t>((size_t)n);
-    DBBC_CUDA(cudaMemsetAsync(acc, 0, (size_t)(2 * nnz) * 8, s));
+    DBBC_CUDA(cudaMemsetAsync(acc, 0, words * (size_t)nnz * 8, s));
     DBBC_CUDA(cudaMemsetAsync(d_status, 0, 2 * sizeof(unsigned), s));
     TipOut o;
     o.eb = acc;
-    o.eu = acc + nnz;
+    o.eu = words == 2 ? acc + nnz : nullptr;
     o.nnz = nnz;
     enqueue_tips<false, true>(g, s, o, d_status, sc);
     row_of_id_kernel<<<grid_1d(n), 256, 0, s>>>(g->vertex, n, row_of);
