@@ -181,7 +181,7 @@ def _stream_ptr(stream) -> int:
     if stream is None:
         try:
             import torch
-            if torch.cuda.is_available():
+            if torch.cuda.is_initialized():  # else no stream but the default one can be current
                 return int(torch.cuda.current_stream().cuda_stream)
         except ImportError:  # pragma: no cover
             pass

@@ -60,6 +60,42 @@ void raise_device_status(unsigned h) {
   if (h) throw Error{DBBC_EINTERNAL, "device status"};
 }
 
+int resident_ctas(const void* fn, int threads, size_t smem, size_t max_smem) {
+  struct Entry {
+    int dev;
+    const void* fn;
+    size_t smem;
+    int ctas;
+  };
+  static std::mutex mu;
+  static std::vector<Entry> known;
+  int dev = 0;
+  DBBC_CUDA(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lock(mu);
+  for (const Entry& e : known)
+    if (e.dev == dev && e.fn == fn && e.smem == smem) return e.ctas;
+  int b = 0;
+  DBBC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)max_smem));
+  DBBC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, threads, smem));
+  known.push_back(Entry{dev, fn, smem, b > 0 ? b : 1});
+  return known.back().ctas;
+}
+
+int num_sms() {
+  static std::mutex mu;
+  static std::vector<int> sms;
+  int dev = 0;
+  DBBC_CUDA(cudaGetDevice(&dev));
+  std::lock_guard<std::mutex> lock(mu);
+  if ((int)sms.size() <= dev) sms.resize((size_t)dev + 1, 0);
+  int& n = sms[(size_t)dev];
+  if (!n) {
+    DBBC_CUDA(cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev));
+    if (n <= 0) n = kNumSMs;
+  }
+  return n;
+}
+
 void note_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
 void note_launches(uint64_t k) { g_launches.fetch_add(k, std::memory_order_relaxed); }
 uint64_t launches_so_far() { return g_launches.load(std::memory_order_relaxed); }
@@ -136,13 +172,6 @@ static dbbc_status guarded(F&& f) {
   } catch (...) {
     return DBBC_EINTERNAL;
   }
-}
-
-static void check_status_word(const unsigned* d_status, cudaStream_t s) {
-  unsigned h = 0;
-  DBBC_CUDA(cudaMemcpyAsync(&h, d_status, sizeof(h), cudaMemcpyDeviceToHost, s));
-  DBBC_CUDA(cudaStreamSynchronize(s));
-  raise_device_status(h);
 }
 
 }  // namespace dbbc
@@ -339,55 +368,53 @@ dbbc_status dbbc_count_async(const dbbc_graph* g, void* cuda_stream, uint64_t* d
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   return guarded([&] {
     Scratch sc(s);
-    unsigned* d_status = sc.get<unsigned>(1);
-    DBBC_CUDA(cudaMemsetAsync(d_status, 0, sizeof(unsigned), s));
+    CountScratch* d = sc.get<CountScratch>(1);
+    DBBC_CUDA(cudaMemsetAsync(d, 0, sizeof(CountScratch), s));
     DBBC_CUDA(cudaMemsetAsync(d_out, 0, 2 * sizeof(uint64_t), s));
-    enqueue_count(g, s, reinterpret_cast<unsigned long long*>(d_out), d_status, sc);
+    enqueue_count(g, s, reinterpret_cast<unsigned long long*>(d_out), d, sc);
   });
+}
+
+static dbbc_status count_sync(const dbbc_graph* g, cudaStream_t s, uint64_t* balanced, uint64_t* unbalanced,
+                              CountProfiler* cp) {
+  CountScratch h;
+  const dbbc_status st = guarded([&] {
+    Scratch sc(s);
+    CountScratch* d = sc.get<CountScratch>(1);
+    DBBC_CUDA(cudaMemsetAsync(d, 0, sizeof(CountScratch), s));
+    enqueue_count(g, s, d->out, d, sc, cp);
+    DBBC_CUDA(cudaMemcpyAsync(&h, d, sizeof(h), cudaMemcpyDeviceToHost, s));
+    DBBC_CUDA(cudaStreamSynchronize(s));
+    raise_device_status(h.status);
+  });
+  if (st != DBBC_OK) return st;
+  if (balanced) *balanced = h.out[0];
+  if (unbalanced) *unbalanced = h.out[1];
+  if (cp) cp->list_visits = h.visits;
+  return DBBC_OK;
 }
 
 dbbc_status dbbc_count(const dbbc_graph* g, void* cuda_stream, uint64_t* balanced, uint64_t* unbalanced) {
   if (!g) return DBBC_EINVAL;
-  cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  uint64_t h[2] = {0, 0};
-  const dbbc_status st = guarded([&] {
-    Scratch sc(s);
-    unsigned long long* d_out = sc.get<unsigned long long>(2);
-    unsigned* d_status = sc.get<unsigned>(1);
-    DBBC_CUDA(cudaMemsetAsync(d_status, 0, sizeof(unsigned), s));
-    DBBC_CUDA(cudaMemsetAsync(d_out, 0, 2 * sizeof(uint64_t), s));
-    enqueue_count(g, s, d_out, d_status, sc);
-    DBBC_CUDA(cudaMemcpyAsync(h, d_out, sizeof(h), cudaMemcpyDeviceToHost, s));
-    check_status_word(d_status, s);  // synchronizes
-  });
-  if (st != DBBC_OK) return st;
-  if (balanced) *balanced = h[0];
-  if (unbalanced) *unbalanced = h[1];
-  return DBBC_OK;
+  return count_sync(g, static_cast<cudaStream_t>(cuda_stream), balanced, unbalanced, nullptr);
 }
 
 dbbc_status dbbc_count_profiled(const dbbc_graph* g, void* cuda_stream, uint64_t* balanced, uint64_t* unbalanced,
                                 dbbc_count_profile* prof) {
   if (!g) return DBBC_EINVAL;
-  cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-  uint64_t h[2] = {0, 0};
+  uint64_t b = 0, u = 0;
   dbbc_count_profile p;
   std::memset(&p, 0, sizeof(p));
-  const dbbc_status st = guarded([&] {
-    Scratch sc(s);
+  dbbc_status st = DBBC_OK;
+  const dbbc_status ev = guarded([&] {
     CountProfiler cp;
-    unsigned long long* d_out = sc.get<unsigned long long>(2);
-    unsigned* d_status = sc.get<unsigned>(1);
-    DBBC_CUDA(cudaMemsetAsync(d_status, 0, sizeof(unsigned), s));
-    DBBC_CUDA(cudaMemsetAsync(d_out, 0, 2 * sizeof(uint64_t), s));
-    enqueue_count(g, s, d_out, d_status, sc, &cp);
-    DBBC_CUDA(cudaMemcpyAsync(h, d_out, sizeof(h), cudaMemcpyDeviceToHost, s));
-    check_status_word(d_status, s);  // synchronizes
-    cp.summarize(&p);
+    st = count_sync(g, static_cast<cudaStream_t>(cuda_stream), &b, &u, &cp);
+    if (st == DBBC_OK) cp.summarize(&p);
   });
   if (st != DBBC_OK) return st;
-  if (balanced) *balanced = h[0];
-  if (unbalanced) *unbalanced = h[1];
+  if (ev != DBBC_OK) return ev;
+  if (balanced) *balanced = b;
+  if (unbalanced) *unbalanced = u;
   if (prof) *prof = p;
   return DBBC_OK;
 }

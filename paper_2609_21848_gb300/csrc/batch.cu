@@ -41,7 +41,9 @@ struct GatherJob {
   int64_t medium_off, light_off;
 };
 
-__device__ __forceinline__ CsrView view_of(const GraphDesc& d) { return CsrView{d.row_ptr, d.col, d.lower, d.n_u, d.n, d.nnz}; }
+__device__ __forceinline__ CsrView view_of(const GraphDesc& d) {
+  return CsrView{d.row_ptr, d.col, d.lower, d.n_u, d.n, d.nnz};
+}
 
 // One CTA per graph copies its medium and light pivots into the batch lists.
 __global__ void gather_pivots_kernel(const GatherJob* __restrict__ jobs, BatchPivot* __restrict__ med,
@@ -419,7 +421,9 @@ static size_t medium_smem_bytes(const dbbc_batch* b) { return ((size_t)1 << b->m
 // union's CSR; pivots and hub items are tagged with their component.
 static void plan_components(dbbc_batch* b, const dbbc_graph* g) {
   cudaStream_t s = b->stream;
-  std::vector<GraphDesc> desc((size_t)b->n_graphs, GraphDesc{g->row_ptr, g->col, g->lower, g->work, g->n, g->nnz, g->n_u, g->tune.hash_mult_log});
+  std::vector<GraphDesc> desc((size_t)b->n_graphs,
+                              GraphDesc{g->row_ptr, g->col, g->lower, g->work, g->n, g->nnz, g->n_u,
+                                        g->tune.hash_mult_log});
   b->n_medium = g->n_medium;
   b->n_light = g->n_light;
   plan_items(b, {HubJob{g->sweep_items, g->lower, 0, 0}}, g->n_sweep_items, g->component);
@@ -472,22 +476,26 @@ static void finish_plan(dbbc_batch* b, const std::vector<GraphDesc>& desc) {
   b->out = static_cast<unsigned long long*>(batch_alloc(b, (size_t)n * 2 * sizeof(unsigned long long)));
   b->counters = static_cast<int*>(batch_alloc(b, 3 * sizeof(int)));
   b->status = static_cast<unsigned*>(batch_alloc(b, sizeof(unsigned)));
-  b->hub_grid = (int)std::min<int64_t>(num_sms() * blocks_per_sm((const void*)DBBC_WIDE_SWEEP, kSweepThreads,
-                                                                 kSweepSmem), std::max<int64_t>(b->n_wide, 1));
-  b->narrow_grid = (int)std::min<int64_t>(num_sms() * blocks_per_sm((const void*)DBBC_NARROW_SWEEP, kNarrowThreads,
-                                                                    kNarrowSmem), std::max<int64_t>(b->n_narrow, 1));
+  b->hub_grid = (int)std::min<int64_t>(num_sms() * resident_ctas((const void*)DBBC_WIDE_SWEEP, kSweepThreads,
+                                                                 kSweepSmem, kSweepSmem),
+                                       std::max<int64_t>(b->n_wide, 1));
+  b->narrow_grid = (int)std::min<int64_t>(num_sms() * resident_ctas((const void*)DBBC_NARROW_SWEEP, kNarrowThreads,
+                                                                    kNarrowSmem, kNarrowSmem),
+                                          std::max<int64_t>(b->n_narrow, 1));
   if (b->n_wide > 0)
     b->cursors = static_cast<uint2*>(batch_alloc(b, (size_t)b->hub_grid * (size_t)b->lower_wide * sizeof(uint2)));
   if (b->n_narrow > 0)
-    b->narrow_cursors = static_cast<uint2*>(batch_alloc(b, (size_t)b->narrow_grid * (size_t)b->lower_narrow * sizeof(uint2)));
+    b->narrow_cursors =
+        static_cast<uint2*>(batch_alloc(b, (size_t)b->narrow_grid * (size_t)b->lower_narrow * sizeof(uint2)));
   {
     const int sms = num_sms();
     const int64_t want = ceil_div<int64_t>(ceil_div<int64_t>(b->n_light, 32), kLightWarps);
-    const int64_t cap = (int64_t)sms * blocks_per_sm((const void*)count_light_batch_kernel, kLightWarps * 32,
-                                                     light_smem_bytes(b));
+    const int64_t cap = (int64_t)sms * resident_ctas((const void*)count_light_batch_kernel, kLightWarps * 32,
+                                                     light_smem_bytes(b),
+                                                     (size_t)kLightWarps * kLightSlots * kHashSlotBytes);
     b->light_grid = (int)std::max<int64_t>(1, std::min(want, cap));
-    const int64_t mcap = (int64_t)sms * blocks_per_sm((const void*)count_medium_batch_kernel, kMediumThreads,
-                                                      medium_smem_bytes(b));
+    const int64_t mcap = (int64_t)sms * resident_ctas((const void*)count_medium_batch_kernel, kMediumThreads,
+                                                      medium_smem_bytes(b), (size_t)kMediumSlots * kHashSlotBytes);
     b->medium_grid = (int)std::max<int64_t>(1, std::min<int64_t>(b->n_medium, mcap));
   }
   if (!b->side) {
@@ -540,15 +548,6 @@ static void enqueue_batch(dbbc_batch* b, cudaStream_t s) {
   }
 }
 
-static void set_batch_attributes() {
-  DBBC_CUDA(cudaFuncSetAttribute(count_light_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)((size_t)kLightWarps * kLightSlots * kHashSlotBytes)));
-  DBBC_CUDA(cudaFuncSetAttribute(count_medium_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)((size_t)kMediumSlots * kHashSlotBytes)));
-  DBBC_CUDA(cudaFuncSetAttribute(DBBC_WIDE_SWEEP, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepSmem));
-  DBBC_CUDA(cudaFuncSetAttribute(DBBC_NARROW_SWEEP, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kNarrowSmem));
-}
-
 static void check_batch_status(const dbbc_batch* b, cudaStream_t s) {
   unsigned h = 0;
   DBBC_CUDA(cudaMemcpyAsync(&h, b->status, sizeof(h), cudaMemcpyDeviceToHost, s));
@@ -582,7 +581,6 @@ void count_subset(const dbbc_graph* g, cudaStream_t s, const std::vector<int32_t
   uint64_t h[2] = {0, 0};
   try {
     DBBC_CUDA(cudaGetDevice(&b->device));
-    set_batch_attributes();
     std::vector<GraphDesc> desc(1, GraphDesc{g->row_ptr, g->col, g->lower, g->work, g->n, g->nnz, g->n_u,
                                               g->tune.hash_mult_log});
     b->n_medium = (int64_t)medium_rows.size();
@@ -637,7 +635,6 @@ dbbc_status dbbc_batch_create(const dbbc_graph* const* gs, int32_t n_graphs, voi
   b->n_graphs = n_graphs;
   const dbbc_status st = batch_guard([&] {
     DBBC_CUDA(cudaGetDevice(&b->device));
-    set_batch_attributes();
     plan_batch(b, gs);
   });
   if (st != DBBC_OK) {
@@ -718,7 +715,6 @@ dbbc_status dbbc_count_components(const dbbc_graph* g, void* cuda_stream, uint64
   std::vector<uint64_t> h((size_t)n * 2);
   const dbbc_status st = batch_guard([&] {
     DBBC_CUDA(cudaGetDevice(&b->device));
-    set_batch_attributes();
     plan_components(b, g);
     enqueue_batch(b, b->stream);
     DBBC_CUDA(cudaMemcpyAsync(h.data(), b->out, h.size() * 8, cudaMemcpyDeviceToHost, b->stream));

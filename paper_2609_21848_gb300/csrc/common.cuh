@@ -104,6 +104,43 @@ inline T ceil_div(T a, T b) {
   return (a + b - 1) / b;
 }
 
+// ---------------------------------------------------------------- kernel attributes
+// Lets kernel fn use up to max_smem bytes of dynamic shared memory and returns
+// how many of its CTAs (`threads` threads, smem bytes) fit an SM of the current
+// device. Asked of the driver once per device, kernel and size: a count of a
+// resident 20k-edge graph spent a quarter of its 45 us on these queries and on
+// separate clears and read-backs.
+int resident_ctas(const void* fn, int threads, size_t smem, size_t max_smem);
+int num_sms();  // of the current device
+
+// ---------------------------------------------------------------- overlapped launches
+// Kernels launched by launch_overlapped may start while the kernel before them
+// on the stream still runs (programmatic dependent launch): once all CTAs of
+// that kernel have called let_next_start, or ended. They wait for its end and
+// its writes in wait_for_previous, which every kernel that is launched this
+// way calls in every CTA. Sequences of short kernels lose the launch gaps:
+// with this and the cached queries above, a 20k-edge build takes 158 instead of
+// 184 us, a 2M-edge one with repeated pairs 722 instead of 781 us, and a
+// count of a resident 1M-edge graph, whose tiers overlap, 318 instead of 353 us.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+template <typename... P, typename... A>
+void launch_overlapped(void (*kernel)(P...), int64_t grid, int threads, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3((unsigned)grid);
+  c.blockDim = dim3((unsigned)threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = at;
+  c.numAttrs = 1;
+  DBBC_CUDA(cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...));
+  note_launch();
+}
+
 // ---------------------------------------------------------------- allocator
 void* dev_alloc(size_t bytes, cudaStream_t s);
 void dev_free(void* p, cudaStream_t s);

@@ -23,6 +23,7 @@ __global__ void __launch_bounds__(kLightWarps * 32) count_light_kernel(CsrView g
                                                                        int hash_mult_log, int slots_log,
                                                                        unsigned long long* out, unsigned* status) {
   extern __shared__ __align__(16) unsigned char light_smem[];
+  let_next_start();
   const int slots = 1 << slots_log;
   uint32_t* tables = reinterpret_cast<uint32_t*>(light_smem);
   const int w = threadIdx.x >> 5;
@@ -52,6 +53,7 @@ __global__ void __launch_bounds__(kLightWarps * 32) count_light_kernel(CsrView g
   }
   if (full) atomicOr(status, DBBC_DEV_HASH_FULL);
   block_add_pair<kLightWarps * 32>(bal, unb, out);
+  wait_for_previous();
 }
 
 // ------------------------------------------------------------------ medium tier
@@ -61,6 +63,7 @@ __global__ void __launch_bounds__(kMediumThreads) count_medium_kernel(CsrView g,
                                                                       int64_t n_piv, int hash_mult_log, int slots_log,
                                                                       unsigned long long* out, unsigned* status) {
   extern __shared__ __align__(16) unsigned char med_smem[];
+  let_next_start();
   const int slots = 1 << slots_log;
   uint32_t* keys = reinterpret_cast<uint32_t*>(med_smem);
   uint32_t* vals = keys + slots;
@@ -87,6 +90,7 @@ __global__ void __launch_bounds__(kMediumThreads) count_medium_kernel(CsrView g,
   }
   if (full) atomicOr(status, DBBC_DEV_HASH_FULL);
   block_add_pair<kMediumThreads>(bal, unb, out);
+  wait_for_previous();
 }
 
 // ------------------------------------------------------------------ hub tier
@@ -104,6 +108,7 @@ __global__ void __launch_bounds__(kSweepThreads) hub_sweep_kernel(CsrView g, con
   extern __shared__ __align__(16) unsigned char sweep_smem[];
   uint32_t* cnt_words = reinterpret_cast<uint32_t*>(sweep_smem);
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sweep_smem);
+  let_next_start();
   __shared__ int item_sh;
   __shared__ ListState ls;
   __shared__ uint32_t nbn[2];
@@ -138,6 +143,7 @@ __global__ void __launch_bounds__(kSweepThreads) hub_sweep_kernel(CsrView g, con
   }
   block_add_pair<kSweepThreads>(bal, unb, out);
   if (visits && tid == 0 && n_visits) atomicAdd(visits, (unsigned long long)n_visits);
+  wait_for_previous();
 }
 
 // ------------------------------------------------------------------ host
@@ -162,7 +168,6 @@ void CountProfiler::summarize(dbbc_count_profile* out) {
     DBBC_CUDA(cudaEventElapsedTime(&t, mk.a, mk.b));
     ms[mk.tier] += t;
   }
-  if (d_visits) DBBC_CUDA(cudaMemcpy(&list_visits, d_visits, sizeof(list_visits), cudaMemcpyDeviceToHost));
   out->ms_light = ms[LIGHT];
   out->ms_medium = ms[MEDIUM];
   out->ms_hub_aggregate = ms[HUB_AGG];
@@ -182,103 +187,107 @@ CountProfiler::~CountProfiler() {
   }
 }
 
-// Launches of the three tiers, shared by enqueue_count and
-// enqueue_count_prealloc.
+// Launches of the tiers, shared by enqueue_count and enqueue_count_prealloc.
+// The tiers only add to the same two words, so a tier may start as soon as the
+// one before it leaves room (launch_overlapped): every kernel lets the next
+// one start at its beginning and waits for the one before it at its end, which
+// keeps the end of the last kernel the end of the count. The hub sweep, whose
+// CTAs fill an SM each, goes first, and the other tiers fill its last wave.
+// `first`: the first kernel after something else on the stream.
+template <typename... P, typename... A>
+static void launch_tier(bool first, void (*kernel)(P...), int64_t grid, int threads, size_t smem, cudaStream_t s,
+                        A&&... args) {
+  if (first) {
+    kernel<<<(unsigned)grid, threads, smem, s>>>(args...);
+    DBBC_LAUNCH_CHECK();
+  } else {
+    launch_overlapped(kernel, grid, threads, smem, s, args...);
+  }
+}
+
 static void launch_light(const dbbc_graph* g, const CsrView& view, cudaStream_t s, unsigned long long* d_out,
-                         unsigned* d_status) {
+                         unsigned* d_status, bool first) {
   const int slots_log = tier_slots_log(g->tune.light_max_work, g->tune.hash_mult_log, 10);
   const size_t smem = (size_t)kLightWarps * ((size_t)1 << slots_log) * kHashSlotBytes;
-  DBBC_CUDA(cudaFuncSetAttribute(count_light_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)((size_t)kLightWarps * kLightSlots * kHashSlotBytes)));
   const int64_t want = ceil_div<int64_t>(g->n_light, kLightWarps);
-  const int64_t cap = (int64_t)num_sms() * blocks_per_sm((const void*)count_light_kernel, kLightWarps * 32, smem);
-  count_light_kernel<<<(unsigned)std::min(want, cap), kLightWarps * 32, smem, s>>>(
-      view, g->order + g->n_hub + g->n_medium, g->work, g->n_light, g->tune.hash_mult_log, slots_log, d_out,
-      d_status);
-  DBBC_LAUNCH_CHECK();
+  const int64_t cap = (int64_t)num_sms() * resident_ctas((const void*)count_light_kernel, kLightWarps * 32, smem,
+                                                         (size_t)kLightWarps * kLightSlots * kHashSlotBytes);
+  launch_tier(first, count_light_kernel, std::min(want, cap), kLightWarps * 32, smem, s, view,
+              g->order + g->n_hub + g->n_medium, g->work, g->n_light, g->tune.hash_mult_log, slots_log, d_out,
+              d_status);
 }
 
 static void launch_medium(const dbbc_graph* g, const CsrView& view, cudaStream_t s, unsigned long long* d_out,
-                          unsigned* d_status) {
+                          unsigned* d_status, bool first) {
   const int slots_log = tier_slots_log(g->tune.medium_max_work, g->tune.hash_mult_log, 13);
   const size_t smem = ((size_t)1 << slots_log) * kHashSlotBytes;
-  DBBC_CUDA(cudaFuncSetAttribute(count_medium_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)((size_t)kMediumSlots * kHashSlotBytes)));
-  const int64_t cap = (int64_t)num_sms() * blocks_per_sm((const void*)count_medium_kernel, kMediumThreads, smem);
-  count_medium_kernel<<<(unsigned)std::min<int64_t>(g->n_medium, cap), kMediumThreads, smem, s>>>(
-      view, g->order + g->n_hub, g->work, g->n_medium, g->tune.hash_mult_log, slots_log, d_out, d_status);
-  DBBC_LAUNCH_CHECK();
+  const int64_t cap = (int64_t)num_sms() * resident_ctas((const void*)count_medium_kernel, kMediumThreads, smem,
+                                                         (size_t)kMediumSlots * kHashSlotBytes);
+  launch_tier(first, count_medium_kernel, std::min<int64_t>(g->n_medium, cap), kMediumThreads, smem, s, view,
+              g->order + g->n_hub, g->work, g->n_medium, g->tune.hash_mult_log, slots_log, d_out, d_status);
 }
 
 // CTAs the hub sweep can keep resident (one per SM: its counters fill the
 // SM's shared memory).
 static int64_t hub_full_grid() {
-  DBBC_CUDA(cudaFuncSetAttribute(hub_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepSmem));
-  return (int64_t)num_sms() * blocks_per_sm((const void*)hub_sweep_kernel, kSweepThreads, kSweepSmem);
+  return (int64_t)num_sms() * resident_ctas((const void*)hub_sweep_kernel, kSweepThreads, kSweepSmem, kSweepSmem);
 }
 
 // The hub sweep on `grid` CTAs with per-CTA cursors (sweep_max_lower each)
-// and, if `lists` is given, per-CTA list scratch (sweep_list_cap slots each);
-// `next` is the item counter, cleared here.
-static void launch_hub(const dbbc_graph* g, const CsrView& view, cudaStream_t s, int grid, int* next,
-                       uint2* cursors, uint2* lists, unsigned long long* d_out, unsigned long long* visits) {
-  DBBC_CUDA(cudaMemsetAsync(next, 0, sizeof(int), s));
-  hub_sweep_kernel<<<grid, kSweepThreads, kSweepSmem, s>>>(view, g->sweep_items, g->n_sweep_items, next, cursors,
-                                                           g->sweep_max_lower, lists,
-                                                           lists ? g->sweep_list_cap : 0, d_out, visits);
+// and, if `lists` is given, per-CTA list scratch (sweep_list_cap slots each).
+static void launch_hub(const dbbc_graph* g, const CsrView& view, cudaStream_t s, int grid, uint2* cursors,
+                       uint2* lists, unsigned long long* d_out, CountScratch* d, bool count_visits) {
+  hub_sweep_kernel<<<grid, kSweepThreads, kSweepSmem, s>>>(view, g->sweep_items, g->n_sweep_items, &d->next, cursors,
+                                                           g->sweep_max_lower, lists, lists ? g->sweep_list_cap : 0,
+                                                           d_out, count_visits ? &d->visits : nullptr);
   DBBC_LAUNCH_CHECK();
 }
 
-void enqueue_count(const dbbc_graph* g, cudaStream_t s, unsigned long long* d_out, unsigned* d_status,
-                   Scratch& sc, CountProfiler* prof) {
+void enqueue_count(const dbbc_graph* g, cudaStream_t s, unsigned long long* d_out, CountScratch* d, Scratch& sc,
+                   CountProfiler* prof) {
   if (g->n_piv == 0) return;
   const CsrView view{g->row_ptr, g->col, g->lower, g->n_u, g->n, g->nnz};
   cudaEvent_t t_all = prof ? prof->begin(s) : nullptr;
   cudaEvent_t t0 = nullptr;
-  if (g->n_light > 0) {
+  if (g->n_hub > 0) {
+    const int grid = (int)hub_full_grid();
+    uint2* cursors = sc.get<uint2>((size_t)grid * (size_t)g->sweep_max_lower);
+    uint2* lists = g->sweep_list_cap > 0 ? sc.get<uint2>((size_t)grid * (size_t)g->sweep_list_cap) : nullptr;
     if (prof) t0 = prof->begin(s);
-    launch_light(g, view, s, d_out, d_status);
+    launch_hub(g, view, s, grid, cursors, lists, d_out, d, prof != nullptr);
     if (prof) {
-      prof->end(CountProfiler::LIGHT, t0, s);
-      prof->launches[CountProfiler::LIGHT]++;
+      prof->end(CountProfiler::HUB_AGG, t0, s);
+      prof->launches[CountProfiler::HUB_AGG]++;
     }
   }
   if (g->n_medium > 0) {
     if (prof) t0 = prof->begin(s);
-    launch_medium(g, view, s, d_out, d_status);
+    launch_medium(g, view, s, d_out, &d->status, g->n_hub == 0);
     if (prof) {
       prof->end(CountProfiler::MEDIUM, t0, s);
       prof->launches[CountProfiler::MEDIUM]++;
     }
   }
-  if (g->n_hub > 0) {
-    const int grid = (int)hub_full_grid();
-    uint2* cursors = sc.get<uint2>((size_t)grid * (size_t)g->sweep_max_lower);
-    uint2* lists = g->sweep_list_cap > 0 ? sc.get<uint2>((size_t)grid * (size_t)g->sweep_list_cap) : nullptr;
-    int* next = sc.get<int>(1);
+  if (g->n_light > 0) {
+    if (prof) t0 = prof->begin(s);
+    launch_light(g, view, s, d_out, &d->status, g->n_hub + g->n_medium == 0);
     if (prof) {
-      prof->d_visits = sc.get<unsigned long long>(1);
-      DBBC_CUDA(cudaMemsetAsync(prof->d_visits, 0, sizeof(unsigned long long), s));
-      t0 = prof->begin(s);
-    }
-    launch_hub(g, view, s, grid, next, cursors, lists, d_out, prof ? prof->d_visits : nullptr);
-    if (prof) {
-      prof->end(CountProfiler::HUB_AGG, t0, s);
-      prof->launches[CountProfiler::HUB_AGG]++;
+      prof->end(CountProfiler::LIGHT, t0, s);
+      prof->launches[CountProfiler::LIGHT]++;
     }
   }
   if (prof) prof->end(CountProfiler::TOTAL, t_all, s);
 }
 
 // The kernels of enqueue_count with all device scratch supplied by the caller:
-// d_status (one word) and d_next (one int) are cleared here, and the hub
-// sweep keeps its per-CTA cursors (8 bytes per lower neighbour of the largest
-// hub) in `cursors` (cursor_bytes long, 8-byte aligned), which bounds how many
-// CTAs it can run; it runs without list scratch (cursor mode for every item,
-// same counts). Throws DBBC_EOVERFLOW when not even one CTA's cursors fit.
-void enqueue_count_prealloc(const dbbc_graph* g, cudaStream_t s, unsigned long long* d_out, unsigned* d_status,
-                            int* d_next, uint32_t* cursors, size_t cursor_bytes) {
-  DBBC_CUDA(cudaMemsetAsync(d_status, 0, sizeof(unsigned), s));
+// *d and d_out are cleared here, and the hub sweep keeps its per-CTA cursors
+// (8 bytes per lower neighbour of the largest hub) in `cursors` (cursor_bytes
+// long, 8-byte aligned), which bounds how many CTAs it can run; it runs
+// without list scratch (cursor mode for every item, same counts). Throws
+// DBBC_EOVERFLOW when not even one CTA's cursors fit.
+void enqueue_count_prealloc(const dbbc_graph* g, cudaStream_t s, unsigned long long* d_out, CountScratch* d,
+                            uint32_t* cursors, size_t cursor_bytes) {
+  DBBC_CUDA(cudaMemsetAsync(d, 0, sizeof(CountScratch), s));
   DBBC_CUDA(cudaMemsetAsync(d_out, 0, 2 * sizeof(unsigned long long), s));
   if (g->n_piv == 0) return;
   const CsrView view{g->row_ptr, g->col, g->lower, g->n_u, g->n, g->nnz};
@@ -288,12 +297,12 @@ void enqueue_count_prealloc(const dbbc_graph* g, cudaStream_t s, unsigned long l
     hub_grid = (int64_t)(cursor_bytes / per_cta);
     if (hub_grid < 1) throw Error{DBBC_EOVERFLOW, "hub cursors exceed the fixed scratch"};
   }
-  if (g->n_light > 0) launch_light(g, view, s, d_out, d_status);
-  if (g->n_medium > 0) launch_medium(g, view, s, d_out, d_status);
   if (g->n_hub > 0) {
     const int grid = (int)std::min<int64_t>(hub_full_grid(), hub_grid);
-    launch_hub(g, view, s, grid, d_next, reinterpret_cast<uint2*>(cursors), nullptr, d_out, nullptr);
+    launch_hub(g, view, s, grid, reinterpret_cast<uint2*>(cursors), nullptr, d_out, d, false);
   }
+  if (g->n_medium > 0) launch_medium(g, view, s, d_out, &d->status, g->n_hub == 0);
+  if (g->n_light > 0) launch_light(g, view, s, d_out, &d->status, g->n_hub + g->n_medium == 0);
 }
 
 }  // namespace dbbc

@@ -301,21 +301,4 @@ struct ItemWindows {
   }
 };
 
-inline int blocks_per_sm(const void* fn, int threads, size_t smem) {
-  int b = 0;
-  DBBC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, fn, threads, smem));
-  return b > 0 ? b : 1;
-}
-
-inline int num_sms() {
-  static int sms = 0;
-  if (!sms) {
-    int dev = 0;
-    DBBC_CUDA(cudaGetDevice(&dev));
-    DBBC_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    if (sms <= 0) sms = kNumSMs;
-  }
-  return sms;
-}
-
 }  // namespace dbbc

@@ -200,8 +200,7 @@ struct CountProfiler {
     cudaEvent_t a, b;
   };
   std::vector<Mark> marks;
-  unsigned long long* d_visits = nullptr;  // device counter of list-mode (neighbour, window) visits
-  uint64_t list_visits = 0;
+  uint64_t list_visits = 0;  // list-mode (neighbour, window) visits
   int64_t launches[NTIERS] = {0, 0, 0, 0, 0};
   cudaEvent_t begin(cudaStream_t s);
   void end(int tier, cudaEvent_t a, cudaStream_t s);
@@ -210,13 +209,23 @@ struct CountProfiler {
   ~CountProfiler();
 };
 
+// Device words of one count, all zero before it: its result when the caller
+// has no device output, the list-mode visits, the status word and the hub item
+// counter.
+struct CountScratch {
+  unsigned long long out[2];
+  unsigned long long visits;
+  unsigned status;
+  int next;
+};
+
 // count.cu: enqueue the counting kernels of one graph, accumulating
-// {balanced, unbalanced} into d_out[0..1] (device, must be zeroed by caller).
-void enqueue_count(const dbbc_graph* g, cudaStream_t stream, unsigned long long* d_out, unsigned* d_status,
+// {balanced, unbalanced} into d_out[0..1] (device, zeroed by the caller).
+void enqueue_count(const dbbc_graph* g, cudaStream_t stream, unsigned long long* d_out, CountScratch* d,
                    Scratch& scratch, CountProfiler* prof = nullptr);
 
 // count.cu: the same kernels with caller-supplied scratch (see noalloc.cu).
-void enqueue_count_prealloc(const dbbc_graph* g, cudaStream_t stream, unsigned long long* d_out, unsigned* d_status,
-                            int* d_next, uint32_t* cursors, size_t cursor_bytes);
+void enqueue_count_prealloc(const dbbc_graph* g, cudaStream_t stream, unsigned long long* d_out, CountScratch* d,
+                            uint32_t* cursors, size_t cursor_bytes);
 
 }  // namespace dbbc

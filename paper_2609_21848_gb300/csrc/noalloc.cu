@@ -21,7 +21,7 @@
 namespace dbbc {
 
 constexpr size_t kNoAllocScratchBytes = size_t(32) << 20;
-constexpr size_t kNoAllocHeaderBytes = 256;  // status word and work-item counter
+constexpr size_t kNoAllocHeaderBytes = 256;  // the count's CountScratch
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
 
@@ -55,10 +55,9 @@ extern "C" dbbc_status dbbc_count_noalloc(const dbbc_graph* g, void* cuda_stream
   cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
   try {
     unsigned char* base = noalloc_scratch_address();
-    unsigned* d_status = reinterpret_cast<unsigned*>(base);
-    int* d_next = reinterpret_cast<int*>(base + 64);
+    CountScratch* d = reinterpret_cast<CountScratch*>(base);
     uint32_t* cursors = reinterpret_cast<uint32_t*>(base + kNoAllocHeaderBytes);
-    enqueue_count_prealloc(g, s, reinterpret_cast<unsigned long long*>(d_out), d_status, d_next, cursors,
+    enqueue_count_prealloc(g, s, reinterpret_cast<unsigned long long*>(d_out), d, cursors,
                            kNoAllocScratchBytes - kNoAllocHeaderBytes);
     return DBBC_OK;
   } catch (const Error& e) {

@@ -78,6 +78,8 @@ __global__ void degree_kernel(const int32_t* __restrict__ eu, const int32_t* __r
                               const int8_t* __restrict__ es, int64_t m, int32_t n_u, int32_t n_v,
                               int32_t* __restrict__ deg, unsigned* flags) {
   constexpr int kRound = 4;  // edges per thread per round, their loads in flight together
+  let_next_start();
+  wait_for_previous();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t iters = (m + stride - 1) / stride;  // the same for every lane: the warp votes together
   const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -145,7 +147,8 @@ __global__ void __launch_bounds__(kRowThreads) ranks_kernel(const uint64_t* __re
                                                             int bits_comp, int bits_deg, int bits_id, UnionView un,
                                                             int32_t* __restrict__ vertex,
                                                             int32_t* __restrict__ side_rank,
-                                                            int32_t* __restrict__ rowdeg, int64_t* __restrict__ row_ptr,
+                                                            int32_t* __restrict__ rowdeg,
+                                                            int64_t* __restrict__ row_ptr,
                                                             int32_t* __restrict__ component,
                                                             uint64_t* __restrict__ work, uint64_t* state,
                                                             unsigned* counter, unsigned* flags) {
@@ -533,6 +536,8 @@ __global__ void union_ids_kernel(const int32_t* __restrict__ u, const int32_t* _
                                  const int64_t* __restrict__ uoff, const int64_t* __restrict__ voff, int32_t n_graphs,
                                  int64_t m, int32_t* __restrict__ ou, int32_t* __restrict__ ov,
                                  int8_t* __restrict__ os) {
+  let_next_start();
+  wait_for_previous();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
     int32_t c = component_of(eoff, n_graphs, i - (int64_t)lane_id());
     while (i >= eoff[c + 1]) c++;
@@ -697,6 +702,8 @@ __global__ void __launch_bounds__(kRowThreads) plan_hubs_kernel(HubPlanner hp, S
 
 __global__ void gather_items_kernel(const SweepItem* __restrict__ src, const uint32_t* __restrict__ idx, int64_t n,
                                     SweepItem* __restrict__ dst) {
+  let_next_start();
+  wait_for_previous();
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
     dst[i] = src[idx[i]];
 }
@@ -799,9 +806,9 @@ static void plan_hubs(dbbc_graph* g, cudaStream_t s, const UnionView& un, PrepRe
   const Layout l = place(carver);
   DBBC_CUDA(cudaMemsetAsync(zero, 0, l.zeroed, s));
   const HubPlanner hp{g->order, g->lower, g->work, res->below, g->n_hub, g->n_u, un, g->tune};
-  plan_hubs_kernel<<<(unsigned)tiles, kRowThreads, 0, s>>>(hp, l.items, cap, l.key, l.idx, l.sort.hist, &res->hubs,
-                                                           l.state, l.counter, &res->flags);
-  DBBC_LAUNCH_CHECK();
+  launch_overlapped(plan_hubs_kernel,
+                    (unsigned)tiles, kRowThreads, 0, s, hp, l.items, cap, l.key, l.idx, l.sort.hist, &res->hubs,
+                    l.state, l.counter, &res->flags);
   const PrepResult r = read_back(res, s);
   if (r.flags & kPrepTimeout) throw Error{DBBC_EINTERNAL, "a bounded wait of the build gave up"};
   if (r.hubs.items > cap) throw Error{DBBC_EINTERNAL, "hub plan"};
@@ -814,8 +821,8 @@ static void plan_hubs(dbbc_graph* g, cudaStream_t s, const UnionView& un, PrepRe
   if (g->n_sweep_items == 0) return;
   radix_pass<PlainLoad, true, false, false>(PlainLoad{l.key, l.idx}, PassOut{nullptr, l.sorted, nullptr, 0},
                                             g->n_sweep_items, 0, 0, l.sort, &res->flags, s);
-  gather_items_kernel<<<grid_for(g->n_sweep_items), 256, 0, s>>>(l.items, l.sorted, g->n_sweep_items, g->sweep_items);
-  DBBC_LAUNCH_CHECK();
+  launch_overlapped(gather_items_kernel,
+                    grid_for(g->n_sweep_items), 256, 0, s, l.items, l.sorted, g->n_sweep_items, g->sweep_items);
 }
 
 void build_graph_multi(dbbc_graph* g, const int32_t* u, const int32_t* v, const int8_t* sgn,
@@ -861,9 +868,8 @@ void build_graph_multi(dbbc_graph* g, const int32_t* u, const int32_t* v, const 
   int32_t* ov = sc.get<int32_t>((size_t)std::max<int64_t>(m, 1));
   int8_t* os = sc.get<int8_t>((size_t)std::max<int64_t>(m, 1));
   if (m > 0) {
-    union_ids_kernel<<<grid_for(m), 256, 0, s>>>(du, dv, ds, d_meta, d_meta + k, d_meta + 2 * k, n_graphs, m, ou, ov,
-                                                 os);
-    DBBC_LAUNCH_CHECK();
+    launch_overlapped(union_ids_kernel,
+                      grid_for(m), 256, 0, s, du, dv, ds, d_meta, d_meta + k, d_meta + 2 * k, n_graphs, m, ou, ov, os);
   }
   UnionSpec un;
   un.n_graphs = std::max<int32_t>(n_graphs, 1);
@@ -992,28 +998,26 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
   auto build_from_edges = [&](const int32_t* eu, const int32_t* ev, const int8_t* es, int64_t me) -> PrepResult {
     DBBC_CUDA(cudaMemsetAsync(l.res, 0, l.zeroed, s));
     g->col = static_cast<uint32_t*>(graph_alloc(g, (size_t)(2 * me) * 4, kColPad));
-    if (me > 0) {
-      degree_kernel<<<grid_for(me), 256, 0, s>>>(eu, ev, es, me, n_u, n_v, l.deg, d_flags);
-      DBBC_LAUNCH_CHECK();
-    }
+    if (me > 0)
+      launch_overlapped(degree_kernel, grid_for(me), 256, 0, s, eu, ev, es, me, n_u, n_v, l.deg, d_flags);
     if (n > 0) {
-      vertex_keys_kernel<<<count_grid(n), 256, 0, s>>>(l.deg, n, n_u, bits_comp, bits_deg, bits_lid, uv, l.vk0, passes_r,
-                                                     l.rank.hist, d_flags);
-      DBBC_LAUNCH_CHECK();
+      launch_overlapped(vertex_keys_kernel,
+                        count_grid(n), 256, 0, s, l.deg, n, n_u, bits_comp, bits_deg, bits_lid, uv, l.vk0, passes_r,
+                        l.rank.hist, d_flags);
       uint64_t *in = l.vk0, *out = l.vk1;
       for (int p = 0; p < passes_r; p++, std::swap(in, out))
         radix_pass<PlainLoad, false, true, false>(PlainLoad{in, nullptr}, PassOut{out, nullptr, nullptr, 0}, n,
                                                   bits_lid, p, l.rank, d_flags, s);
-      ranks_kernel<<<(unsigned)ceil_div<int64_t>(n, kRowTile), kRowThreads, 0, s>>>(
-          in, n, n_u, bits_comp, bits_deg, bits_lid, uv, g->vertex, l.side_rank, l.rowdeg, g->row_ptr, g->component,
-          g->work, l.row_state, l.counters, d_flags);
-      DBBC_LAUNCH_CHECK();
+      launch_overlapped(ranks_kernel,
+                        (unsigned)ceil_div<int64_t>(n, kRowTile), kRowThreads, 0, s, in, n, n_u, bits_comp, bits_deg,
+                        bits_lid, uv, g->vertex, l.side_rank, l.rowdeg, g->row_ptr, g->component, g->work,
+                        l.row_state, l.counters, d_flags);
     }
     CsrKeys ck{nullptr, nullptr, me, n_u, bits_u};
     if (me > 0) {
-      csr_u_keys_kernel<<<count_grid(me), 256, 0, s>>>(eu, ev, es, me, n_u, l.side_rank, bits_v, l.ck0, passes_u,
-                                                     l.su.hist, d_flags);
-      DBBC_LAUNCH_CHECK();
+      launch_overlapped(csr_u_keys_kernel,
+                        count_grid(me), 256, 0, s, eu, ev, es, me, n_u, l.side_rank, bits_v, l.ck0, passes_u,
+                        l.su.hist, d_flags);
       uint64_t *in = l.ck0, *out = l.ck1;
       for (int p = 0; p < passes_u; p++, std::swap(in, out)) {
         const PassOut po{out, nullptr, g->col, (2ull << bits_v) - 1};
@@ -1024,8 +1028,7 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
       }
       ku = in;
       const VKey vk{bits_u, bits_v};
-      csr_v_digits_kernel<<<count_grid(me), 256, 0, s>>>(ku, me, vk, passes_v, l.sv.hist, d_flags);
-      DBBC_LAUNCH_CHECK();
+      launch_overlapped(csr_v_digits_kernel, count_grid(me), 256, 0, s, ku, me, vk, passes_v, l.sv.hist, d_flags);
       uint32_t *vin = l.up0, *vout = l.up1;
       for (int p = 0; p < passes_v; p++, std::swap(in, out), std::swap(vin, vout)) {
         const PassOut po{out, vout, g->col + me, (2ull << bits_u) - 1};
@@ -1042,18 +1045,16 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
     }
     if (n > 0) {
       const DegreeLimits lim{{kNarrowCountLimit, kTinyCountLimit, kQuarterCountLimit, 1}};
-      lower_kernel<<<grid_for(n) + 1, 256, 0, s>>>(g->row_ptr, g->col, l.rowdeg, n, n_u, uv, g->lower, lim,
-                                                   l.res->below, l.res->max_deg, d_flags);
-      DBBC_LAUNCH_CHECK();
-      if (me > 0) {
-        work_kernel<<<grid_for(me), 256, 0, s>>>(ck, g->row_ptr, g->lower,
-                                                 reinterpret_cast<unsigned long long*>(g->work), d_flags);
-        DBBC_LAUNCH_CHECK();
-      }
-      pivots_kernel<<<(unsigned)ceil_div<int64_t>(n, kPivotTile), kRowThreads, 0, s>>>(
-          g->work, g->lower, n, g->tune.light_max_work, g->tune.medium_max_work, l.vk0, l.pr0, l.piv.hist,
-          &l.res->st, l.pivot_state, l.counters + 1, d_flags);
-      DBBC_LAUNCH_CHECK();
+      launch_overlapped(lower_kernel,
+                        grid_for(n) + 1, 256, 0, s, g->row_ptr, g->col, l.rowdeg, n, n_u, uv, g->lower, lim,
+                        l.res->below, l.res->max_deg, d_flags);
+      if (me > 0)
+        launch_overlapped(work_kernel, grid_for(me), 256, 0, s, ck, g->row_ptr, g->lower,
+                          reinterpret_cast<unsigned long long*>(g->work), d_flags);
+      launch_overlapped(pivots_kernel,
+                        (unsigned)ceil_div<int64_t>(n, kPivotTile), kRowThreads, 0, s, g->work, g->lower, n,
+                        g->tune.light_max_work, g->tune.medium_max_work, l.vk0, l.pr0, l.piv.hist, &l.res->st,
+                        l.pivot_state, l.counters + 1, d_flags);
     }
     const PrepResult r = read_back(l.res, s);
     if (r.flags & kPrepInvalid) throw Error{DBBC_EINVAL, "invalid edge id or sign"};
@@ -1072,10 +1073,9 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
     int32_t* ev = sc.get<int32_t>((size_t)m);
     int8_t* es = sc.get<int8_t>((size_t)m);
     DBBC_CUDA(cudaMemsetAsync(d_flags, 0, sizeof(unsigned), s));
-    dedup_kernel<<<(unsigned)ceil_div<int64_t>(m, kRowTile), kRowThreads, 0, s>>>(
-        ku, m, bits_v, n_u, g->vertex, eu, ev, es, reinterpret_cast<uint64_t*>(&l.res->kept), l.dedup_state,
-        l.counters + 2, d_flags);
-    DBBC_LAUNCH_CHECK();
+    launch_overlapped(dedup_kernel,
+                      (unsigned)ceil_div<int64_t>(m, kRowTile), kRowThreads, 0, s, ku, m, bits_v, n_u, g->vertex, eu,
+                      ev, es, reinterpret_cast<uint64_t*>(&l.res->kept), l.dedup_state, l.counters + 2, d_flags);
     const PrepResult d = read_back(l.res, s);
     if (d.flags & kPrepTimeout) throw Error{DBBC_EINTERNAL, "a bounded wait of the build gave up"};
     mu = (int64_t)d.kept;
@@ -1109,7 +1109,8 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
       const PlainLoad in{kin, vin};
       if (p + 1 == passes)
         radix_pass<PlainLoad, true, false, false>(
-            in, PassOut{nullptr, reinterpret_cast<uint32_t*>(g->order), nullptr, 0}, g->n_piv, 0, p, l.piv, d_flags, s);
+            in, PassOut{nullptr, reinterpret_cast<uint32_t*>(g->order), nullptr, 0}, g->n_piv, 0, p, l.piv, d_flags,
+            s);
       else
         radix_pass<PlainLoad, true, true, false>(in, PassOut{kout, vout, nullptr, 0}, g->n_piv, 0, p, l.piv, d_flags,
                                                  s);

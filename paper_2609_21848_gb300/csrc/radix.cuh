@@ -91,15 +91,20 @@ __device__ __forceinline__ T block_excl_scan(T x, T* total) {
   return warp_tot[w] + inc - x;
 }
 
-// Whether this CTA has to return at once (kPrepStop), the same answer in every
-// thread although other CTAs may be setting the flag. Contains __syncthreads.
+// Called first by the build's kernels (see launch_overlapped): whether this CTA
+// has to return at once (kPrepStop), the same answer in every thread although
+// other CTAs may be setting the flag. Contains __syncthreads.
 __device__ __forceinline__ bool cta_stopped(const unsigned* flags) {
+  let_next_start();
+  wait_for_previous();
   return __syncthreads_or(threadIdx.x == 0 && (ld_relaxed(flags) & kPrepStop) != 0) != 0;
 }
 
-// The number of this CTA's tile, the same in every thread, or -1 when the CTA
-// has to return (kPrepStop). Contains __syncthreads.
+// The same for kernels over tiles: the number of this CTA's tile, or -1 when
+// the CTA has to return. Contains __syncthreads.
 __device__ __forceinline__ int64_t take_tile(unsigned* counter, const unsigned* flags) {
+  let_next_start();
+  wait_for_previous();
   __shared__ int64_t tile_sh;
   if (threadIdx.x == 0) tile_sh = (ld_relaxed(flags) & kPrepStop) != 0 ? -1 : (int64_t)atomicAdd(counter, 1u);
   __syncthreads();
@@ -264,9 +269,9 @@ __device__ __forceinline__ unsigned rs_peers(uint32_t d, unsigned valid) {
 constexpr uint32_t kDigitTotal = 0x80000000u;
 
 template <class Load, bool HAS_V, bool WRITE_K, bool AUX>
-__global__ void __launch_bounds__(kRsThreads, DBBC_RS_CTAS) radix_pass_kernel(Load load, PassOut out, int64_t n, int shift,
-                                                                const uint32_t* __restrict__ hist, uint32_t* state,
-                                                                unsigned* counter, unsigned* flags) {
+__global__ void __launch_bounds__(kRsThreads, DBBC_RS_CTAS)
+    radix_pass_kernel(Load load, PassOut out, int64_t n, int shift, const uint32_t* __restrict__ hist, uint32_t* state,
+                      unsigned* counter, unsigned* flags) {
   extern __shared__ __align__(16) unsigned char rs_smem[];
   // warp digit counters first, then the staged tile, in the same memory
   uint32_t* wh = reinterpret_cast<uint32_t*>(rs_smem);
@@ -414,11 +419,10 @@ void radix_pass(const Load& load, const PassOut& out, int64_t n, int begin_bit, 
   auto fn = radix_pass_kernel<Load, HAS_V, WRITE_K, AUX>;
   const size_t staged = (size_t)kRsTile * (8 + (HAS_V ? 4 : 0)), counters = (size_t)kRsWarps * 256 * 4;
   const size_t smem = std::max(staged, counters);
-  DBBC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  (void)resident_ctas((const void*)fn, kRsThreads, smem, smem);
   const int64_t tiles = radix_tiles(n);
-  fn<<<(unsigned)tiles, kRsThreads, smem, s>>>(load, out, n, begin_bit + 8 * pass, st.hist + 256 * pass,
-                                               st.state + (size_t)pass * tiles * 256, st.counters + pass, flags);
-  DBBC_LAUNCH_CHECK();
+  launch_overlapped(fn, tiles, kRsThreads, smem, s, load, out, n, begin_bit + 8 * pass, st.hist + 256 * pass,
+                    st.state + (size_t)pass * tiles * 256, st.counters + pass, flags);
 }
 
 }  // namespace dbbc

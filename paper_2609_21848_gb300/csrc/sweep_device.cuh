@@ -556,7 +556,8 @@ __device__ __forceinline__ void window_clear(int cw, bool fin, uint32_t* cnt, ui
 }
 
 template <int G, bool LIST, bool DEEP>
-__device__ __forceinline__ void window_walk_dispatch(int cw, bool fin, const uint32_t* __restrict__ col, LaneBatch& b, SlotBatch& s,
+__device__ __forceinline__ void window_walk_dispatch(int cw, bool fin, const uint32_t* __restrict__ col,
+                                                     LaneBatch& b, SlotBatch& s,
                                                      const uint2* src, uint32_t n, uint32_t* next, uint2* slots,
                                                      ListState* ls, uint32_t hn, uint32_t rn,
                                                      const Win& w, uint64_t& bal, uint64_t& unb) {
@@ -695,8 +696,8 @@ __device__ __forceinline__ uint64_t sweep_list_item(const CsrView& g, const Swee
         iw.window(s0 + r + 1, lo_n, hi_n, cw_n);
         hn = hi_n << 1;
       }
-      window_walk_dispatch<G, true, false>(cw, fin, g.col, b, sb, lists + (size_t)r * q.L, n, &nbn[r & 1], nullptr, &ls, hn,
-                                    r + 1, w, bal, unb);
+      window_walk_dispatch<G, true, false>(cw, fin, g.col, b, sb, lists + (size_t)r * q.L, n, &nbn[r & 1], nullptr,
+                                           &ls, hn, r + 1, w, bal, unb);
       visits += tid == 0 ? n : 0;
       __syncthreads();  // also publishes the appends to later windows' lists
       if (r + 1 < nwin)

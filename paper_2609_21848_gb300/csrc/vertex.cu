@@ -281,7 +281,8 @@ __device__ __forceinline__ void credit_window(const uint32_t* words, const Win& 
     pu += eu;
   };
   if constexpr (CW == 32) {
-    for (uint32_t k = threadIdx.x; k < whi - wlo; k += kSweepThreads) endpoint(wlo + k, words[2 * k], words[2 * k + 1]);
+    for (uint32_t k = threadIdx.x; k < whi - wlo; k += kSweepThreads) endpoint(wlo + k, words[2 * k],
+                                                                               words[2 * k + 1]);
   } else {
     const uint32_t first = CW == 4 ? wlo & ~3u : CW == 8 ? wlo & ~1u : wlo;  // rank of word 0's first counter
     for (uint32_t k = threadIdx.x; k < w.words; k += kSweepThreads) {
@@ -398,7 +399,8 @@ __device__ __forceinline__ void tips_window(const CsrView& g, const PivotGeom& q
   tips_count<G, CW>(g, q, slots, &sh.next_count, seg, &sh.n_seg, w);
   __syncthreads();
   if (VERT) {
-    credit_window<CW>(words, w, lo, hi, q.base == 0 ? (int64_t)g.n_u : 0, o, pb, pu);  // endpoints share the pivot's side
+    credit_window<CW>(words, w, lo, hi, q.base == 0 ? (int64_t)g.n_u : 0, o, pb,
+                      pu);  // endpoints share the pivot's side
   }
   const uint32_t n = DBBC_CHECK(sh.n_seg <= q.L) ? sh.n_seg : q.L;
   tips_credit<G, CW, VERT, EDGE>(g, q, seg, n, &sh.next_credit, w, o);
@@ -547,10 +549,9 @@ void enqueue_tips(const dbbc_graph* g, cudaStream_t s, const TipOut& o, unsigned
     auto fn = tips_light_kernel<VERT, EDGE>;
     const int slots_log = tier_slots_log(g->tune.light_max_work, g->tune.hash_mult_log, 10);
     const size_t smem = (size_t)kLightWarps * ((size_t)1 << slots_log) * kHashSlotBytes;
-    DBBC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)((size_t)kLightWarps * kLightSlots * kHashSlotBytes)));
     const int64_t want = ceil_div<int64_t>(g->n_light, kLightWarps);
-    const int64_t cap = (int64_t)sms * blocks_per_sm((const void*)fn, kLightWarps * 32, smem);
+    const int64_t cap = (int64_t)sms * resident_ctas((const void*)fn, kLightWarps * 32, smem,
+                                                     (size_t)kLightWarps * kLightSlots * kHashSlotBytes);
     fn<<<(unsigned)std::min(want, cap), kLightWarps * 32, smem, s>>>(
         view, g->order + g->n_hub + g->n_medium, g->work, g->n_light, g->tune.hash_mult_log, slots_log, o, d_status);
     DBBC_LAUNCH_CHECK();
@@ -559,9 +560,8 @@ void enqueue_tips(const dbbc_graph* g, cudaStream_t s, const TipOut& o, unsigned
     auto fn = tips_medium_kernel<VERT, EDGE>;
     const int slots_log = tier_slots_log(g->tune.medium_max_work, g->tune.hash_mult_log, 13);
     const size_t smem = ((size_t)1 << slots_log) * kHashSlotBytes;
-    DBBC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)((size_t)kMediumSlots * kHashSlotBytes)));
-    const int64_t cap = (int64_t)sms * blocks_per_sm((const void*)fn, kMediumThreads, smem);
+    const int64_t cap = (int64_t)sms * resident_ctas((const void*)fn, kMediumThreads, smem,
+                                                     (size_t)kMediumSlots * kHashSlotBytes);
     fn<<<(unsigned)std::min<int64_t>(g->n_medium, cap), kMediumThreads, smem, s>>>(
         view, g->order + g->n_hub, g->work, g->n_medium, g->tune.hash_mult_log, slots_log, o, d_status);
     DBBC_LAUNCH_CHECK();
@@ -569,8 +569,7 @@ void enqueue_tips(const dbbc_graph* g, cudaStream_t s, const TipOut& o, unsigned
   if (g->n_hub > 0) {
     auto fn = tips_sweep_kernel<VERT, EDGE>;
     const size_t smem = kSweepSmem;
-    DBBC_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    const int grid = sms * blocks_per_sm((const void*)fn, kSweepThreads, smem);
+    const int grid = sms * resident_ctas((const void*)fn, kSweepThreads, smem, smem);
     uint2* cursors = sc.get<uint2>((size_t)grid * (size_t)g->sweep_max_lower);
     Segment* segments = sc.get<Segment>((size_t)grid * (size_t)g->sweep_max_lower);
     int* next = sc.get<int>(1);

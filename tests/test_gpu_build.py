@@ -75,3 +75,28 @@ def test_union_components_of_uneven_sizes(sizes):
         bal, unb = dbbc.dbbc_count_components(g)
     want = [oracle.count(*p, n_u, n_v)[:2] if m else (0, 0) for p, (n_u, n_v, m) in zip(parts, sizes)]
     assert list(zip(bal.tolist(), unb.tolist())) == want
+
+
+@pytest.mark.parametrize("entry", ["count_async", "count_noalloc"])
+def test_counts_can_be_captured_and_replayed(entry):
+    """The tiers of a count overlap on the stream; captured into a CUDA graph
+    they keep their order against what comes before and after."""
+    import torch
+    u, v, s = _edges(11, 900, 700, 60_000, 0)
+    want = oracle.count(u, v, s, 900, 700)[:2]
+    count = getattr(dbbc, f"dbbc_{entry}")
+    with dbbc.dbbc_graph_from_coo(u, v, s, 900, 700) as g:
+        info = g.info
+        assert info["n_light"] and info["n_medium"] and info["n_hub"]
+        d_out = torch.zeros(2, dtype=torch.int64, device="cuda")
+        count(g, d_out)  # outside capture first
+        copy = torch.zeros_like(d_out)
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            count(g, d_out)
+            copy.copy_(d_out)
+        for _ in range(3):
+            copy.fill_(-1)
+            graph.replay()
+            torch.cuda.synchronize()
+            assert tuple(copy.tolist()) == want
