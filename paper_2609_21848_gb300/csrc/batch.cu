@@ -167,23 +167,6 @@ __global__ void __launch_bounds__(kMediumThreads) count_medium_batch_kernel(cons
 // otherwise occupy a whole SM each. Measured on GB300 (4,096-graph batch):
 // 64-, 96- and 128-thread narrow CTAs within 1% of each other, 256 threads
 // 12% slower, 512 threads 34% slower.
-#ifndef DBBC_NARROW_THREADS
-#define DBBC_NARROW_THREADS 128
-#endif
-#ifndef DBBC_NARROW_WORDS
-#define DBBC_NARROW_WORDS (6656 + 4)
-#endif
-constexpr int kNarrowThreads = DBBC_NARROW_THREADS;
-constexpr uint32_t kNarrowWords = DBBC_NARROW_WORDS;
-constexpr size_t kNarrowSmem = (size_t)kNarrowWords * 4;
-static_assert(kNarrowWords % 4 == 0, "window buffers are cleared 16 bytes at a time");
-// items above this many estimated wedges stay on wide CTAs (a long item on a
-// narrow CTA would finish last)
-#ifndef DBBC_NARROW_ITEM_WORK
-#define DBBC_NARROW_ITEM_WORK (1u << 20)
-#endif
-constexpr uint64_t kNarrowItemWork = DBBC_NARROW_ITEM_WORK;
-
 template <int THREADS, uint32_t WORDS>
 __global__ void __launch_bounds__(THREADS) hub_sweep_batch_kernel(const GraphDesc* __restrict__ desc,
                                                                   const BatchHubItem* __restrict__ items,

@@ -63,6 +63,25 @@ constexpr int64_t kListCapEntries = int64_t{1} << DBBC_LIST_CAP_LOG;
 // Lemma 1 contribution of every wedge from its atomic's old value.
 constexpr uint64_t kFinalizeWindowWedges = 65536;
 
+// Narrow hub CTAs of batch plans (see hub_sweep_batch_kernel): threads, counter
+// words, and the largest item.
+#ifndef DBBC_NARROW_THREADS
+#define DBBC_NARROW_THREADS 128
+#endif
+#ifndef DBBC_NARROW_WORDS
+#define DBBC_NARROW_WORDS (6656 + 4)
+#endif
+constexpr int kNarrowThreads = DBBC_NARROW_THREADS;
+constexpr uint32_t kNarrowWords = DBBC_NARROW_WORDS;
+constexpr size_t kNarrowSmem = (size_t)kNarrowWords * 4;
+static_assert(kNarrowWords % 4 == 0, "window buffers are cleared 16 bytes at a time");
+// items above this many estimated wedges stay on wide CTAs (a long item on a
+// narrow CTA would finish last)
+#ifndef DBBC_NARROW_ITEM_WORK
+#define DBBC_NARROW_ITEM_WORK (1u << 20)
+#endif
+constexpr uint64_t kNarrowItemWork = DBBC_NARROW_ITEM_WORK;
+
 // Runtime tuning (dbbc_set_tuning), snapshotted into every graph at build.
 struct Tuning {
   uint64_t light_max_work = kLightMaxWork;

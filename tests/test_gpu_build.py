@@ -100,3 +100,31 @@ def test_counts_can_be_captured_and_replayed(entry):
             graph.replay()
             torch.cuda.synchronize()
             assert tuple(copy.tolist()) == want
+
+
+@pytest.mark.parametrize("n_u", [3_300, 3_400, 6_700, 28_700, 57_300, 57_400])
+@pytest.mark.parametrize("finalize", [0, 2**64 - 1])
+def test_hub_windows_at_the_widths_that_fit(n_u, finalize):
+    """Hubs whose endpoint ranks just fit, and just do not fit, one window of
+    32-bit or 16-bit counters on a full and on a narrow CTA: counts of one
+    graph, of a plan and per vertex."""
+    rng = np.random.default_rng(n_u)
+    hubs, n_v = 3, 400
+    u = np.concatenate([rng.integers(0, n_u - hubs, 4 * n_u), np.repeat(np.arange(n_u - hubs, n_u), n_v)])
+    v = np.concatenate([rng.integers(0, n_v, 4 * n_u), np.tile(np.arange(n_v), hubs)])
+    key = np.unique(u.astype(np.int64) * n_v + v)
+    u, v = (key // n_v).astype(np.int32), (key % n_v).astype(np.int32)
+    s = np.where(rng.random(u.shape[0]) < 0.7, 1, -1).astype(np.int8)
+    base = dbbc.dbbc_get_tuning()
+    try:
+        dbbc.dbbc_set_tuning({"finalize_window_wedges": finalize, "light_max_work": 64, "medium_max_work": 64})
+        with dbbc.dbbc_graph_from_coo(u, v, s, n_u, n_v) as g:
+            got = dbbc.dbbc_count(g)
+            with dbbc.dbbc_batch_create([g]) as b:
+                plan = tuple(int(x[0]) for x in dbbc.dbbc_batch_count(b))
+            vb, vu = dbbc.dbbc_count_vertices(g)
+    finally:
+        dbbc.dbbc_set_tuning(base)
+    want = oracle.count(u, v, s, n_u, n_v)[:2]
+    assert got == want and plan == want
+    assert (int(vb.sum(dtype=np.uint64)), int(vu.sum(dtype=np.uint64))) == (4 * want[0], 4 * want[1])
