@@ -234,10 +234,12 @@ static int64_t hub_full_grid() {
 }
 
 // The hub sweep on `grid` CTAs with per-CTA cursors (sweep_max_lower each)
-// and, if `lists` is given, per-CTA list scratch (sweep_list_cap slots each).
-static void launch_hub(const dbbc_graph* g, const CsrView& view, cudaStream_t s, int grid, uint2* cursors,
+// and, if `lists` is given, per-CTA list scratch (sweep_list_cap slots each);
+// `next` is the item counter, cleared here.
+static void launch_hub(const dbbc_graph* g, const CsrView& view, cudaStream_t s, int grid, int* next, uint2* cursors,
                        uint2* lists, unsigned long long* d_out, CountScratch* d, bool count_visits) {
-  hub_sweep_kernel<<<grid, kSweepThreads, kSweepSmem, s>>>(view, g->sweep_items, g->n_sweep_items, &d->next, cursors,
+  DBBC_CUDA(cudaMemsetAsync(next, 0, sizeof(int), s));
+  hub_sweep_kernel<<<grid, kSweepThreads, kSweepSmem, s>>>(view, g->sweep_items, g->n_sweep_items, next, cursors,
                                                            g->sweep_max_lower, lists, lists ? g->sweep_list_cap : 0,
                                                            d_out, count_visits ? &d->visits : nullptr);
   DBBC_LAUNCH_CHECK();
@@ -253,8 +255,9 @@ void enqueue_count(const dbbc_graph* g, cudaStream_t s, unsigned long long* d_ou
     const int grid = (int)hub_full_grid();
     uint2* cursors = sc.get<uint2>((size_t)grid * (size_t)g->sweep_max_lower);
     uint2* lists = g->sweep_list_cap > 0 ? sc.get<uint2>((size_t)grid * (size_t)g->sweep_list_cap) : nullptr;
+    int* next = sc.get<int>(1);
     if (prof) t0 = prof->begin(s);
-    launch_hub(g, view, s, grid, cursors, lists, d_out, d, prof != nullptr);
+    launch_hub(g, view, s, grid, next, cursors, lists, d_out, d, prof != nullptr);
     if (prof) {
       prof->end(CountProfiler::HUB_AGG, t0, s);
       prof->launches[CountProfiler::HUB_AGG]++;
@@ -299,7 +302,7 @@ void enqueue_count_prealloc(const dbbc_graph* g, cudaStream_t s, unsigned long l
   }
   if (g->n_hub > 0) {
     const int grid = (int)std::min<int64_t>(hub_full_grid(), hub_grid);
-    launch_hub(g, view, s, grid, reinterpret_cast<uint2*>(cursors), nullptr, d_out, d, false);
+    launch_hub(g, view, s, grid, &d->next, reinterpret_cast<uint2*>(cursors), nullptr, d_out, d, false);
   }
   if (g->n_medium > 0) launch_medium(g, view, s, d_out, &d->status, g->n_hub == 0);
   if (g->n_light > 0) launch_light(g, view, s, d_out, &d->status, g->n_hub + g->n_medium == 0);

@@ -229,8 +229,8 @@ struct CountProfiler {
 };
 
 // Device words of one count, all zero before it: its result when the caller
-// has no device output, the list-mode visits, the status word and the hub item
-// counter.
+// has no device output, the list-mode visits, the status word and (for callers
+// that supply all scratch) the hub item counter.
 struct CountScratch {
   unsigned long long out[2];
   unsigned long long visits;
