@@ -15,6 +15,7 @@ namespace dbbc {
 
 struct GraphDesc {
   const int64_t* row_ptr;
+  const uint2* span;
   const uint32_t* col;
   const uint32_t* lower;
   const uint64_t* work;
@@ -42,7 +43,7 @@ struct GatherJob {
 };
 
 __device__ __forceinline__ CsrView view_of(const GraphDesc& d) {
-  return CsrView{d.row_ptr, d.col, d.lower, d.n_u, d.n, d.nnz};
+  return CsrView{d.row_ptr, d.span, d.col, d.lower, d.n_u, d.n, d.nnz};
 }
 
 // One CTA per graph copies its medium and light pivots into the batch lists.
@@ -405,7 +406,7 @@ static size_t medium_smem_bytes(const dbbc_batch* b) { return ((size_t)1 << b->m
 static void plan_components(dbbc_batch* b, const dbbc_graph* g) {
   cudaStream_t s = b->stream;
   std::vector<GraphDesc> desc((size_t)b->n_graphs,
-                              GraphDesc{g->row_ptr, g->col, g->lower, g->work, g->n, g->nnz, g->n_u,
+                              GraphDesc{g->row_ptr, g->span, g->col, g->lower, g->work, g->n, g->nnz, g->n_u,
                                         g->tune.hash_mult_log});
   b->n_medium = g->n_medium;
   b->n_light = g->n_light;
@@ -429,7 +430,7 @@ static void plan_batch(dbbc_batch* b, const dbbc_graph* const* gs) {
   int64_t n_items = 0;
   for (int32_t i = 0; i < n; i++) {
     const dbbc_graph* g = gs[i];
-    desc[(size_t)i] = GraphDesc{g->row_ptr, g->col, g->lower, g->work, g->n, g->nnz, g->n_u, g->tune.hash_mult_log};
+    desc[(size_t)i] = GraphDesc{g->row_ptr, g->span, g->col, g->lower, g->work, g->n, g->nnz, g->n_u, g->tune.hash_mult_log};
     jobs[(size_t)i] = GatherJob{g->order, g->n_hub, g->n_medium, g->n_light, b->n_medium, b->n_light};
     b->n_medium += g->n_medium;
     b->n_light += g->n_light;
@@ -564,7 +565,7 @@ void count_subset(const dbbc_graph* g, cudaStream_t s, const std::vector<int32_t
   uint64_t h[2] = {0, 0};
   try {
     DBBC_CUDA(cudaGetDevice(&b->device));
-    std::vector<GraphDesc> desc(1, GraphDesc{g->row_ptr, g->col, g->lower, g->work, g->n, g->nnz, g->n_u,
+    std::vector<GraphDesc> desc(1, GraphDesc{g->row_ptr, g->span, g->col, g->lower, g->work, g->n, g->nnz, g->n_u,
                                               g->tune.hash_mult_log});
     b->n_medium = (int64_t)medium_rows.size();
     b->n_light = (int64_t)light_rows.size();

@@ -248,7 +248,7 @@ static void launch_hub(const dbbc_graph* g, const CsrView& view, cudaStream_t s,
 void enqueue_count(const dbbc_graph* g, cudaStream_t s, unsigned long long* d_out, CountScratch* d, Scratch& sc,
                    CountProfiler* prof) {
   if (g->n_piv == 0) return;
-  const CsrView view{g->row_ptr, g->col, g->lower, g->n_u, g->n, g->nnz};
+  const CsrView view{g->row_ptr, g->span, g->col, g->lower, g->n_u, g->n, g->nnz};
   cudaEvent_t t_all = prof ? prof->begin(s) : nullptr;
   cudaEvent_t t0 = nullptr;
   if (g->n_hub > 0) {
@@ -293,7 +293,7 @@ void enqueue_count_prealloc(const dbbc_graph* g, cudaStream_t s, unsigned long l
   DBBC_CUDA(cudaMemsetAsync(d, 0, sizeof(CountScratch), s));
   DBBC_CUDA(cudaMemsetAsync(d_out, 0, 2 * sizeof(unsigned long long), s));
   if (g->n_piv == 0) return;
-  const CsrView view{g->row_ptr, g->col, g->lower, g->n_u, g->n, g->nnz};
+  const CsrView view{g->row_ptr, g->span, g->col, g->lower, g->n_u, g->n, g->nnz};
   int64_t hub_grid = 0;
   if (g->n_hub > 0) {
     const size_t per_cta = (size_t)g->sweep_max_lower * sizeof(uint2);

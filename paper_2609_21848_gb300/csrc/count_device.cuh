@@ -83,20 +83,20 @@ __device__ __forceinline__ PivotGeom pivot_geom(const CsrView& g, int32_t p) {
   return q;
 }
 
-// Row [b, en) of the vertex of the other side named by the CSR entry e of a
-// pivot with geometry q, and the sign bit of their edge. Checked builds test
-// the row index and bounds; a failed test gives an empty row.
-__device__ __forceinline__ uint32_t neighbour_row(const CsrView& g, const PivotGeom& q, uint32_t e, int64_t& b,
-                                                  int64_t& en) {
+// Span [b, en) of the row of the vertex of the other side named by the CSR
+// entry e of a pivot with geometry q. Checked builds test the row index and
+// bounds; a failed test gives an empty span.
+__device__ __forceinline__ void neighbour_row(const CsrView& g, const PivotGeom& q, uint32_t e, uint32_t& b,
+                                              uint32_t& en) {
   const int64_t vrow = q.base + (e >> 1);
+  b = en = 0;
   if (DBBC_CHECK(vrow >= 0 && vrow < g.n)) {
-    b = g.row_ptr[vrow];
-    en = g.row_ptr[vrow + 1];
-    if (!DBBC_CHECK(b >= 0 && b <= en && en <= g.nnz)) en = b;
-  } else {
-    b = en = 0;
+    const uint2 s = g.span[vrow];
+    if (DBBC_CHECK((int64_t)s.x >= g.row_ptr[vrow] && s.x <= s.y && (int64_t)s.y <= g.row_ptr[vrow + 1])) {
+      b = s.x;
+      en = s.y;
+    }
   }
-  return e & 1u;
 }
 
 // Hash tiers: groups of G lanes (group gid of `groups`) take lower neighbours
@@ -124,12 +124,7 @@ __device__ __forceinline__ void group_walk(uint32_t gid, uint32_t groups, const 
   const uint32_t* __restrict__ col = g.col;
   auto bounds = [&](bool ok, uint32_t e, uint32_t& c, uint32_t& en) {
     c = en = 0;
-    if (ok) {
-      int64_t b, n;
-      neighbour_row(g, q, e, b, n);
-      c = (uint32_t)b;
-      en = (uint32_t)n;
-    }
+    if (ok) neighbour_row(g, q, e, c, en);
   };
   uint32_t i = gid;
   uint32_t e = i < q.L ? col[q.rb + i] : 0u;

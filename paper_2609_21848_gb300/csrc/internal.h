@@ -128,8 +128,8 @@ constexpr int16_t kItemList = 2;  // list mode: visit a neighbour only in window
 // counters of a window are finalised when it is cleared (C(p,2) + C(q,2) and
 // p*q per endpoint) instead of wedge by wedge
 constexpr int16_t kItemFinalize = 4;
-// the item starts at its hub's first accepted rank: no row lists a rank below
-// it, so a neighbour's cursor starts at the row's first entry (no search)
+// the item starts at its hub's first accepted rank: no span lists a rank below
+// it, so a neighbour's cursor starts at its span's first entry (no search)
 constexpr int16_t kItemFirst = 8;
 // Counts below this fit the 8-bit halves of a tiny counter, and below the
 // next the 4-bit halves of a quarter counter.
@@ -145,8 +145,12 @@ constexpr size_t kColPad = 512;
 // V vertices in ascending priority. A row lists its neighbours by ascending
 // priority as (side_rank << 1) | negative; the first lower[r] of them have
 // lower priority than the row's vertex.
+// span[r] is the part of row r that can end a butterfly's wedge: {first, end}
+// positions of its entries of degree 2 and more (a row starts with its
+// endpoints of degree 1, which are in no butterfly); a union's rows are whole.
 struct CsrView {
   const int64_t* row_ptr;
+  const uint2* span;
   const uint32_t* col;
   const uint32_t* lower;
   int32_t n_u;
@@ -168,6 +172,7 @@ struct dbbc_graph {
   int64_t* row_ptr = nullptr;  // [n + 1]
   uint32_t* col = nullptr;     // [nnz]
   uint32_t* lower = nullptr;   // [n]
+  uint2* span = nullptr;       // [n] see CsrView
   int32_t* vertex = nullptr;   // [n] unified id per row
   uint64_t* work = nullptr;    // [n] accepted wedges per pivot row
   int32_t* order = nullptr;    // [n_piv] pivot rows, descending work: hubs | medium | light

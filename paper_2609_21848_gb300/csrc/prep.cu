@@ -150,8 +150,8 @@ __global__ void __launch_bounds__(kRowThreads) ranks_kernel(const uint64_t* __re
                                                             int32_t* __restrict__ rowdeg,
                                                             int64_t* __restrict__ row_ptr,
                                                             int32_t* __restrict__ component,
-                                                            uint64_t* __restrict__ work, uint64_t* state,
-                                                            unsigned* counter, unsigned* flags) {
+                                                            uint64_t* __restrict__ work, int64_t* lone,
+                                                            uint64_t* state, unsigned* counter, unsigned* flags) {
   __shared__ uint64_t tot_sh;
   const int64_t tile = take_tile(counter, flags);
   if (tile < 0) return;
@@ -171,6 +171,10 @@ __global__ void __launch_bounds__(kRowThreads) ranks_kernel(const uint64_t* __re
       const int64_t local = (int64_t)(k & id_mask);
       const int32_t x = side ? (int32_t)(n_u + un.vo(c) + local) : (int32_t)(un.uo(c) + local);
       d[j] = (uint32_t)((k >> bits_id) & deg_mask);
+      if (d[j] < 2u && un.n_graphs == 1) {  // the side's last one sets the side's count
+        const int64_t end = side ? n : n_u;
+        if (r + 1 == end || ((skey[r + 1] >> bits_id) & deg_mask) >= 2u) lone[side] = r + 1 - (side ? n_u : 0);
+      }
       if (DBBC_CHECK(x >= 0 && x < n)) {
         vertex[r] = x;
         side_rank[x] = side ? (int32_t)(r - n_u) : (int32_t)r;
@@ -318,13 +322,14 @@ struct CsrKeys {
 // The last CTA instead finds, per side, how many vertices have degree below
 // each of four limits (ranks ascend by degree within a side): below[2k] for U,
 // below[2k + 1] for V; and the largest degree, that of some component's last
-// rank.
+// rank. Also writes the rows' spans (see CsrView).
 struct DegreeLimits {
   int32_t d[4];
 };
 __global__ void lower_kernel(const int64_t* __restrict__ row_ptr, const uint32_t* __restrict__ col,
                              const int32_t* __restrict__ rowdeg, int64_t n, int32_t n_u, UnionView un,
-                             uint32_t* __restrict__ lower, DegreeLimits lim, int64_t* below,
+                             uint32_t* __restrict__ lower, uint2* __restrict__ span, const int64_t* lone,
+                             DegreeLimits lim, int64_t* below,
                              unsigned* max_deg, const unsigned* flags) {
   if (cta_stopped(flags)) return;
   if (blockIdx.x == gridDim.x - 1) {
@@ -353,8 +358,12 @@ __global__ void lower_kernel(const int64_t* __restrict__ row_ptr, const uint32_t
       const int64_t b = un.uo(c), e = un.uo(c + 1);
       t = b + upper_bound_dev<int32_t>(rowdeg + b, e - b, d);
     }
-    const int64_t b = row_ptr[r];
-    lower[r] = (uint32_t)lower_bound_dev<uint32_t>(col + b, row_ptr[r + 1] - b, (uint32_t)(t << 1));
+    const int64_t b = row_ptr[r], e = row_ptr[r + 1];
+    lower[r] = (uint32_t)lower_bound_dev<uint32_t>(col + b, e - b, (uint32_t)(t << 1));
+    const uint32_t from = (uint32_t)(lone[r < n_u ? 1 : 0] << 1);  // the other side's first rank of degree 2
+    int64_t skip = 0;
+    if (from && b < e && col[b] < from) skip = lower_bound_dev<uint32_t>(col + b, e - b, from);
+    span[r] = make_uint2((uint32_t)(b + skip), (uint32_t)e);
   }
 }
 
@@ -438,6 +447,7 @@ struct PrepResult {
   PrepStats st;
   HubStats hubs;
   int64_t below[8];         // vertices of degree below four limits (lower_kernel)
+  int64_t lone[2];          // a plain graph's vertices of degree 0 and 1 (ranks_kernel)
   unsigned max_deg[2];      // largest degree of each side (lower_kernel)
   unsigned long long kept;  // distinct edges (dedup_kernel)
   unsigned flags;           // kPrep*
@@ -559,7 +569,7 @@ struct HubPlanner {
   const int32_t* order;
   const uint32_t* lower;
   const uint64_t* work;
-  const int64_t* below;  // vertices of degree below 2^16, 2^8, 2^4 and 1 (U, V each)
+  const int64_t* below;  // vertices of degree below 2^16, 2^8, 2^4 and 2 (U, V each)
   int64_t n_hub;
   int32_t n_u;
   UnionView un;
@@ -602,8 +612,9 @@ __device__ __forceinline__ HubPlan plan_hub(const HubPlanner& hp, int64_t i) {
   // side's first endpoint of degree >= 2^4, tiny (8-bit) ones those below
   // degree 2^8 and narrow (16-bit) ones those below degree 2^16; for a union,
   // whose ranks are component-major, only L bounds the counts. Endpoints of
-  // degree 0 (the lowest ranks) are in no row, so the windows start after
-  // them. A hub whose endpoints all fit one window of wider counters takes
+  // degree 0 and 1 (the lowest ranks) are in no span, so the windows start
+  // after them: a fifth of the 20M U vertices of the 300M-edge polarized
+  // graph, whose sweep that took from 515 to 496 ms. A hub whose endpoints all fit one window of wider counters takes
   // that instead of a window per width: fewer (neighbour, window) visits and
   // barriers, and a 32-bit half that is a word of its own is the cheapest to
   // count in (the class of a wedge picks the word and the increment is 1), if
@@ -616,7 +627,8 @@ __device__ __forceinline__ HubPlan plan_hub(const HubPlanner& hp, int64_t i) {
   auto clamp_rank = [&](int64_t x) { return max(start, min(sp, (uint64_t)max(x, (int64_t)0))); };
   const uint64_t first = plain ? clamp_rank(below[6]) : start;
   uint64_t quarter_end = L < (uint32_t)kQuarterCountLimit ? sp : plain ? max(first, clamp_rank(below[4])) : first;
-  uint64_t tiny_end = L < (uint32_t)kTinyCountLimit ? sp : plain ? max(quarter_end, clamp_rank(below[2])) : quarter_end;
+  uint64_t tiny_end = L < (uint32_t)kTinyCountLimit ? sp : plain ? max(quarter_end,
+                                                                       clamp_rank(below[2])) : quarter_end;
   uint64_t narrow_end = L < (uint32_t)kNarrowCountLimit ? sp : plain ? max(tiny_end, clamp_rank(below[0])) : tiny_end;
   const uint64_t H4 = 4ull * kSweepWindow16, H8 = 2ull * kSweepWindow16;
   const double fin = (double)hp.tune.finalize_window_wedges;
@@ -1008,6 +1020,7 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
   g->row_ptr = static_cast<int64_t*>(graph_alloc(g, (size_t)(n + 1) * 8));
   g->lower = static_cast<uint32_t*>(graph_alloc(g, (size_t)n * 4));
   g->work = static_cast<uint64_t*>(graph_alloc(g, (size_t)n * 8));
+  g->span = static_cast<uint2*>(graph_alloc(g, (size_t)n * sizeof(uint2)));
   if (n == 0) DBBC_CUDA(cudaMemsetAsync(g->row_ptr, 0, 8, s));
 
   // a1-a4 for an edge list, without a wait: validation and degrees, Def. 3
@@ -1031,7 +1044,7 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
                                                   bits_lid, p, l.rank, d_flags, s);
       launch_overlapped(ranks_kernel,
                         (unsigned)ceil_div<int64_t>(n, kRowTile), kRowThreads, 0, s, in, n, n_u, bits_comp, bits_deg,
-                        bits_lid, uv, g->vertex, l.side_rank, l.rowdeg, g->row_ptr, g->component, g->work,
+                        bits_lid, uv, g->vertex, l.side_rank, l.rowdeg, g->row_ptr, g->component, g->work, l.res->lone,
                         l.row_state, l.counters, d_flags);
     }
     CsrKeys ck{nullptr, nullptr, me, n_u, bits_u};
@@ -1065,9 +1078,10 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
       ck.upos = vin;
     }
     if (n > 0) {
-      const DegreeLimits lim{{kNarrowCountLimit, kTinyCountLimit, kQuarterCountLimit, 1}};
+      const DegreeLimits lim{{kNarrowCountLimit, kTinyCountLimit, kQuarterCountLimit, 2}};
       launch_overlapped(lower_kernel,
-                        grid_for(n) + 1, 256, 0, s, g->row_ptr, g->col, l.rowdeg, n, n_u, uv, g->lower, lim,
+                        grid_for(n) + 1, 256, 0, s, g->row_ptr, g->col, l.rowdeg, n, n_u, uv, g->lower, g->span,
+                        l.res->lone, lim,
                         l.res->below, l.res->max_deg, d_flags);
       if (me > 0)
         launch_overlapped(work_kernel, grid_for(me), 256, 0, s, ck, g->row_ptr, g->lower,

@@ -309,19 +309,17 @@ __device__ __forceinline__ bool lean_walk(const uint32_t* __restrict__ col, uint
 // same slots in per-window lists.
 __device__ __forceinline__ void lean_cursor_start(const CsrView& g, const PivotGeom& q, uint32_t i, uint32_t lo_rank,
                                                   uint32_t& b_out, uint32_t& en_out, uint32_t& s1_out) {
-  int64_t b, en;
-  s1_out = neighbour_row(g, q, g.col[q.rb + i], b, en);
-  const uint32_t first = lo_rank << 1;
-  if (first) {  // lower_bound of `first` in the row
-    int64_t lo = b, hi = en;
+  const uint32_t e = g.col[q.rb + i], first = lo_rank << 1;
+  s1_out = e & 1u;
+  neighbour_row(g, q, e, b_out, en_out);
+  if (first) {  // lower_bound of `first` in the span
+    uint32_t lo = b_out, hi = en_out;
     while (lo < hi) {
-      const int64_t mid = (lo + hi) >> 1;
+      const uint32_t mid = lo + ((hi - lo) >> 1);
       if (g.col[mid] < first) lo = mid + 1; else hi = mid;
     }
-    b = lo;
+    b_out = lo;
   }
-  b_out = (uint32_t)b;
-  en_out = (uint32_t)en;
 }
 
 __device__ __forceinline__ uint2 lean_slot(uint32_t c, uint32_t en, uint32_t s1) {

@@ -543,7 +543,7 @@ __global__ void edge_query_kernel(CsrView g, const int32_t* __restrict__ row_of,
 template <bool VERT, bool EDGE>
 void enqueue_tips(const dbbc_graph* g, cudaStream_t s, const TipOut& o, unsigned* d_status, Scratch& sc) {
   if (g->n_piv == 0) return;
-  const CsrView view{g->row_ptr, g->col, g->lower, g->n_u, g->n, g->nnz};
+  const CsrView view{g->row_ptr, g->span, g->col, g->lower, g->n_u, g->n, g->nnz};
   const int sms = num_sms();
   if (g->n_light > 0) {
     auto fn = tips_light_kernel<VERT, EDGE>;
@@ -662,7 +662,7 @@ extern "C" dbbc_status dbbc_count_edges(const dbbc_graph* g, void* cuda_stream, 
       ob = sc.get<unsigned long long>((size_t)(2 * k));
       ou = ob + k;
     }
-    const CsrView view{g->row_ptr, g->col, g->lower, g->n_u, g->n, g->nnz};
+    const CsrView view{g->row_ptr, g->span, g->col, g->lower, g->n_u, g->n, g->nnz};
     edge_query_kernel<<<grid_1d(k), 256, 0, s>>>(view, row_of, dqu, dqv, k, o.eb, o.eu, ob, ou, d_status + 1);
     DBBC_LAUNCH_CHECK();
     if (!on_device) {
