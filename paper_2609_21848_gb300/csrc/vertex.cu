@@ -353,16 +353,21 @@ __device__ __forceinline__ void tips_credit(const CsrView& g, const PivotGeom& q
     // would spread them over G sectors: 28.5 instead of 19.8 ms of sweep on the
     // 20M-edge rating graph). Vertices: four entries per lane by one load.
     constexpr uint32_t kLane = EDGE ? 1u : 4u, kItem = EDGE ? (uint32_t)G : 1u;
-    for (uint32_t j = 0; j < trips; j++) {
-      const uint32_t pos = start + j * (4u * G) + gl * kLane;
-      uint32_t x[kLU] = {0u, 0u, 0u, 0u};
+    auto load = [&](uint32_t pos, uint32_t (&x)[kLU]) {
       if constexpr (EDGE) {
 #pragma unroll
-        for (int u = 0; u < kLU; u++)
-          if (pos + u * kItem < t.end) x[u] = __ldg(g.col + pos + u * kItem);
+        for (int u = 0; u < kLU; u++) x[u] = pos + u * kItem < t.end ? __ldg(g.col + pos + u * kItem) : 0u;
       } else {
+        x[0] = x[1] = x[2] = x[3] = 0u;
         if (pos < t.end) lean_load(g.col, pos, x);
       }
+    };
+    uint32_t pos = start + gl * kLane;
+    uint32_t x[kLU];
+    load(pos, x);
+    for (uint32_t j = 0; j < trips; j++, pos += 4u * G) {
+      uint32_t y[kLU];
+      load(pos + 4u * G, y);  // the next chunk, while this one is credited
 #pragma unroll
       for (int u = 0; u < kLU; u++) {
         if (pos + u * kItem - t.c < len) {
@@ -372,6 +377,7 @@ __device__ __forceinline__ void tips_credit(const CsrView& g, const PivotGeom& q
           sb += own - 1u;
           su += other;
         }
+        x[u] = y[u];
       }
     }
 #pragma unroll
