@@ -99,7 +99,8 @@ __global__ void __launch_bounds__(kMediumThreads) count_medium_kernel(CsrView g,
 // (list_cap slots per CTA); with no room for them (list_cap below three slots
 // per lower neighbour) it is swept by cursors like every other item, which
 // gives the same counts.
-__global__ void __launch_bounds__(kSweepThreads) hub_sweep_kernel(CsrView g, const SweepItem* __restrict__ items,
+template <class S>
+__global__ void __launch_bounds__(S::kThreads, FullShape::kThreads / S::kThreads) hub_sweep_kernel(CsrView g, const SweepItem* __restrict__ items,
                                                                       int64_t n_items, int* next_item,
                                                                       uint2* __restrict__ cursors, int64_t cur_cap,
                                                                       uint2* __restrict__ lists, int64_t list_cap,
@@ -110,10 +111,10 @@ __global__ void __launch_bounds__(kSweepThreads) hub_sweep_kernel(CsrView g, con
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sweep_smem);
   let_next_start();
   __shared__ int item_sh;
-  __shared__ ListState ls;
+  __shared__ ListState<S> ls;
   __shared__ uint32_t nbn[2];
   const int tid = threadIdx.x;
-  zero_words(cnt_words, kSweepWords);
+  zero_words<S::kThreads>(cnt_words, S::kWords);
   if (tid < 2) nbn[tid] = 0u;
   uint2* cur = cursors + (int64_t)blockIdx.x * cur_cap;
   uint2* my_lists = lists ? lists + (int64_t)blockIdx.x * list_cap : nullptr;
@@ -132,16 +133,17 @@ __global__ void __launch_bounds__(kSweepThreads) hub_sweep_kernel(CsrView g, con
       continue;
     }
     const uint32_t L = DBBC_CHECK((int64_t)q.L <= cur_cap) ? q.L : 0u;  // checked builds: cursor capacity
-    for (uint32_t i = tid; i < L; i += kSweepThreads) {
+    for (uint32_t i = tid; i < L; i += S::kThreads) {
       uint32_t b, en, s1;
       lean_cursor_start(g, q, i, (item.flags & kItemFirst) ? 0u : item.lo, b, en, s1);
       cur[i] = lean_slot(b, en, s1);
     }
     __syncthreads();
-    sweep_cursor_item_dispatch(item.group_log, g.col, L, cur, ItemWindows(item), (item.flags & kItemFinalize) != 0,
-                               sbase, cnt_words, nbn, bal, unb);
+    sweep_cursor_item_dispatch<S::kThreads, S::kWords>(item.group_log, g.col, L, cur, typename S::Windows(item),
+                                                       (item.flags & kItemFinalize) != 0, sbase, cnt_words, nbn, bal,
+                                                       unb);
   }
-  block_add_pair<kSweepThreads>(bal, unb, out);
+  block_add_pair<S::kThreads>(bal, unb, out);
   if (visits && tid == 0 && n_visits) atomicAdd(visits, (unsigned long long)n_visits);
   wait_for_previous();
 }
@@ -227,10 +229,13 @@ static void launch_medium(const dbbc_graph* g, const CsrView& view, cudaStream_t
               g->order + g->n_hub, g->work, g->n_medium, g->tune.hash_mult_log, slots_log, d_out, d_status);
 }
 
-// CTAs the hub sweep can keep resident (one per SM: its counters fill the
-// SM's shared memory).
-static int64_t hub_full_grid() {
-  return (int64_t)num_sms() * resident_ctas((const void*)hub_sweep_kernel, kSweepThreads, kSweepSmem, kSweepSmem);
+// CTAs the hub sweep can keep resident (their counters fill the SM's shared
+// memory: one full or two half CTAs per SM).
+static int64_t hub_full_grid(const dbbc_graph* g) {
+  return num_sms() * (g->half_ctas ? (int64_t)resident_ctas((const void*)hub_sweep_kernel<HalfShape>, kHalfThreads,
+                                                            HalfShape::kSmem, HalfShape::kSmem)
+                                   : (int64_t)resident_ctas((const void*)hub_sweep_kernel<FullShape>, kSweepThreads,
+                                                            kSweepSmem, kSweepSmem));
 }
 
 // The hub sweep on `grid` CTAs with per-CTA cursors (sweep_max_lower each)
@@ -239,9 +244,14 @@ static int64_t hub_full_grid() {
 static void launch_hub(const dbbc_graph* g, const CsrView& view, cudaStream_t s, int grid, int* next, uint2* cursors,
                        uint2* lists, unsigned long long* d_out, CountScratch* d, bool count_visits) {
   DBBC_CUDA(cudaMemsetAsync(next, 0, sizeof(int), s));
-  hub_sweep_kernel<<<grid, kSweepThreads, kSweepSmem, s>>>(view, g->sweep_items, g->n_sweep_items, next, cursors,
-                                                           g->sweep_max_lower, lists, lists ? g->sweep_list_cap : 0,
-                                                           d_out, count_visits ? &d->visits : nullptr);
+  const int64_t list_cap = lists ? g->sweep_list_cap : 0;
+  unsigned long long* visits = count_visits ? &d->visits : nullptr;
+  if (g->half_ctas)
+    hub_sweep_kernel<HalfShape><<<grid, kHalfThreads, HalfShape::kSmem, s>>>(
+        view, g->sweep_items, g->n_sweep_items, next, cursors, g->sweep_max_lower, lists, list_cap, d_out, visits);
+  else
+    hub_sweep_kernel<FullShape><<<grid, kSweepThreads, kSweepSmem, s>>>(
+        view, g->sweep_items, g->n_sweep_items, next, cursors, g->sweep_max_lower, lists, list_cap, d_out, visits);
   DBBC_LAUNCH_CHECK();
 }
 
@@ -252,7 +262,7 @@ void enqueue_count(const dbbc_graph* g, cudaStream_t s, unsigned long long* d_ou
   cudaEvent_t t_all = prof ? prof->begin(s) : nullptr;
   cudaEvent_t t0 = nullptr;
   if (g->n_hub > 0) {
-    const int grid = (int)hub_full_grid();
+    const int grid = (int)hub_full_grid(g);
     uint2* cursors = sc.get<uint2>((size_t)grid * (size_t)g->sweep_max_lower);
     uint2* lists = g->sweep_list_cap > 0 ? sc.get<uint2>((size_t)grid * (size_t)g->sweep_list_cap) : nullptr;
     int* next = sc.get<int>(1);
@@ -301,7 +311,7 @@ void enqueue_count_prealloc(const dbbc_graph* g, cudaStream_t s, unsigned long l
     if (hub_grid < 1) throw Error{DBBC_EOVERFLOW, "hub cursors exceed the fixed scratch"};
   }
   if (g->n_hub > 0) {
-    const int grid = (int)std::min<int64_t>(hub_full_grid(), hub_grid);
+    const int grid = (int)std::min<int64_t>(hub_full_grid(g), hub_grid);
     launch_hub(g, view, s, grid, &d->next, reinterpret_cast<uint2*>(cursors), nullptr, d_out, d, false);
   }
   if (g->n_medium > 0) launch_medium(g, view, s, d_out, &d->status, g->n_hub == 0);

@@ -243,57 +243,61 @@ __device__ __forceinline__ void zero_words(uint32_t* w, uint32_t words) {
 // neighbours (a count never exceeds either). CW = 4: four endpoints per word,
 // each (asym << 4) | sym, four times the ranks, where counts stay below 16.
 // CW = 32: one 64-bit word per endpoint, half the ranks.
-template <int CW>
+// W16: the window's 16-bit counters (kSweepWindow16, or kHalfWindow16 in the half
+// CTAs of small graphs).
+template <int CW, uint32_t W16 = kSweepWindow16>
 __host__ __device__ constexpr uint32_t window_ranks() {
-  return CW == 4 ? 4 * kSweepWindow16 : CW == 8 ? 2 * kSweepWindow16 : CW == 16 ? kSweepWindow16 : kSweepWindow32;
+  return CW == 4 ? 4 * W16 : CW == 8 ? 2 * W16 : CW == 16 ? W16 : W16 / 2;
 }
 
 // The windows of a work item: quarter ones over [lo, qe), tiny ones over
 // [qe, te), narrow ones over [te, ne), wide ones over [ne, hi), numbered in
 // rank order.
-struct ItemWindows {
+template <uint32_t W16>
+struct ItemWindowsOf {
   uint32_t lo, qe, te, ne, hi;
   uint32_t rq, rt, rn, rw;
-  ItemWindows() = default;
-  __device__ __forceinline__ explicit ItemWindows(const SweepItem& it) {
+  ItemWindowsOf() = default;
+  __device__ __forceinline__ explicit ItemWindowsOf(const SweepItem& it) {
     lo = it.lo;
     hi = it.hi;
     qe = min(max(it.q_end, lo), hi);
     te = min(max(it.t_end, qe), hi);
     ne = min(max(it.n_end, te), hi);
-    rq = (qe - lo + window_ranks<4>() - 1) / window_ranks<4>();
-    rt = (te - qe + window_ranks<8>() - 1) / window_ranks<8>();
-    rn = (ne - te + window_ranks<16>() - 1) / window_ranks<16>();
-    rw = (hi - ne + window_ranks<32>() - 1) / window_ranks<32>();
+    rq = (qe - lo + window_ranks<4, W16>() - 1) / window_ranks<4, W16>();
+    rt = (te - qe + window_ranks<8, W16>() - 1) / window_ranks<8, W16>();
+    rn = (ne - te + window_ranks<16, W16>() - 1) / window_ranks<16, W16>();
+    rw = (hi - ne + window_ranks<32, W16>() - 1) / window_ranks<32, W16>();
   }
   __device__ __forceinline__ uint32_t count() const { return rq + rt + rn + rw; }
   // window r: its ranks [wlo, whi) and counter width
   __device__ __forceinline__ void window(uint32_t r, uint32_t& wlo, uint32_t& whi, int& cw) const {
     if (r < rq) {
-      wlo = lo + r * window_ranks<4>();
-      whi = min(wlo + window_ranks<4>(), qe);
+      wlo = lo + r * window_ranks<4, W16>();
+      whi = min(wlo + window_ranks<4, W16>(), qe);
       cw = 4;
     } else if (r < rq + rt) {
-      wlo = qe + (r - rq) * window_ranks<8>();
-      whi = min(wlo + window_ranks<8>(), te);
+      wlo = qe + (r - rq) * window_ranks<8, W16>();
+      whi = min(wlo + window_ranks<8, W16>(), te);
       cw = 8;
     } else if (r < rq + rt + rn) {
-      wlo = te + (r - rq - rt) * window_ranks<16>();
-      whi = min(wlo + window_ranks<16>(), ne);
+      wlo = te + (r - rq - rt) * window_ranks<16, W16>();
+      whi = min(wlo + window_ranks<16, W16>(), ne);
       cw = 16;
     } else {
-      wlo = ne + (r - rq - rt - rn) * window_ranks<32>();
-      whi = min(wlo + window_ranks<32>(), hi);
+      wlo = ne + (r - rq - rt - rn) * window_ranks<32, W16>();
+      whi = min(wlo + window_ranks<32, W16>(), hi);
       cw = 32;
     }
   }
   // the window holding rank x (lo <= x < hi)
   __device__ __forceinline__ uint32_t index_of(uint32_t x) const {
-    if (x < qe) return (x - lo) / window_ranks<4>();
-    if (x < te) return rq + (x - qe) / window_ranks<8>();
-    if (x < ne) return rq + rt + (x - te) / window_ranks<16>();
-    return rq + rt + rn + (x - ne) / window_ranks<32>();
+    if (x < qe) return (x - lo) / window_ranks<4, W16>();
+    if (x < te) return rq + (x - qe) / window_ranks<8, W16>();
+    if (x < ne) return rq + rt + (x - te) / window_ranks<16, W16>();
+    return rq + rt + rn + (x - ne) / window_ranks<32, W16>();
   }
 };
+using ItemWindows = ItemWindowsOf<kSweepWindow16>;
 
 }  // namespace dbbc

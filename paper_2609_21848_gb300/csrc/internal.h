@@ -29,6 +29,11 @@ constexpr int kMediumSlots = 8192;
 constexpr uint32_t kSweepWindow16 = DBBC_SWEEP_WINDOW16;     // 32-bit counters packing two 16-bit halves
 constexpr uint32_t kSweepWindow32 = DBBC_SWEEP_WINDOW16 / 2;  // 64-bit counters packing two 32-bit halves
 constexpr uint64_t kSweepItemWork = 1u << 20;  // target accepted wedges per work item
+// Half CTAs of the hub sweep: half the threads and half the window, two per SM,
+// for small graphs (see plan_hubs in prep.cu).
+constexpr int kHalfThreads = 512;
+constexpr uint32_t kHalfWindow16 = 28416;
+constexpr int64_t kHalfMaxSide = int64_t{1} << 17;
 // mean (neighbour, window) segment length at which 32 / 16 / 8 / 4 lanes walk a segment
 #ifndef DBBC_GROUP_T32
 #define DBBC_GROUP_T32 40
@@ -186,6 +191,7 @@ struct dbbc_graph {
   int64_t n_sweep_items = 0;
   int64_t sweep_max_lower = 0;  // largest lower-neighbour count of a hub (cursor scratch per CTA)
   int64_t sweep_list_cap = 0;   // largest windows x lower neighbours of a list-mode item (list slots per CTA)
+  bool half_ctas = false;       // the sweep's CTAs: full, or two half ones per SM
   int64_t max_deg_u = 0, max_deg_v = 0;            // largest degree of each side
   // disjoint union of several graphs (dbbc_graph_from_coo_multi): component
   // of every row, 0 for a plain handle (n_components == 1)

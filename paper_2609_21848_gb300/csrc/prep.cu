@@ -574,6 +574,7 @@ struct HubPlanner {
   int32_t n_u;
   UnionView un;
   Tuning tune;
+  uint32_t window16;  // 16-bit counters of a window
 };
 
 // 32-bit counters for a whole hub need this many wedges per counter.
@@ -584,17 +585,18 @@ struct HubPlan {
   uint64_t first, sp, W;
   uint64_t rq, rt, rn, windows;  // quarter, tiny and narrow windows, all windows
   uint64_t spans;
-  uint32_t L;
+  uint32_t L, window16;
   uint64_t span_windows;     // list mode: windows whose lists fit the scratch
 };
 
 // The first rank of window w of the hub (windows numbered in rank order over
 // the quarter, tiny, narrow and wide parts).
 __device__ __forceinline__ uint64_t window_start(const HubPlan& p, uint64_t w) {
-  if (w < p.rq) return p.first + w * 4ull * kSweepWindow16;
-  if (w < p.rq + p.rt) return p.it.q_end + (w - p.rq) * 2ull * kSweepWindow16;
-  if (w < p.rq + p.rt + p.rn) return p.it.t_end + (w - p.rq - p.rt) * kSweepWindow16;
-  return min(p.sp, (uint64_t)p.it.n_end + (w - p.rq - p.rt - p.rn) * kSweepWindow32);
+  const uint64_t w16 = p.window16;
+  if (w < p.rq) return p.first + w * 4 * w16;
+  if (w < p.rq + p.rt) return p.it.q_end + (w - p.rq) * 2 * w16;
+  if (w < p.rq + p.rt + p.rn) return p.it.t_end + (w - p.rq - p.rt) * w16;
+  return min(p.sp, (uint64_t)p.it.n_end + (w - p.rq - p.rt - p.rn) * (w16 / 2));
 }
 
 __device__ __forceinline__ HubPlan plan_hub(const HubPlanner& hp, int64_t i) {
@@ -630,10 +632,10 @@ __device__ __forceinline__ HubPlan plan_hub(const HubPlanner& hp, int64_t i) {
   uint64_t tiny_end = L < (uint32_t)kTinyCountLimit ? sp : plain ? max(quarter_end,
                                                                        clamp_rank(below[2])) : quarter_end;
   uint64_t narrow_end = L < (uint32_t)kNarrowCountLimit ? sp : plain ? max(tiny_end, clamp_rank(below[0])) : tiny_end;
-  const uint64_t H4 = 4ull * kSweepWindow16, H8 = 2ull * kSweepWindow16;
+  const uint64_t full = hp.window16, H4 = 4 * full, H8 = 2 * full;
   const double fin = (double)hp.tune.finalize_window_wedges;
   {  // wider counters where they fit one window
-    const uint64_t ranks = sp - first, full = kSweepWindow16;
+    const uint64_t ranks = sp - first;
     uint64_t words = max(min(quarter_end - first, H4) >> 2, min(tiny_end - quarter_end, H8) >> 1);
     words = max(words, max(min(narrow_end - tiny_end, full), 2 * min(sp - narrow_end, full / 2)));
     // (a narrow CTA's item keeps fitting one)
@@ -647,8 +649,9 @@ __device__ __forceinline__ HubPlan plan_hub(const HubPlanner& hp, int64_t i) {
   }
   p.rq = (quarter_end - first + H4 - 1) / H4;
   p.rt = (tiny_end - quarter_end + H8 - 1) / H8;
-  p.rn = (narrow_end - tiny_end + kSweepWindow16 - 1) / kSweepWindow16;
-  const uint64_t rw = (sp - narrow_end + kSweepWindow32 - 1) / kSweepWindow32;
+  p.rn = (narrow_end - tiny_end + full - 1) / full;
+  const uint64_t rw = (sp - narrow_end + full / 2 - 1) / (full / 2);
+  p.window16 = hp.window16;
   p.windows = p.rq + p.rt + p.rn + rw;
   p.first = first;
   p.sp = sp;
@@ -803,12 +806,23 @@ struct Carver {
 
 // Plans the hubs on the device, behind the pivot sort; returns once the
 // items are counted. Throws when a bounded wait of the build gave up.
-static void plan_hubs(dbbc_graph* g, cudaStream_t s, const UnionView& un, PrepResult* res, Scratch& sc) {
+static void plan_hubs(dbbc_graph* g, cudaStream_t s, const UnionView& un, PrepResult* res, uint64_t max_work,
+                      Scratch& sc) {
   if (g->n_hub == 0) return;
+  // Two half CTAs per SM hide each other's barriers and window ends, at the
+  // price of up to twice the windows. They pay where the sides are small and no
+  // hub alone would keep a half CTA busy past the others' end: hub sweeps of a
+  // 1M-edge graph 0.198 -> 0.167 ms and of a 1.7M-edge one 0.301 -> 0.241 ms;
+  // where one large hub outlasts the rest (151k edges) 0.101 -> 0.129 ms, with
+  // larger sides (9.2M edges, 540k vertices) 3.8 -> 4.8 ms.
+  const int64_t half_ctas = 2 * (int64_t)num_sms();
+  g->half_ctas = std::max(g->n_u, g->n_v) <= kHalfMaxSide &&
+                 max_work <= 4 * (g->wedges_hub / (uint64_t)half_ctas);
   // a hub has at most W / hub_item_work items, rounded up, and no more than windows
   const uint64_t side = (uint64_t)std::max(g->n_u, g->n_v);
+  const uint32_t window16 = g->half_ctas ? kHalfWindow16 : kSweepWindow16;
   const uint64_t cap = std::min((uint64_t)g->n_hub + g->wedges_hub / g->tune.hub_item_work,
-                                (uint64_t)g->n_hub * (side / kSweepWindow32 + 4));
+                                (uint64_t)g->n_hub * (side / (window16 / 2) + 4));
   const int64_t tiles = ceil_div<int64_t>(g->n_hub, kRowThreads);
   struct Layout {
     RadixState sort;
@@ -838,7 +852,7 @@ static void plan_hubs(dbbc_graph* g, cudaStream_t s, const UnionView& un, PrepRe
   carver.used = 0;
   const Layout l = place(carver);
   DBBC_CUDA(cudaMemsetAsync(zero, 0, l.zeroed, s));
-  const HubPlanner hp{g->order, g->lower, g->work, res->below, g->n_hub, g->n_u, un, g->tune};
+  const HubPlanner hp{g->order, g->lower, g->work, res->below, g->n_hub, g->n_u, un, g->tune, window16};
   launch_overlapped(plan_hubs_kernel,
                     (unsigned)tiles, kRowThreads, 0, s, hp, l.items, cap, l.key, l.idx, l.sort.hist, &res->hubs,
                     l.state, l.counter, &res->flags);
@@ -1153,7 +1167,7 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
   }
   g->max_deg_u = r.max_deg[0];
   g->max_deg_v = r.max_deg[1];
-  plan_hubs(g, s, uv, l.res, sc);
+  plan_hubs(g, s, uv, l.res, st.max_work, sc);
   if (read_back(d_flags, s) & kPrepTimeout) throw Error{DBBC_EINTERNAL, "a bounded wait of the build gave up"};
 }
 

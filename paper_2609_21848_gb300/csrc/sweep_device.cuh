@@ -44,6 +44,19 @@ constexpr int kLU = 4;
 constexpr uint32_t kSweepWords = kSweepWindow16 + 4;
 constexpr size_t kSweepSmem = (size_t)kSweepWords * 4;
 
+// The sweep's CTA shapes: threads, 16-bit counters of a window, counter words.
+template <int THREADS, uint32_t W16>
+struct SweepShape {
+  static constexpr int kThreads = THREADS;
+  static constexpr uint32_t kWindow16 = W16;
+  static constexpr uint32_t kWords = W16 + 4;
+  static constexpr size_t kSmem = (size_t)kWords * 4;
+  using Windows = ItemWindowsOf<W16>;
+};
+using FullShape = SweepShape<kSweepThreads, kSweepWindow16>;
+using HalfShape = SweepShape<kHalfThreads, kHalfWindow16>;
+static_assert(kHalfWindow16 % 4 == 0 && kListMaxWindows <= kHalfThreads, "half CTAs");
+
 // A window of side ranks [wlo, whi): entries below h lie in it (cursors start
 // at its first rank), and the counter word of rank r is at shared byte address
 // wb + (r >> 2) * 4 (4-bit counters, four ranks per word, aligned to a
@@ -336,6 +349,7 @@ __device__ __forceinline__ uint2 lean_slot(uint32_t c, uint32_t en, uint32_t s1)
 // the item, or to no list at the end of its row or of the item. A neighbour is
 // in at most one list at a time and in each list at most once, so L slots
 // per list never overflow.
+template <class S>
 struct ListState {
   uint2* lists;                // [Rsub][L] window lists of the span
   uint2* over;                 // [L] neighbours waiting for the next span
@@ -343,7 +357,7 @@ struct ListState {
   int ocnt;                    // overflow list length
   uint32_t L;
   uint32_t nwin;               // windows (lists) of the span
-  ItemWindows iw;              // the item's windows
+  typename S::Windows iw;      // the item's windows
   uint32_t s0;                 // first window of the span
   uint32_t hl;                 // (last rank of the span + 1) << 1
   uint32_t item_hl;            // (last rank of the item + 1) << 1
@@ -352,7 +366,8 @@ struct ListState {
 // Queue a neighbour whose cursor c (row end en, edge sign s1) stopped at entry
 // x (see ListState). Most neighbours go on in the very next window: entries
 // below hn (twice its end rank; 0: none in this span) go to list rn.
-__device__ __forceinline__ void list_queue(ListState& ls, uint32_t x, uint32_t c, uint32_t en, uint32_t s1,
+template <class S>
+__device__ __forceinline__ void list_queue(ListState<S>& ls, uint32_t x, uint32_t c, uint32_t en, uint32_t s1,
                                            uint32_t hn, uint32_t rn) {
   const uint2 slot = lean_slot(c, en, s1);
   uint32_t r = rn;
@@ -419,9 +434,9 @@ __device__ __forceinline__ void window_fetch(const uint32_t* __restrict__ col, c
 // Walk a batch in window w. Cursor mode (LIST false) writes each neighbour's
 // new position back to its slot in `slots`; list mode queues the neighbour by
 // its next entry.
-template <int G, int CW, bool RET, bool LIST>
+template <int G, int CW, bool RET, bool LIST, class LS>
 __device__ __forceinline__ void batch_walk(const uint32_t* __restrict__ col, LaneBatch& b, uint32_t n, uint2* slots,
-                                           ListState* ls, uint32_t hn, uint32_t rn, const Win& w, uint64_t& bal,
+                                           LS* ls, uint32_t hn, uint32_t rn, const Win& w, uint64_t& bal,
                                            uint64_t& unb) {
   const int gl = threadIdx.x & (G - 1);
   const uint32_t i = b.base + lane_id() / G;
@@ -440,9 +455,9 @@ __device__ __forceinline__ void batch_walk(const uint32_t* __restrict__ col, Lan
 // All n slots of one window: the warp's first batches were fetched already
 // (possibly while the previous window was being cleared); the warp then
 // fetches and walks batches until the slots run out. hn, rn: see list_queue.
-template <int G, int CW, bool RET, bool LIST, bool DEEP>
+template <int G, int CW, bool RET, bool LIST, bool DEEP, class LS>
 __device__ __forceinline__ void window_walk(const uint32_t* __restrict__ col, LaneBatch& b, SlotBatch& s,
-                                            const uint2* src, uint32_t n, uint32_t* next, uint2* slots, ListState* ls,
+                                            const uint2* src, uint32_t n, uint32_t* next, uint2* slots, LS* ls,
                                             uint32_t hn, uint32_t rn, const Win& w, uint64_t& bal, uint64_t& unb) {
   while (b.base < n) {  // warp-uniform
     if constexpr (DEEP) {
@@ -553,11 +568,11 @@ __device__ __forceinline__ void window_clear(int cw, bool fin, uint32_t* cnt, ui
   }
 }
 
-template <int G, bool LIST, bool DEEP>
+template <int G, bool LIST, bool DEEP, class LS>
 __device__ __forceinline__ void window_walk_dispatch(int cw, bool fin, const uint32_t* __restrict__ col,
                                                      LaneBatch& b, SlotBatch& s,
                                                      const uint2* src, uint32_t n, uint32_t* next, uint2* slots,
-                                                     ListState* ls, uint32_t hn, uint32_t rn,
+                                                     LS* ls, uint32_t hn, uint32_t rn,
                                                      const Win& w, uint64_t& bal, uint64_t& unb) {
   if (cw == 4) {
     if (fin) window_walk<G, 4, false, LIST, DEEP>(col, b, s, src, n, next, slots, ls, hn, rn, w, bal, unb);
@@ -582,11 +597,11 @@ __device__ __forceinline__ void window_walk_dispatch(int cw, bool fin, const uin
 // chunks) and only then clear the counters, which hides that load latency
 // behind the clear.
 // THREADS and WORDS: the CTA's threads and counter words.
-template <int G, int THREADS = kSweepThreads, uint32_t WORDS = kSweepWords>
+template <int G, int THREADS, uint32_t WORDS, class IW>
 __device__ __forceinline__ void sweep_cursor_item(const uint32_t* __restrict__ col, uint32_t L, uint2* cur,
-                                                  const ItemWindows& iw, bool fin, uint32_t sbase, uint32_t* cnt_words,
+                                                  const IW& iw, bool fin, uint32_t sbase, uint32_t* cnt_words,
                                                   uint32_t* nbn, uint64_t& bal, uint64_t& unb) {
-  constexpr bool kDeep = THREADS < kSweepThreads;
+  constexpr bool kDeep = THREADS == kNarrowThreads;
   const uint32_t R = iw.count();
   LaneBatch b;
   SlotBatch sb;
@@ -596,7 +611,8 @@ __device__ __forceinline__ void sweep_cursor_item(const uint32_t* __restrict__ c
     int cw;
     iw.window(r, lo, hi, cw);
     const Win w = make_win<WORDS>(cw, lo, hi, sbase);
-    window_walk_dispatch<G, false, kDeep>(cw, fin, col, b, sb, cur, L, &nbn[r & 1], cur, nullptr, 0u, 0u, w, bal, unb);
+    window_walk_dispatch<G, false, kDeep>(cw, fin, col, b, sb, cur, L, &nbn[r & 1], cur, static_cast<ListState<FullShape>*>(nullptr),
+                                           0u, 0u, w, bal, unb);
     __syncthreads();
     if (r + 1 < R) window_fetch<G, kDeep>(col, cur, L, &nbn[(r + 1) & 1], b, sb);
     window_clear<THREADS>(cw, fin, cnt_words, w.words, bal, unb);
@@ -605,9 +621,9 @@ __device__ __forceinline__ void sweep_cursor_item(const uint32_t* __restrict__ c
   }
 }
 
-template <int THREADS = kSweepThreads, uint32_t WORDS = kSweepWords>
+template <int THREADS, uint32_t WORDS, class IW>
 __device__ __forceinline__ void sweep_cursor_item_dispatch(int group_log, const uint32_t* __restrict__ col,
-                                                           uint32_t L, uint2* cur, const ItemWindows& iw, bool fin,
+                                                           uint32_t L, uint2* cur, const IW& iw, bool fin,
                                                            uint32_t sbase, uint32_t* cnt_words, uint32_t* nbn,
                                                            uint64_t& bal, uint64_t& unb) {
   switch (group_log) {
@@ -626,12 +642,12 @@ __device__ __forceinline__ void sweep_cursor_item_dispatch(int group_log, const 
 // lies past the current span waits in an overflow list and is queued when its
 // span starts. Windows end as in sweep_cursor_item. Returns the visits
 // (listed neighbours), counted by thread 0.
-template <int G>
+template <int G, class S>
 __device__ __forceinline__ uint64_t sweep_list_item(const CsrView& g, const SweepItem& item, const PivotGeom& q,
-                                                    uint2* lists, int64_t list_cap, ListState& ls, uint32_t sbase,
+                                                    uint2* lists, int64_t list_cap, ListState<S>& ls, uint32_t sbase,
                                                     uint32_t* cnt_words, uint32_t* nbn, uint64_t& bal, uint64_t& unb) {
   const int tid = threadIdx.x;
-  const ItemWindows iw(item);
+  const typename S::Windows iw(item);
   const uint32_t R = iw.count();
   const bool fin = (item.flags & kItemFinalize) != 0;
   const int64_t per_nb = list_cap / (int64_t)q.L;
@@ -667,13 +683,13 @@ __device__ __forceinline__ uint64_t sweep_list_item(const CsrView& g, const Swee
     if (tid < kListMaxWindows) ls.cnt[tid] = 0;
     __syncthreads();
     if (s0 == 0) {  // each neighbour joins the list of the window of its first entry
-      for (uint32_t i = tid; i < q.L; i += kSweepThreads) {
+      for (uint32_t i = tid; i < q.L; i += S::kThreads) {
         uint32_t b, en, s1;
         lean_cursor_start(g, q, i, (item.flags & kItemFirst) ? 0u : item.lo, b, en, s1);
         if (b < en) list_queue(ls, g.col[b], b, en, s1, 0u, 0u);
       }
     } else {  // the neighbours that waited for this span
-      for (uint32_t j = tid; j < n_in; j += kSweepThreads) {
+      for (uint32_t j = tid; j < n_in; j += S::kThreads) {
         const uint2 e = over_in[j];
         const uint32_t c = e.x, en = e.x + (e.y & 0x7FFFFFFFu);
         if (DBBC_CHECK(c < en && (int64_t)en <= g.nnz)) list_queue(ls, g.col[c], c, en, e.y >> 31, 0u, 0u);
@@ -685,7 +701,7 @@ __device__ __forceinline__ uint64_t sweep_list_item(const CsrView& g, const Swee
     window_fetch<G, false>(g.col, lists, listed(0), &nbn[0], b, sb);
     for (uint32_t r = 0; r < nwin; r++) {
       iw.window(s0 + r, wlo, whi, cw);
-      const Win w = make_win(cw, wlo, whi, sbase);
+      const Win w = make_win<S::kWords>(cw, wlo, whi, sbase);
       const uint32_t n = listed(r);
       uint32_t hn = 0;  // twice the end rank of the span's next window
       if (r + 1 < nwin) {
@@ -700,7 +716,7 @@ __device__ __forceinline__ uint64_t sweep_list_item(const CsrView& g, const Swee
       __syncthreads();  // also publishes the appends to later windows' lists
       if (r + 1 < nwin)
         window_fetch<G, false>(g.col, lists + (size_t)(r + 1) * q.L, listed(r + 1), &nbn[(r + 1) & 1], b, sb);
-      window_clear(cw, fin, cnt_words, w.words, bal, unb);
+      window_clear<S::kThreads>(cw, fin, cnt_words, w.words, bal, unb);
       if (tid == 0) nbn[r & 1] = 0u;
       __syncthreads();
     }
@@ -709,16 +725,17 @@ __device__ __forceinline__ uint64_t sweep_list_item(const CsrView& g, const Swee
   return visits;
 }
 
+template <class S>
 __device__ __forceinline__ uint64_t sweep_list_item_dispatch(const CsrView& g, const SweepItem& item,
                                                              const PivotGeom& q, uint2* lists, int64_t list_cap,
-                                                             ListState& ls, uint32_t sbase, uint32_t* cnt_words,
+                                                             ListState<S>& ls, uint32_t sbase, uint32_t* cnt_words,
                                                              uint32_t* nbn, uint64_t& bal, uint64_t& unb) {
   switch (item.group_log) {
-    case 0: return sweep_list_item<1>(g, item, q, lists, list_cap, ls, sbase, cnt_words, nbn, bal, unb);
-    case 2: return sweep_list_item<4>(g, item, q, lists, list_cap, ls, sbase, cnt_words, nbn, bal, unb);
-    case 3: return sweep_list_item<8>(g, item, q, lists, list_cap, ls, sbase, cnt_words, nbn, bal, unb);
-    case 4: return sweep_list_item<16>(g, item, q, lists, list_cap, ls, sbase, cnt_words, nbn, bal, unb);
-    default: return sweep_list_item<32>(g, item, q, lists, list_cap, ls, sbase, cnt_words, nbn, bal, unb);
+    case 0: return sweep_list_item<1, S>(g, item, q, lists, list_cap, ls, sbase, cnt_words, nbn, bal, unb);
+    case 2: return sweep_list_item<4, S>(g, item, q, lists, list_cap, ls, sbase, cnt_words, nbn, bal, unb);
+    case 3: return sweep_list_item<8, S>(g, item, q, lists, list_cap, ls, sbase, cnt_words, nbn, bal, unb);
+    case 4: return sweep_list_item<16, S>(g, item, q, lists, list_cap, ls, sbase, cnt_words, nbn, bal, unb);
+    default: return sweep_list_item<32, S>(g, item, q, lists, list_cap, ls, sbase, cnt_words, nbn, bal, unb);
   }
 }
 

@@ -128,3 +128,24 @@ def test_hub_windows_at_the_widths_that_fit(n_u, finalize):
     want = oracle.count(u, v, s, n_u, n_v)[:2]
     assert got == want and plan == want
     assert (int(vb.sum(dtype=np.uint64)), int(vu.sum(dtype=np.uint64))) == (4 * want[0], 4 * want[1])
+
+
+@pytest.mark.parametrize("n_u,n_v,m", [(131_072, 3_000, 600_000), (131_073, 3_000, 600_000), (30_000, 28_416, 900_000)])
+@pytest.mark.parametrize("list_density", [0.0, 1e9])
+def test_counts_on_full_and_half_ctas(n_u, n_v, m, list_density):
+    """Graphs on both sides of the size up to which the hub sweep runs half
+    CTAs, with cursors and with neighbour lists."""
+    rng = np.random.default_rng(n_u)
+    w = rng.pareto(1.2, n_v) + 1
+    key = np.unique(rng.integers(0, n_u, m).astype(np.int64) * n_v + rng.choice(n_v, m, p=w / w.sum()))
+    u, v = (key // n_v).astype(np.int32), (key % n_v).astype(np.int32)
+    s = np.where(rng.random(u.shape[0]) < 0.7, 1, -1).astype(np.int8)
+    base = dbbc.dbbc_get_tuning()
+    try:
+        dbbc.dbbc_set_tuning({"list_density": list_density, "light_max_work": 32, "medium_max_work": 128})
+        with dbbc.dbbc_graph_from_coo(u, v, s, n_u, n_v) as g:
+            assert g.info["n_hub"] > 304
+            got = dbbc.dbbc_count(g)
+    finally:
+        dbbc.dbbc_set_tuning(base)
+    assert got == oracle.count(u, v, s, n_u, n_v, threads=8)[:2]
