@@ -430,7 +430,8 @@ static void plan_batch(dbbc_batch* b, const dbbc_graph* const* gs) {
   int64_t n_items = 0;
   for (int32_t i = 0; i < n; i++) {
     const dbbc_graph* g = gs[i];
-    desc[(size_t)i] = GraphDesc{g->row_ptr, g->span, g->col, g->lower, g->work, g->n, g->nnz, g->n_u, g->tune.hash_mult_log};
+    desc[(size_t)i] = GraphDesc{g->row_ptr, g->span, g->col, g->lower, g->work, g->n, g->nnz, g->n_u,
+                                g->tune.hash_mult_log};
     jobs[(size_t)i] = GatherJob{g->order, g->n_hub, g->n_medium, g->n_light, b->n_medium, b->n_light};
     b->n_medium += g->n_medium;
     b->n_light += g->n_light;

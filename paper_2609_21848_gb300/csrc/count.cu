@@ -100,12 +100,10 @@ __global__ void __launch_bounds__(kMediumThreads) count_medium_kernel(CsrView g,
 // per lower neighbour) it is swept by cursors like every other item, which
 // gives the same counts.
 template <class S>
-__global__ void __launch_bounds__(S::kThreads, FullShape::kThreads / S::kThreads) hub_sweep_kernel(CsrView g, const SweepItem* __restrict__ items,
-                                                                      int64_t n_items, int* next_item,
-                                                                      uint2* __restrict__ cursors, int64_t cur_cap,
-                                                                      uint2* __restrict__ lists, int64_t list_cap,
-                                                                      unsigned long long* out,
-                                                                      unsigned long long* visits) {
+__global__ void __launch_bounds__(S::kThreads, FullShape::kThreads / S::kThreads)
+    hub_sweep_kernel(CsrView g, const SweepItem* __restrict__ items, int64_t n_items, int* next_item,
+                     uint2* __restrict__ cursors, int64_t cur_cap, uint2* __restrict__ lists, int64_t list_cap,
+                     unsigned long long* out, unsigned long long* visits) {
   extern __shared__ __align__(16) unsigned char sweep_smem[];
   uint32_t* cnt_words = reinterpret_cast<uint32_t*>(sweep_smem);
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(sweep_smem);

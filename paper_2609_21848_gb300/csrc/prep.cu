@@ -640,10 +640,10 @@ __device__ __forceinline__ HubPlan plan_hub(const HubPlanner& hp, int64_t i) {
     words = max(words, max(min(narrow_end - tiny_end, full), 2 * min(sp - narrow_end, full / 2)));
     // (a narrow CTA's item keeps fitting one)
     const uint64_t limit = W <= kNarrowItemWork && words + 1 <= kNarrowWords ? (uint64_t)kNarrowWords : full;
-    const bool one = (quarter_end > first) + (tiny_end > quarter_end) + (narrow_end > tiny_end) + (sp > narrow_end) <= 1;
+    const int widths = (quarter_end > first) + (tiny_end > quarter_end) + (narrow_end > tiny_end) + (sp > narrow_end);
     if (2 * ranks <= limit && W >= kWideWedgesPerRank * ranks && (double)W >= fin) {
       quarter_end = tiny_end = narrow_end = first;
-    } else if (!one && ranks <= limit && narrow_end == sp) {
+    } else if (widths > 1 && ranks <= limit && narrow_end == sp) {
       quarter_end = tiny_end = first;
     }
   }

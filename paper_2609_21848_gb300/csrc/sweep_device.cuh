@@ -611,8 +611,8 @@ __device__ __forceinline__ void sweep_cursor_item(const uint32_t* __restrict__ c
     int cw;
     iw.window(r, lo, hi, cw);
     const Win w = make_win<WORDS>(cw, lo, hi, sbase);
-    window_walk_dispatch<G, false, kDeep>(cw, fin, col, b, sb, cur, L, &nbn[r & 1], cur, static_cast<ListState<FullShape>*>(nullptr),
-                                           0u, 0u, w, bal, unb);
+    window_walk_dispatch<G, false, kDeep>(cw, fin, col, b, sb, cur, L, &nbn[r & 1], cur,
+                                          static_cast<ListState<FullShape>*>(nullptr), 0u, 0u, w, bal, unb);
     __syncthreads();
     if (r + 1 < R) window_fetch<G, kDeep>(col, cur, L, &nbn[(r + 1) & 1], b, sb);
     window_clear<THREADS>(cw, fin, cnt_words, w.words, bal, unb);

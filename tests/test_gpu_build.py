@@ -132,7 +132,7 @@ def test_hub_windows_at_the_widths_that_fit(n_u, finalize):
 
 @pytest.mark.parametrize("n_u,n_v,m", [(131_072, 3_000, 600_000), (131_073, 3_000, 600_000), (30_000, 28_416, 900_000)])
 @pytest.mark.parametrize("list_density", [0.0, 1e9])
-def test_counts_on_full_and_half_ctas(n_u, n_v, m, list_density):
+def test_counts_on_whole_and_half_ctas(n_u, n_v, m, list_density):
     """Graphs on both sides of the size up to which the hub sweep runs half
     CTAs, with cursors and with neighbour lists."""
     rng = np.random.default_rng(n_u)
