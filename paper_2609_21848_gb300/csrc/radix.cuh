@@ -106,7 +106,10 @@ __device__ __forceinline__ int64_t take_tile(unsigned* counter, const unsigned* 
   let_next_start();
   wait_for_previous();
   __shared__ int64_t tile_sh;
-  if (threadIdx.x == 0) tile_sh = (ld_relaxed(flags) & kPrepStop) != 0 ? -1 : (int64_t)atomicAdd(counter, 1u);
+  if (threadIdx.x == 0) {
+    const unsigned t = atomicAdd(counter, 1u);  // both requests in flight together
+    tile_sh = (ld_relaxed(flags) & kPrepStop) != 0 ? -1 : (int64_t)t;
+  }
   __syncthreads();
   return tile_sh;
 }
@@ -280,6 +283,8 @@ __global__ void __launch_bounds__(kRsThreads, DBBC_RS_CTAS)
   __shared__ uint32_t bstart[256], gofs[256];
   __shared__ uint32_t tot_sh;
   __shared__ int ok_sh;
+  for (int i = threadIdx.x; i < kRsWarps * 256; i += kRsThreads) wh[i] = 0;
+  if (threadIdx.x == 0) ok_sh = 1;
   const int64_t tile = take_tile(counter, flags);
   if (tile < 0) return;
   const int w = threadIdx.x >> 5;
@@ -299,9 +304,6 @@ __global__ void __launch_bounds__(kRsThreads, DBBC_RS_CTAS)
   // exclusive prefix of the digit's count over smaller digits
   const uint32_t digit_base =
       block_excl_scan<uint32_t, kRsThreads>(threadIdx.x < 256 ? hist[threadIdx.x] : 0u, &tot_sh);
-  for (int i = threadIdx.x; i < kRsWarps * 256; i += kRsThreads) wh[i] = 0;
-  if (threadIdx.x == 0) ok_sh = 1;
-  __syncthreads();
 
   // rank within the warp, item by item in input order
   const unsigned lt_mask = (1u << lane) - 1u;
