@@ -143,6 +143,7 @@ void launch_overlapped(void (*kernel)(P...), int64_t grid, int threads, size_t s
 
 // ---------------------------------------------------------------- allocator
 void* dev_alloc(size_t bytes, cudaStream_t s);
+void* scratch_alloc(size_t bytes, cudaStream_t s);  // for the length of one call
 void dev_free(void* p, cudaStream_t s);
 
 // Scratch allocations released (stream-ordered) when the scope ends.
@@ -155,7 +156,7 @@ class Scratch {
   template <typename T>
   T* get(size_t n) {
     if (n == 0) n = 1;
-    void* p = dev_alloc(n * sizeof(T), s_);
+    void* p = scratch_alloc(n * sizeof(T), s_);
     if (!p) throw Error{DBBC_ENOMEM, "Scratch::get"};
     ptrs_.push_back(p);
     return static_cast<T*>(p);
