@@ -132,7 +132,9 @@ DBBC_API dbbc_status dbbc_count_vertices(const dbbc_graph* g, void* cuda_stream,
  * per pair.
  *   qu, qv, balanced_e, unbalanced_e : k entries each, all four HOST or all
  *       four DEVICE memory per `flags` (DBBC_INPUT_HOST / DBBC_INPUT_DEVICE).
- * Device scratch: 16 bytes per CSR entry (2m) plus 4 bytes per vertex.
+ * Device scratch: at most 16 bytes per CSR entry (2m), 8 when the product of
+ * the two sides' largest degrees is below 2^32, plus 4 bytes per vertex and 24
+ * bytes per SM and lower neighbour of the largest hub.
  * Synchronous. Errors: DBBC_EINVAL (NULL graph or array, k < 0, unknown
  * flags, an id out of range), DBBC_ENOMEM, DBBC_ECUDA, DBBC_EINTERNAL. */
 DBBC_API dbbc_status dbbc_count_edges(const dbbc_graph* g, void* cuda_stream, const int32_t* qu, const int32_t* qv,
@@ -261,7 +263,7 @@ DBBC_API dbbc_status dbbc_graph_export(const dbbc_graph* g, void* cuda_stream, i
 /* Device allocator hook (e.g. a framework's caching allocator). alloc returns
  * NULL on failure. Passing NULL for both restores the default: stream-ordered
  * allocations (cudaMallocFromPoolAsync) from one memory pool per device owned
- * by the library, which keeps up to 8 GiB of freed memory mapped between
+ * by the library, which keeps up to 32 GiB of freed memory mapped between
  * calls instead of returning it to the device at every synchronization.
  * Not thread-safe against concurrent library calls. */
 DBBC_API void dbbc_set_allocator(void* (*alloc_fn)(size_t bytes, void* cuda_stream, void* ctx),
