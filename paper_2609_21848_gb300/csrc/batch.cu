@@ -6,6 +6,7 @@
 // captured into a CUDA graph on the first count and replayed afterwards, so a
 // batch count costs one graph launch however many graphs it holds.
 #include <algorithm>
+#include <memory>
 #include <numeric>
 
 #include "radix.cuh"
@@ -322,6 +323,7 @@ struct dbbc_batch {
   cudaGraphExec_t exec = nullptr;
   uint64_t kernels_per_replay = 0;
   std::vector<void*> allocations;
+  std::vector<std::shared_ptr<void>> uploads;  // host arrays that copies on `stream` may still read
 };
 
 namespace dbbc {
@@ -333,7 +335,25 @@ static void* batch_alloc(dbbc_batch* b, size_t bytes) {
   return p;
 }
 
+// Copies `src` to the device in stream order. An asynchronous copy may read its
+// source long after the call, so the plan keeps the array until the stream has
+// been waited for (`uploads` is cleared where that happens, or by batch_release).
+template <typename T>
+static void upload(dbbc_batch* b, T* dst, std::vector<T> src) {
+  if (src.empty()) return;
+  auto kept = std::make_shared<std::vector<T>>(std::move(src));
+  b->uploads.push_back(kept);
+  DBBC_CUDA(cudaMemcpyAsync(dst, kept->data(), kept->size() * sizeof(T), cudaMemcpyHostToDevice, b->stream));
+}
+
+static void wait_for_uploads(dbbc_batch* b) {
+  DBBC_CUDA(cudaStreamSynchronize(b->stream));
+  b->uploads.clear();
+}
+
 static void batch_release(dbbc_batch* b) {
+  if (!b->uploads.empty()) (void)cudaStreamSynchronize(b->stream);  // a call that failed half-way
+  b->uploads.clear();
   if (b->exec) cudaGraphExecDestroy(b->exec);
   b->exec = nullptr;
   for (void* p : b->allocations) dev_free(p, b->stream);
@@ -347,17 +367,18 @@ static void batch_release(dbbc_batch* b) {
   b->fork = b->join = nullptr;
 }
 
-static void finish_plan(dbbc_batch* b, const std::vector<GraphDesc>& desc);
+static void finish_plan(dbbc_batch* b, std::vector<GraphDesc> desc);
 
-// The plan's hub items, from `n_jobs` jobs over n_items items: wide ones, then
-// narrow ones.
-static void plan_items(dbbc_batch* b, const std::vector<HubJob>& jobs, int64_t n_items, const int32_t* comp) {
+// The plan's hub items, from jobs over n_items items: wide ones, then narrow
+// ones.
+static void plan_items(dbbc_batch* b, std::vector<HubJob> jobs, int64_t n_items, const int32_t* comp) {
   if (n_items == 0) return;
+  const int32_t n_jobs = (int32_t)jobs.size();
   cudaStream_t s = b->stream;
   Scratch sc(s);
   const int64_t tiles = radix_tiles(n_items);
   HubJob* d_jobs = sc.get<HubJob>(jobs.size());
-  DBBC_CUDA(cudaMemcpyAsync(d_jobs, jobs.data(), jobs.size() * sizeof(HubJob), cudaMemcpyHostToDevice, s));
+  upload(b, d_jobs, std::move(jobs));
   // zeroed: the split, the sort's digit counts, tile counter and tile states
   const size_t words = (sizeof(HubSplit) + 255) / 256 * 64;
   uint32_t* zero = sc.get<uint32_t>(words + 512 + (size_t)tiles * 256);
@@ -369,7 +390,7 @@ static void plan_items(dbbc_batch* b, const std::vector<HubJob>& jobs, int64_t n
   uint32_t* idx = sc.get<uint32_t>((size_t)n_items * 2);
   b->hub = static_cast<BatchHubItem*>(batch_alloc(b, (size_t)n_items * sizeof(BatchHubItem)));
   const unsigned grid = (unsigned)std::min<int64_t>((n_items + 255) / 256, (int64_t)kNumSMs * 4);
-  plan_items_kernel<<<grid, 256, 0, s>>>(d_jobs, (int32_t)jobs.size(), n_items, comp, tmp, key, idx, st.hist, split);
+  plan_items_kernel<<<grid, 256, 0, s>>>(d_jobs, n_jobs, n_items, comp, tmp, key, idx, st.hist, split);
   DBBC_LAUNCH_CHECK();
   radix_pass<PlainLoad, true, false, false>(PlainLoad{key, idx}, PassOut{nullptr, idx + n_items, nullptr, 0}, n_items,
                                             0, 0, st, &split->flags, s);
@@ -377,7 +398,7 @@ static void plan_items(dbbc_batch* b, const std::vector<HubJob>& jobs, int64_t n
   DBBC_LAUNCH_CHECK();
   HubSplit h;
   DBBC_CUDA(cudaMemcpyAsync(&h, split, sizeof(h), cudaMemcpyDeviceToHost, s));
-  DBBC_CUDA(cudaStreamSynchronize(s));
+  wait_for_uploads(b);
   if (h.flags & kPrepTimeout) throw Error{DBBC_EINTERNAL, "a bounded wait of the plan gave up"};
   b->n_wide = (int64_t)h.wide;
   b->n_narrow = n_items - b->n_wide;
@@ -412,7 +433,7 @@ static void plan_components(dbbc_batch* b, const dbbc_graph* g) {
   b->n_light = g->n_light;
   plan_items(b, {HubJob{g->sweep_items, g->lower, 0, 0}}, g->n_sweep_items, g->component);
   plan_table_logs(b, &g, 1);
-  finish_plan(b, desc);
+  finish_plan(b, std::move(desc));
   if (b->n_medium + b->n_light > 0) {
     const int64_t total = b->n_medium + b->n_light;
     gather_component_pivots_kernel<<<(unsigned)std::min<int64_t>((total + 255) / 256, 4096), 256, 0, s>>>(
@@ -438,22 +459,21 @@ static void plan_batch(dbbc_batch* b, const dbbc_graph* const* gs) {
     hubs[(size_t)i] = HubJob{g->sweep_items, g->lower, n_items, i};
     n_items += g->n_sweep_items;
   }
-  plan_items(b, hubs, n_items, nullptr);
+  plan_items(b, std::move(hubs), n_items, nullptr);
   plan_table_logs(b, gs, n);
-  finish_plan(b, desc);
+  finish_plan(b, std::move(desc));
   GatherJob* d_jobs = static_cast<GatherJob*>(batch_alloc(b, jobs.size() * sizeof(GatherJob)));
-  DBBC_CUDA(cudaMemcpyAsync(d_jobs, jobs.data(), jobs.size() * sizeof(GatherJob), cudaMemcpyHostToDevice, s));
+  upload(b, d_jobs, std::move(jobs));
   if (n > 0) {
     gather_pivots_kernel<<<(unsigned)n, 256, 0, s>>>(d_jobs, b->medium, b->light);
     DBBC_LAUNCH_CHECK();
   }
-  DBBC_CUDA(cudaStreamSynchronize(s));  // host vectors above must outlive the copies
+  wait_for_uploads(b);
 }
 
 // Allocations, launch shapes and uploads shared by all kinds of plan (the hub
 // items are placed already).
-static void finish_plan(dbbc_batch* b, const std::vector<GraphDesc>& desc) {
-  cudaStream_t s = b->stream;
+static void finish_plan(dbbc_batch* b, std::vector<GraphDesc> desc) {
   const int32_t n = b->n_graphs;
   b->desc = static_cast<GraphDesc*>(batch_alloc(b, desc.size() * sizeof(GraphDesc)));
   b->light = static_cast<BatchPivot*>(batch_alloc(b, (size_t)b->n_light * sizeof(BatchPivot)));
@@ -488,7 +508,7 @@ static void finish_plan(dbbc_batch* b, const std::vector<GraphDesc>& desc) {
     DBBC_CUDA(cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming));
     DBBC_CUDA(cudaEventCreateWithFlags(&b->join, cudaEventDisableTiming));
   }
-  DBBC_CUDA(cudaMemcpyAsync(b->desc, desc.data(), desc.size() * sizeof(GraphDesc), cudaMemcpyHostToDevice, s));
+  upload(b, b->desc, std::move(desc));
 }
 
 // The batch count: clear outputs and counters, then the tiers on two
@@ -533,10 +553,11 @@ static void enqueue_batch(dbbc_batch* b, cudaStream_t s) {
   }
 }
 
-static void check_batch_status(const dbbc_batch* b, cudaStream_t s) {
+static void check_batch_status(dbbc_batch* b, cudaStream_t s) {
   unsigned h = 0;
   DBBC_CUDA(cudaMemcpyAsync(&h, b->status, sizeof(h), cudaMemcpyDeviceToHost, s));
   DBBC_CUDA(cudaStreamSynchronize(s));
+  if (s == b->stream) b->uploads.clear();
   raise_device_status(h);
 }
 
@@ -576,21 +597,17 @@ void count_subset(const dbbc_graph* g, cudaStream_t s, const std::vector<int32_t
     for (size_t k = 0; k < hub_items.size(); k++) items[k] = BatchHubItem{0, 0, hub_items[k]};
     b->n_wide = (int64_t)items.size();
     b->hub = static_cast<BatchHubItem*>(batch_alloc(b, items.size() * sizeof(BatchHubItem)));
-    if (!items.empty())
-      DBBC_CUDA(cudaMemcpyAsync(b->hub, items.data(), items.size() * sizeof(BatchHubItem), cudaMemcpyHostToDevice, s));
+    upload(b, b->hub, std::move(items));
     plan_table_logs(b, &g, 1);
-    finish_plan(b, desc);
+    finish_plan(b, std::move(desc));
     std::vector<BatchPivot> med(medium_rows.size()), light(light_rows.size());
     for (size_t k = 0; k < medium_rows.size(); k++) med[k] = BatchPivot{0, medium_rows[k]};
     for (size_t k = 0; k < light_rows.size(); k++) light[k] = BatchPivot{0, light_rows[k]};
-    if (!med.empty())
-      DBBC_CUDA(cudaMemcpyAsync(b->medium, med.data(), med.size() * sizeof(BatchPivot), cudaMemcpyHostToDevice, s));
-    if (!light.empty())
-      DBBC_CUDA(cudaMemcpyAsync(b->light, light.data(), light.size() * sizeof(BatchPivot), cudaMemcpyHostToDevice,
-                                s));
+    upload(b, b->medium, std::move(med));
+    upload(b, b->light, std::move(light));
     enqueue_batch(b, s);
     DBBC_CUDA(cudaMemcpyAsync(h, b->out, sizeof(h), cudaMemcpyDeviceToHost, s));
-    check_batch_status(b, s);  // synchronizes (the host vectors outlive the copies)
+    check_batch_status(b, s);  // synchronizes
   } catch (...) {
     batch_release(b);
     throw;

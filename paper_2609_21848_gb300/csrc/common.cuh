@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <exception>
 #include <new>
 #include <stdexcept>
 #include <vector>
@@ -20,6 +21,17 @@ constexpr int kNumSMs = 152;  // GB300: 2 dies x 76 SMs (used only as a default)
 struct Error {
   dbbc_status status;
   const char* where;
+};
+
+// Declared after host memory that an asynchronous copy on the stream reads:
+// when an exception ends the scope, waits for the stream before that memory is
+// given back.
+struct WaitOnThrow {
+  cudaStream_t s;
+  int uncaught = std::uncaught_exceptions();
+  ~WaitOnThrow() {
+    if (std::uncaught_exceptions() > uncaught) (void)cudaStreamSynchronize(s);
+  }
 };
 
 #define DBBC_CUDA(call)                                           \

@@ -906,6 +906,7 @@ void build_graph_multi(dbbc_graph* g, const int32_t* u, const int32_t* v, const 
   // edge, U and V offsets in one upload
   const size_t k = (size_t)n_graphs + 1;
   std::vector<int64_t> meta(3 * k);
+  const WaitOnThrow wait_for_copy{s};
   std::copy(edge_offsets, edge_offsets + k, meta.begin());
   std::copy(uoff.begin(), uoff.end(), meta.begin() + (ptrdiff_t)k);
   std::copy(voff.begin(), voff.end(), meta.begin() + (ptrdiff_t)(2 * k));
