@@ -291,12 +291,6 @@ __global__ void __launch_bounds__(256) plan_items_kernel(const HubJob* __restric
   dc.finish(hist);
 }
 
-__global__ void gather_hub_items_kernel(const BatchHubItem* __restrict__ src, const uint32_t* __restrict__ idx,
-                                        int64_t n, BatchHubItem* __restrict__ dst) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    dst[i] = src[idx[i]];
-}
-
 }  // namespace dbbc
 
 struct dbbc_batch {
@@ -394,8 +388,7 @@ static void plan_items(dbbc_batch* b, std::vector<HubJob> jobs, int64_t n_items,
   DBBC_LAUNCH_CHECK();
   radix_pass<PlainLoad, true, false, false>(PlainLoad{key, idx}, PassOut{nullptr, idx + n_items, nullptr, 0}, n_items,
                                             0, 0, st, &split->flags, s);
-  gather_hub_items_kernel<<<grid, 256, 0, s>>>(tmp, idx + n_items, n_items, b->hub);
-  DBBC_LAUNCH_CHECK();
+  launch_overlapped(gather_kernel<BatchHubItem>, grid, 256, 0, s, tmp, idx + n_items, n_items, b->hub, &split->flags);
   HubSplit h;
   DBBC_CUDA(cudaMemcpyAsync(&h, split, sizeof(h), cudaMemcpyDeviceToHost, s));
   wait_for_uploads(b);

@@ -736,14 +736,6 @@ __global__ void __launch_bounds__(kRowThreads) plan_hubs_kernel(HubPlanner hp, S
   dc.finish(hist);
 }
 
-__global__ void gather_items_kernel(const SweepItem* __restrict__ src, const uint32_t* __restrict__ idx, int64_t n,
-                                    SweepItem* __restrict__ dst) {
-  let_next_start();
-  wait_for_previous();
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    dst[i] = src[idx[i]];
-}
-
 // ------------------------------------------------------------------ host
 static unsigned grid_for(int64_t n, int threads = 256) {
   int64_t b = ceil_div<int64_t>(n > 0 ? n : 1, threads);
@@ -868,8 +860,8 @@ static void plan_hubs(dbbc_graph* g, cudaStream_t s, const UnionView& un, PrepRe
   if (g->n_sweep_items == 0) return;
   radix_pass<PlainLoad, true, false, false>(PlainLoad{l.key, l.idx}, PassOut{nullptr, l.sorted, nullptr, 0},
                                             g->n_sweep_items, 0, 0, l.sort, &res->flags, s);
-  launch_overlapped(gather_items_kernel,
-                    grid_for(g->n_sweep_items), 256, 0, s, l.items, l.sorted, g->n_sweep_items, g->sweep_items);
+  launch_overlapped(gather_kernel<SweepItem>, grid_for(g->n_sweep_items), 256, 0, s, l.items, l.sorted,
+                    g->n_sweep_items, g->sweep_items, &res->flags);
 }
 
 void build_graph_multi(dbbc_graph* g, const int32_t* u, const int32_t* v, const int8_t* sgn,

@@ -9,7 +9,8 @@
 // start, so every tile that one waits for is running or done. Each wait is
 // bounded all the same: a tile that polls kSpinLimit times sets kPrepTimeout in
 // the pass's flag word and returns, every other wait then ends at once, and
-// the kernels that follow see the flag and return.
+// the kernels that follow (gather_kernel included: its indexes are then partly
+// unwritten) see the flag and return.
 #pragma once
 
 #include <algorithm>
@@ -30,7 +31,13 @@ enum : unsigned {
   kPrepStop = kPrepInvalid | kPrepDup | kPrepTimeout,
 };
 
-constexpr uint32_t kSpinLimit = 1u << 22;  // polls of one wait (seconds; a wait normally takes microseconds)
+// Polls of one wait (seconds; a wait normally takes microseconds). With 0, for
+// tests of what follows a wait that gave up, every tile but a pass's first one
+// gives up before it polls.
+#ifndef DBBC_SPIN_LIMIT
+#define DBBC_SPIN_LIMIT (1u << 22)
+#endif
+constexpr uint32_t kSpinLimit = DBBC_SPIN_LIMIT;
 
 __device__ __forceinline__ uint32_t ld_relaxed(const uint32_t* p) {
   uint32_t v;
@@ -57,6 +64,13 @@ __device__ __forceinline__ bool wait_over(uint32_t polls, unsigned* flags) {
     return true;
   }
   return (polls & 63u) == 63u && (ld_relaxed(flags) & kPrepTimeout) != 0;
+}
+
+// Whether a tile may wait for the ones before it (always, but for kSpinLimit 0).
+__device__ __forceinline__ bool may_wait(int64_t tile, unsigned* flags) {
+  if (kSpinLimit > 0 || tile == 0) return true;
+  atomicOr(flags, (unsigned)kPrepTimeout);
+  return false;
 }
 
 // ------------------------------------------------------------------ scans
@@ -128,10 +142,10 @@ __device__ __forceinline__ bool tile_prefix(uint64_t* state, int64_t tile, uint6
     const unsigned lane = lane_id();
     if (lane == 0) st_relaxed(&state[tile], (tile == 0 ? kTileTotal : kTileSum) | sum);
     uint64_t pre = 0;
-    bool ok = true;
+    bool ok = may_wait(tile, flags);
     int64_t end = tile;  // the tiles [end, tile) are in `pre`
     uint32_t polls = 0;
-    while (end > 0) {
+    while (ok && end > 0) {
       const int64_t t = end - 1 - (int64_t)lane;
       const uint64_t s = t >= 0 ? ld_relaxed(&state[t]) : kTileTotal;
       // lanes up to the first running total count, if all before it are there
@@ -358,8 +372,8 @@ __global__ void __launch_bounds__(kRsThreads, DBBC_RS_CTAS)
     const int d = threadIdx.x;
     const uint32_t count = gofs[d];
     uint32_t before = 0, polls = 0;
-    bool ok = true;
-    for (int64_t t = tile - 1; t >= 0;) {
+    bool ok = may_wait(tile, flags);
+    for (int64_t t = tile - 1; ok && t >= 0;) {
       uint32_t s[4];
 #pragma unroll
       for (int k = 0; k < 4; k++) s[k] = t - k >= 0 ? ld_relaxed(&state[(t - k) * 256 + d]) : kDigitTotal;
@@ -425,6 +439,17 @@ void radix_pass(const Load& load, const PassOut& out, int64_t n, int begin_bit, 
   const int64_t tiles = radix_tiles(n);
   launch_overlapped(fn, tiles, kRsThreads, smem, s, load, out, n, begin_bit + 8 * pass, st.hist + 256 * pass,
                     st.state + (size_t)pass * tiles * 256, st.counters + pass, flags);
+}
+
+// dst[i] = src[idx[i]]: a list in the order that a sort found.
+template <typename T>
+__global__ void gather_kernel(const T* __restrict__ src, const uint32_t* __restrict__ idx, int64_t n,
+                              T* __restrict__ dst, const unsigned* flags) {
+  if (cta_stopped(flags)) return;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t j = idx[i];
+    if (DBBC_CHECK((int64_t)j < n)) dst[i] = src[j];
+  }
 }
 
 }  // namespace dbbc
