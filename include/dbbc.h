@@ -261,7 +261,7 @@ DBBC_API dbbc_status dbbc_graph_export(const dbbc_graph* g, void* cuda_stream, i
                               uint32_t* lower, int32_t* vertex, uint64_t* work);
 
 /* Device allocator hook (e.g. a framework's caching allocator). alloc returns
- * NULL on failure. Passing NULL for both restores the default: stream-ordered
+ * memory aligned to at least 8 bytes, or NULL on failure. Passing NULL for both restores the default: stream-ordered
  * allocations (cudaMallocFromPoolAsync) from one memory pool per device owned
  * by the library, which keeps up to 32 GiB of freed memory mapped between
  * calls instead of returning it to the device at every synchronization.

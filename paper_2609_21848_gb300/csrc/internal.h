@@ -141,8 +141,11 @@ constexpr int16_t kItemFirst = 8;
 constexpr int32_t kTinyCountLimit = 256;
 constexpr int32_t kQuarterCountLimit = 16;
 
-// Bytes allocated past the CSR's last entry: the hub sweep reads rows in
-// aligned chunks of up to 128 entries, the last of which may pass the end.
+// The hub sweep reads rows in chunks of up to 128 entries, 16 aligned bytes per
+// lane: the CSR's entries start at a multiple of kColAlign, whatever alignment
+// an installed allocator has, and have kColPad bytes allocated past the last
+// one, which the last chunk may pass.
+constexpr size_t kColAlign = 16;
 constexpr size_t kColPad = 512;
 
 // Read-only view of the device CSR passed to kernels by value.

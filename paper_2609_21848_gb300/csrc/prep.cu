@@ -1036,9 +1036,11 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
   // up, the kernels that follow return at once and the flags say why. *ku_out
   // gets the U-sorted keys.
   const uint64_t* ku = nullptr;
+  void* col_block = nullptr;  // the allocation that holds g->col
   auto build_from_edges = [&](const int32_t* eu, const int32_t* ev, const int8_t* es, int64_t me) -> PrepResult {
     DBBC_CUDA(cudaMemsetAsync(l.res, 0, l.zeroed, s));
-    g->col = static_cast<uint32_t*>(graph_alloc(g, (size_t)(2 * me) * 4, kColPad));
+    col_block = graph_alloc(g, (size_t)(2 * me) * 4, kColPad + kColAlign);
+    g->col = reinterpret_cast<uint32_t*>(((uintptr_t)col_block + kColAlign - 1) / kColAlign * kColAlign);
     if (me > 0)
       launch_overlapped(degree_kernel, grid_for(me), 256, 0, s, eu, ev, es, me, n_u, n_v, l.deg, d_flags);
     if (n > 0) {
@@ -1121,7 +1123,7 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
     const PrepResult d = read_back(l.res, s);
     if (d.flags & kPrepTimeout) throw Error{DBBC_EINTERNAL, "a bounded wait of the build gave up"};
     mu = (int64_t)d.kept;
-    graph_release(g, g->col, (size_t)(2 * m) * 4);
+    graph_release(g, col_block, (size_t)(2 * m) * 4);
     g->col = nullptr;
     r = build_from_edges(eu, ev, es, mu);
     if (r.flags & kPrepDup) throw Error{DBBC_EINTERNAL, "duplicates left after deduplication"};
