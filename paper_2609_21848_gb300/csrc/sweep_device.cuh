@@ -222,6 +222,10 @@ __device__ __forceinline__ void lean_load(const uint32_t* __restrict__ col, uint
   x[3] = v.w;
 }
 
+// Whether the n entries from position c on (c <= en) lie in a row that ends at
+// en. Positions reach 2^32 - 2, so c + n may not fit 32 bits.
+__host__ __device__ __forceinline__ bool chunk_in_row(uint32_t c, uint32_t en, uint32_t n) { return en - c >= n; }
+
 // Entries of the lane's four positions from pos on that lie past the row's end
 // become ~0.
 __device__ __forceinline__ void lean_mask_end(uint32_t pos, uint32_t en, uint32_t (&x)[kLU]) {
@@ -279,7 +283,7 @@ __device__ __forceinline__ bool lean_walk(const uint32_t* __restrict__ col, uint
       end += (uint32_t)(G * kLU);
     }
     for (;;) {
-      const bool full = last_entry() < h && end <= en && more;
+      const bool full = last_entry() < h && more && chunk_in_row(c, en, (uint32_t)(G * kLU));
       if (!__any_sync(kFullMask, full)) break;
       if (full) {
         uint32_t y[kLU];
