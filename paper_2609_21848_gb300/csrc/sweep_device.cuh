@@ -222,9 +222,10 @@ __device__ __forceinline__ void lean_load(const uint32_t* __restrict__ col, uint
   x[3] = v.w;
 }
 
-// Whether the n entries from position c on (c <= en) lie in a row that ends at
-// en. Positions reach 2^32 - 2, so c + n may not fit 32 bits.
-__host__ __device__ __forceinline__ bool chunk_in_row(uint32_t c, uint32_t en, uint32_t n) { return en - c >= n; }
+// The last position at which n entries of a row that ends at en (at least n) can
+// start. A chunk is compared with it and not by its own end, since positions
+// reach 2^32 - 2 and the end of a chunk past the row may not fit 32 bits.
+__host__ __device__ __forceinline__ uint32_t last_chunk(uint32_t en, uint32_t n) { return en - n; }
 
 // Entries of the lane's four positions from pos on that lie past the row's end
 // become ~0.
@@ -275,29 +276,28 @@ __device__ __forceinline__ bool lean_walk(const uint32_t* __restrict__ col, uint
   for (int u = 0; u < kLU; u++) lean_add<CW, RET, true>(x[u], h, s1, w, a_lo, a_hi, bal, unb);
   const bool more = last_entry() < h;  // the first chunk lies wholly inside: the segment goes on
   if (__any_sync(kFullMask, more)) {
+    constexpr uint32_t kChunk = G * kLU;
     const uint32_t* p = col + 4u * (uint32_t)gl;
-    uint32_t end = (c & ~3u) + (uint32_t)(G * kLU);  // the end of the chunk in x
+    const uint32_t hl = more ? h : 0u;
+    const uint32_t last = last_chunk(en, kChunk);  // (where `more`: the row is that long)
     if (more) {
-      lean_load(p, end, x);
-      c = end;
-      end += (uint32_t)(G * kLU);
+      c = (c & ~3u) + kChunk;  // the chunk in x from here on starts at c
+      lean_load(p, c, x);
     }
     for (;;) {
-      const bool full = last_entry() < h && more && chunk_in_row(c, en, (uint32_t)(G * kLU));
+      const bool full = last_entry() < hl && c <= last;
       if (!__any_sync(kFullMask, full)) break;
       if (full) {
         uint32_t y[kLU];
-        lean_load(p, end, y);  // the next chunk, while this one is counted
+        lean_load(p + kChunk, c, y);  // the next chunk, while this one is counted
 #pragma unroll
         for (int u = 0; u < kLU; u++) lean_add<CW, RET, false>(x[u], 0u, s1, w, a_lo, a_hi, bal, unb);
-        c = end;
-        end += (uint32_t)(G * kLU);
+        c += kChunk;
 #pragma unroll
         for (int u = 0; u < kLU; u++) x[u] = y[u];
       }
     }
     if (more) lean_mask_end(c + 4u * (uint32_t)gl, en, x);
-    const uint32_t hl = more ? h : 0u;
 #pragma unroll
     for (int u = 0; u < kLU; u++) lean_add<CW, RET, true>(x[u], hl, s1, w, a_lo, a_hi, bal, unb);
   }

@@ -1,5 +1,6 @@
 // Host check of the hub sweep's test that a chunk lies inside its row, at the
-// last positions that 32 bits hold, against 64-bit sums.
+// last positions that 32 bits hold, against 64-bit sums. Chunks that the walk
+// reaches start at or before the end of a row of at least a chunk.
 #include <cstdio>
 
 #include "../paper_2609_21848_gb300/csrc/sweep_device.cuh"
@@ -9,9 +10,9 @@ int main() {
   int wrong = 0;
   for (uint32_t en : ends)
     for (uint32_t back = 0; back <= 300 && back <= en; back++)
-      for (uint32_t n = 4; n <= 128; n *= 2) {
+      for (uint32_t n = 4; n <= 128 && n <= en; n *= 2) {
         const uint32_t c = en - back;
-        wrong += dbbc::chunk_in_row(c, en, n) != ((uint64_t)c + n <= (uint64_t)en);
+        wrong += (c <= dbbc::last_chunk(en, n)) != ((uint64_t)c + n <= (uint64_t)en);
       }
   std::printf("%d wrong\n", wrong);
   return wrong ? 1 : 0;
