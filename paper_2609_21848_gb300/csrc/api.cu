@@ -342,12 +342,13 @@ size_t dbbc_graph_device_bytes(const dbbc_graph* g) { return g ? g->device_bytes
 size_t dbbc_estimate_bytes(int64_t m, int32_t n_u, int32_t n_v) {
   if (m < 0 || n_u < 0 || n_v < 0) return 0;
   const size_t n = (size_t)n_u + (size_t)n_v, mm = (size_t)m;
-  // handle: row_ptr 8(n+1), col 8m, lower/vertex 8n, work 8n, order 4n, items (the row spans' 8n are covered by
-  // the build's margin)
-  const size_t handle = 8 * (n + 1) + 8 * mm + 8 * n + 8 * n + 4 * n + 16 * (mm / 64 + 16);
+  // handle: row_ptr 8(n+1), col 8m, lower/vertex 8n, spans 8n, work 8n, order 4n, items
+  const size_t handle = 8 * (n + 1) + 8 * mm + 8 * n + 8 * n + 8 * n + 4 * n + 16 * (mm / 64 + 16);
   // build peak, with a wide margin: inputs 9m, edge keys and their U positions 24m, sort states 2m, distinct
-  // edges 9m, vertex keys and ranks 36n
-  const size_t build = 9 * mm + 32 * mm + 9 * mm + 32 * mm + 8 * mm + 48 * n + (mm / 4096 + 1) * 1024;
+  // edges 9m, vertex keys and ranks 36n and their sort states 3n; whatever the size, a kilobyte of digit counts
+  // and one of tile states per digit pass of four sorts (at most 64), and about 40 arrays' round-up to 256 bytes
+  const size_t build =
+      9 * mm + 32 * mm + 9 * mm + 32 * mm + 8 * mm + 48 * n + (mm / 4096 + 1) * 1024 + (size_t{96} << 10);
   return handle + build;
 }
 

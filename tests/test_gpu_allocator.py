@@ -1,5 +1,7 @@
-"""An installed allocator whose memory is aligned to 8 bytes and no more: every
-entry point that allocates must count as with the library's own pool."""
+"""Calls on an installed allocator: one whose memory is aligned to 8 bytes and no
+more, on which every entry point that allocates must count as with the library's
+own pool, and one that adds up what a build holds at once, which may not pass
+the upper estimate that admission control goes by."""
 import ctypes
 
 import numpy as np
@@ -60,3 +62,41 @@ def test_counts_on_memory_aligned_to_eight_bytes(eight_byte_allocator, repeats):
         dbbc.dbbc_set_tuning(base)
     assert [int(x.sum(dtype=np.uint64)) for x in (vb, vu, eb, eu)] == [4 * want[0], 4 * want[1]] * 2
     assert [x.tolist() for x in plan] == [x.tolist() for x in parts] == [[want[0]] * 2, [want[1]] * 2]
+
+
+@pytest.mark.parametrize("hubs", [False, True])  # True: every pivot that can close a butterfly is a hub
+@pytest.mark.parametrize("n_u,n_v,m,repeats", [(3, 4, 5, 0), (3, 4, 9, 3), (60, 40, 700, 0), (1_000, 900, 20, 0),
+                                               (2_000_000, 1_000_003, 10, 0), (40_000, 9_000, 600_000, 30_000),
+                                               (3_000, 2_000, 400_000, 0)])
+def test_builds_stay_within_the_estimate(n_u, n_v, m, repeats, hubs):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    torch.cuda.set_device(0)
+    rng = np.random.default_rng(m)
+    k = np.unique(rng.integers(0, n_u * n_v, 2 * m)) if n_u * n_v > 100 * m else np.arange(n_u * n_v)
+    k = rng.permutation(k)[:m - repeats]
+    k = np.concatenate([k, k[:repeats]])
+    u, v = (k // n_v).astype(np.int32), (k % n_v).astype(np.int32)
+    s = np.where(rng.random(m) < 0.5, 1, -1).astype(np.int8)
+    live, peak = {}, [0]
+
+    def alloc(size, stream, ctx):
+        block = torch.empty(size, dtype=torch.uint8, device="cuda")
+        live[block.data_ptr()] = block
+        peak[0] = max(peak[0], sum(b.numel() for b in live.values()))
+        return block.data_ptr()
+
+    refs = (dbbc._ALLOC_FN(alloc), dbbc._FREE_FN(lambda p, stream, ctx: live.pop(int(p))))
+    base = dbbc.dbbc_get_tuning()
+    dbbc.lib().dbbc_set_allocator(ctypes.cast(refs[0], ctypes.c_void_p), ctypes.cast(refs[1], ctypes.c_void_p), None)
+    try:
+        if hubs:
+            dbbc.dbbc_set_tuning({"light_max_work": 1, "medium_max_work": 1})
+        with dbbc.dbbc_graph_from_coo(u, v, s, n_u, n_v):
+            pass
+        torch.cuda.synchronize()
+    finally:
+        dbbc.lib().dbbc_set_allocator(None, None, None)
+        dbbc.dbbc_set_tuning(base)
+    assert 0 < peak[0] <= dbbc.dbbc_estimate_bytes(m, n_u, n_v), peak
