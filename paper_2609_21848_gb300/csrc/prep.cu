@@ -268,7 +268,8 @@ __global__ void __launch_bounds__(256) csr_v_digits_kernel(const uint64_t* __res
 // run (the sorts are stable, so the latest input occurrence), compacted in one
 // pass over tiles of kRowTile edges. *count gets their number.
 __global__ void __launch_bounds__(kRowThreads) dedup_kernel(const uint64_t* __restrict__ ku, int64_t m, int bits_v,
-                                                            int32_t n_u, const int32_t* __restrict__ vertex,
+                                                            int32_t n_u, int64_t n,
+                                                            const int32_t* __restrict__ vertex,
                                                             int32_t* __restrict__ eu, int32_t* __restrict__ ev,
                                                             int8_t* __restrict__ es, uint64_t* count, uint64_t* state,
                                                             unsigned* counter, unsigned* flags) {
@@ -295,9 +296,11 @@ __global__ void __launch_bounds__(kRowThreads) dedup_kernel(const uint64_t* __re
   for (int j = 0; j < kRowItems; j++) {
     if (keep[j]) {
       const uint64_t ru = k[j] >> (bits_v + 1), rv = (k[j] >> 1) & ((1ull << bits_v) - 1);
-      eu[at] = vertex[ru];
-      ev[at] = vertex[n_u + rv] - n_u;
-      es[at] = (k[j] & 1u) ? (int8_t)-1 : (int8_t)1;
+      if (DBBC_CHECK(at < (uint64_t)m && ru < (uint64_t)n_u && (int64_t)(n_u + rv) < n)) {
+        eu[at] = vertex[ru];
+        ev[at] = vertex[n_u + rv] - n_u;
+        es[at] = (k[j] & 1u) ? (int8_t)-1 : (int8_t)1;
+      }
       at++;
     }
     if (i0 + j == m - 1) *count = at;
@@ -526,8 +529,10 @@ __global__ void __launch_bounds__(kRowThreads) pivots_kernel(const uint64_t* __r
 #pragma unroll
   for (int j = 0; j < kPivotItems; j++) {
     if (mine >> j & 1u) {
-      key[at] = ~w[j];
-      row[at] = (uint32_t)(r0 + j);
+      if (DBBC_CHECK(at < (uint64_t)n)) {
+        key[at] = ~w[j];
+        row[at] = (uint32_t)(r0 + j);
+      }
       dc.add(~w[j]);
       at++;
     }
@@ -717,7 +722,10 @@ __global__ void __launch_bounds__(kRowThreads) plan_hubs_kernel(HubPlanner hp, S
     it.hi = (uint32_t)(w1 == p.windows ? p.sp : window_start(p, w1));
     if (w0 == 0) it.flags |= kItemFirst;
     const uint64_t at = prefix + ex + k;
-    if (at >= cap) break;  // cannot happen: cap bounds the number of items
+    if (at >= cap) {  // cannot happen: cap bounds the number of items
+      (void)DBBC_CHECK(false);
+      break;
+    }
     items[at] = it;
     idx[at] = (uint32_t)at;
     const uint64_t d = estimate_digit(it.est, 3, 256u);
@@ -1118,8 +1126,8 @@ void build_graph(dbbc_graph* g, const int32_t* u_in, const int32_t* v_in, const 
     int8_t* es = sc.get<int8_t>((size_t)m);
     DBBC_CUDA(cudaMemsetAsync(d_flags, 0, sizeof(unsigned), s));
     launch_overlapped(dedup_kernel,
-                      (unsigned)ceil_div<int64_t>(m, kRowTile), kRowThreads, 0, s, ku, m, bits_v, n_u, g->vertex, eu,
-                      ev, es, reinterpret_cast<uint64_t*>(&l.res->kept), l.dedup_state, l.counters + 2, d_flags);
+                      (unsigned)ceil_div<int64_t>(m, kRowTile), kRowThreads, 0, s, ku, m, bits_v, n_u, n, g->vertex,
+                      eu, ev, es, reinterpret_cast<uint64_t*>(&l.res->kept), l.dedup_state, l.counters + 2, d_flags);
     const PrepResult d = read_back(l.res, s);
     if (d.flags & kPrepTimeout) throw Error{DBBC_EINTERNAL, "a bounded wait of the build gave up"};
     mu = (int64_t)d.kept;

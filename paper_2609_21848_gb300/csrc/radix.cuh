@@ -414,6 +414,8 @@ __global__ void __launch_bounds__(kRsThreads, DBBC_RS_CTAS)
         if (WRITE_K) out.key[g] = k;
         if (HAS_V) out.val[g] = sv[i];
         if (AUX) out.aux[g] = (uint32_t)(k & out.aux_mask);
+      } else {
+        (void)DBBC_CHECK(false);  // checked builds: recorded
       }
     }
   }
