@@ -2,7 +2,9 @@
 // LSD radix sort with one kernel per digit. Written for sm_103a; no CUB.
 //
 // Both chain their tiles by decoupled look-back (Merrill and Garland,
-// "Single-pass Parallel Prefix Scan with Decoupled Look-back", 2016): a tile
+// "Single-pass Parallel Prefix Scan with Decoupled Look-back", 2016; one kernel
+// per radix digit that way: Adinets and Merrill, "Onesweep: A Faster Least
+// Significant Digit Radix Sort for GPUs", 2022): a tile
 // publishes its own sum, adds up what the tiles before it have published until
 // it meets one whose running total is known, and publishes its own running
 // total. Tiles are numbered by a counter in the order in which their CTAs

@@ -40,7 +40,7 @@ constexpr int kLU = 4;
 
 // Shared counters of the sweep: one window, plus one word so that a window of
 // 4-bit (8-bit) counters may start at the multiple of 4 (even rank) below its
-// first rank.
+// first rank, rounded up to the 16 bytes that windows are cleared by.
 constexpr uint32_t kSweepWords = kSweepWindow16 + 4;
 constexpr size_t kSweepSmem = (size_t)kSweepWords * 4;
 
@@ -254,9 +254,11 @@ __device__ __forceinline__ void lean_load_first(const uint32_t* __restrict__ col
 // A group of G lanes walks one neighbour's entries inside window w from
 // cursor c (row end en, first chunk already in x). One lane of the group gets
 // true back, and in c_next the cursor past the window and in x_next the
-// neighbour's entry there (~0 at the end of its row). The first and the last chunk of a segment are counted
-// entry by entry against the window's end; the chunks between them lie wholly
-// inside the window and the row, and their entries need no test. All groups of
+// neighbour's entry there (~0 at the end of its row). The first and the last
+// chunk of a segment are counted entry by entry against the window's end; the
+// chunks between them lie wholly inside the window and the row (their last entry
+// does, and they start no later than the row's last whole chunk), and their
+// entries need no test. All groups of
 // the warp run the loop in lockstep until the last of them has met its last
 // chunk: the loop's only exit follows a warp-wide vote, so every shuffle and
 // vote in it is reached by the whole warp. A group that is not `active` (no
